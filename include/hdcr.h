@@ -157,6 +157,17 @@ int hdcr_tc_gemm_info(unsigned long long* calls, unsigned long long* fallbacks);
  */
 int hdcr_apply_g5dwf(const hdcr_geom* g, const hdcr_dwf_params* p, const void* U,
                      const void* in, void* out, int dtype, int nrhs, void* stream);
+/* The same with device scratch from the caller.  An FP64 application (HDCR_C128)
+ * encodes its operands as fixed-point integers in device memory first, in
+ * hdcr_apply_scratch_bytes bytes for all nrhs fields; with less, a multiple of fields at a time
+ * that fits (at least hdcr_apply_scratch_bytes for one field), and with less than that
+ * on the FP64 pipe from the operands themselves, several times slower.  hdcr_apply_g5dwf
+ * allocates the scratch on ``stream`` from the device's memory pool.  ``scratch`` is 16-byte
+ * aligned and used on ``stream`` only until the call's work there is done; it may be null.
+ * hdcr_apply_scratch_bytes is 0 for other dtypes and for a geometry that is not admissible. */
+size_t hdcr_apply_scratch_bytes(const hdcr_geom* g, int dtype, int nrhs);
+int hdcr_apply_g5dwf_scratch(const hdcr_geom* g, const hdcr_dwf_params* p, const void* U, const void* in, void* out,
+                             int dtype, int nrhs, void* scratch, size_t scratch_bytes, void* stream);
 
 /* Tile-shape autotuner of the FP32 operator (a property of this library, not a
  * step of the method).  The FP32 kernel runs one CTA per tile of 4d sites;

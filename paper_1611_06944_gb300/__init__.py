@@ -198,9 +198,38 @@ def apply_g5dwf(lat: Lattice, U: torch.Tensor, psi: torch.Tensor, M5: float, mf:
     out = torch.empty_like(psi) if out is None else out
     g = lat.c_geom()
     p = _params(M5, mf)
-    _check(_L.hdcr_apply_g5dwf(C_ref(g), C_ref(p), _dev(U, "U"), _dev(psi, "psi"), _dev(out, "out"),
-                               _code(psi), n, _stream(stream)), "apply_g5dwf")
+    args = (C_ref(g), C_ref(p), _dev(U, "U"), _dev(psi, "psi"), _dev(out, "out"), _code(psi), n)
+    scratch = _apply_scratch(g, psi, n, stream)
+    if scratch is None:
+        _check(_L.hdcr_apply_g5dwf(*args, _stream(stream)), "apply_g5dwf")
+    else:
+        _check(_L.hdcr_apply_g5dwf_scratch(*args, scratch.data_ptr(), scratch.numel(), _stream(stream)),
+               "apply_g5dwf")
     return out
+
+
+_SCRATCH_MAX = 1 << 30  # most scratch bytes an application over many fields asks torch for
+
+
+def _apply_scratch(g, psi, n, stream):
+    """Scratch of an FP64 application from torch's allocator, allocated on the stream that
+    uses it; None where the library allocates what it can itself: under stream capture, and
+    when torch is out of memory."""
+    if psi.dtype != torch.complex128:
+        return None
+    one = _L.hdcr_apply_scratch_bytes(C_ref(g), _lib.HDCR_C128, 1)
+    size = max(one, min(_L.hdcr_apply_scratch_bytes(C_ref(g), _lib.HDCR_C128, n), _SCRATCH_MAX))
+    if torch.cuda.is_current_stream_capturing():
+        return None
+    try:
+        if stream is None:
+            return torch.empty(size, dtype=torch.uint8, device=psi.device)
+        with torch.cuda.stream(stream):
+            if torch.cuda.is_current_stream_capturing():
+                return None
+            return torch.empty(size, dtype=torch.uint8, device=psi.device)
+    except torch.OutOfMemoryError:
+        return None
 
 
 def _cf_params(beta, R: float) -> _lib.hdcr_cf_params:

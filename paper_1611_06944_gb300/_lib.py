@@ -103,6 +103,8 @@ SIGNATURES = {
     "hdcr_probe_fma_rate": (_I, [_I, C.POINTER(C.c_double), _P]),
     "hdcr_tc_gemm_info": (_I, [C.POINTER(C.c_ulonglong), C.POINTER(C.c_ulonglong)]),
     "hdcr_apply_g5dwf": (_I, [_G, _DP, _P, _P, _P, _I, _I, _P]),
+    "hdcr_apply_scratch_bytes": (_SZ, [_G, _I, _I]),
+    "hdcr_apply_g5dwf_scratch": (_I, [_G, _DP, _P, _P, _P, _I, _I, _P, _SZ, _P]),
     "hdcr_stencil_tune": (_I, [_I, _I]),
     "hdcr_mobius_to_shamir": (_I, [_DP, _D, _P, _P, _I, _SZ, _DP, _P]),
     "hdcr_fermion_encode_h16": (_I, [_G, _P, _I, _P, _I, _P]),

@@ -114,6 +114,11 @@ int cheb_smoother(const FineOp<R>& H, const cpx<R>* r, cpx<R>* out, const std::v
   const long long n = H.n();
   const int nb = num_blocks(n, 256, 4096);
   const int order = (int)c.size() - 1;
+  if constexpr (sizeof(R) == 8)
+    if (H.fixed() && order >= 1) {
+      HDCR_TRY(launch_fx_encode(H.g, r, H.nrhs, H.fx->e0, nullptr, H.fx->u, st));
+      return cheb_smoother_fx(H, H.fx->e0, H.fx->e1, out, c, lo, hi, w, st, matvecs);
+    }
   const R a = (R)(2.0 / (hi - lo)), b = (R)(-(hi + lo) / (hi - lo));
   // v = H r (held in t0 = T_0 v)
   HDCR_TRY(H.apply(r, w.t0, st));
@@ -167,6 +172,45 @@ int cheb_smoother(const FineOp<R>& H, const cpx<R>* r, cpx<R>* out, const std::v
     cur = t;
   }
   *matvecs += mv;
+  return HDCR_OK;
+}
+
+int cheb_smoother_fx(const FineOp<double>& H, const FxField& a, const FxField& b, cpx<double>* out,
+                     const std::vector<double>& c, double lo, double hi, ChebWork<double>& w, cudaStream_t st,
+                     int* matvecs) {
+  const int order = (int)c.size() - 1;
+  const Geom& g = H.g;
+  const FxLinks& u = H.fx->u;
+  const long long sites = g.V5 * H.nrhs;
+  auto timed = [&](int kind, auto launch) {
+    int slot;
+    stencil_timer_begin(kind, sites, st, &slot);
+    const int s = launch();
+    stencil_timer_end(slot, st);
+    ++*matvecs;
+    return s;
+  };
+  FxChebStep step{};
+  step.a = 2.0 / (hi - lo);
+  step.b = -(hi + lo) / (hi - lo);
+  // T_0 = v = H r, kept and encoded; then T_k from H (H T_{k-1}), the inner one only encoded
+  HDCR_TRY(timed(0, [&] { return launch_fx_g5dwf(g, H.M5, H.mf, u, a, w.t0, H.nrhs, st, &b); }));
+  cpx<double>* prev = w.t0;
+  cpx<double>* cur = w.t0;
+  for (int k = 1; k <= order; ++k) {
+    HDCR_TRY(timed(0, [&] { return launch_fx_g5dwf(g, H.M5, H.mf, u, b, nullptr, H.nrhs, st, &a); }));
+    step.first = k == 1;
+    step.last = k == order && k > 1;
+    step.cur = cur;
+    step.prev = k == 1 ? w.t1 : prev;
+    step.acc = out;
+    step.ck = c[k];
+    step.c0 = 0.5 * c[0];
+    HDCR_TRY(timed(3, [&] { return launch_fx_g5dwf_cheb(g, H.M5, H.mf, u, a, step, b, H.nrhs, st); }));
+    prev = cur;
+    cur = step.prev;
+  }
+  if (order == 1) HDCR_TRY(launch_fx_encode(g, out, H.nrhs, b, nullptr, u, st));
   return HDCR_OK;
 }
 

@@ -29,6 +29,13 @@ template <typename R>
 int cheb_smoother(const FineOp<R>& H, const cpx<R>* r, cpx<R>* out, const std::vector<double>& c, double lo,
                   double hi, ChebWork<R>& w, cudaStream_t st, int* matvecs);
 
+// The same in FP64 through the encoded fields of H.fx (H.fixed() must hold, order >= 1): r is
+// given encoded in ``a``, and out is left encoded in ``b`` as well (a and b the two fields of
+// H.fx).  Terms pass between the applications encoded.
+int cheb_smoother_fx(const FineOp<double>& H, const FxField& a, const FxField& b, cpx<double>* out,
+                     const std::vector<double>& c, double lo, double hi, ChebWork<double>& w, cudaStream_t st,
+                     int* matvecs);
+
 // x <- T_order(t(H^2)) x / |.|, t mapping [lam_cut^2, lam_max^2] onto [-1, 1]
 template <typename R>
 int cheb_filter(const FineOp<R>& H, cpx<R>* x, int order, double lam_cut, double lam_max, ChebWork<R>& w,

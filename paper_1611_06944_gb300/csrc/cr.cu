@@ -293,6 +293,9 @@ static int cr_solve_impl(const Geom& g, const hdcr_dwf_params* p, const void* U,
   FineOp<R> H{g, p->M5, p->mf, (const cpx<R>*)U};
   CRWork<R> w;
   HDCR_TRY(crwork_alloc<R>(&w, H.n()));
+  FxCtx fx;
+  if (sizeof(R) == 8) fx_ctx_alloc(&fx, g, 1);
+  H.fx = &fx;
   CRConfig cfg;
   cfg.tol = tol;
   cfg.max_iter = max_iter;
@@ -300,7 +303,8 @@ static int cr_solve_impl(const Geom& g, const hdcr_dwf_params* p, const void* U,
   CRGraph graph;  // the iterations between host checks replay from one CUDA graph
   cfg.graph = &graph;
   CRResult res;
-  int s = cr_run<R>(H, (const cpx<R>*)b, (cpx<R>*)x, w, cfg, &res, st);
+  int s = fx_ctx_links(fx, g, (const cpx<double>*)U, st);
+  if (s == HDCR_OK) s = cr_run<R>(H, (const cpx<R>*)b, (cpx<R>*)x, w, cfg, &res, st);
   cr_graph_free(&graph);
   double tr = -1.0;
   if (s == HDCR_OK) {
@@ -317,6 +321,7 @@ static int cr_solve_impl(const Geom& g, const hdcr_dwf_params* p, const void* U,
   }
   cudaStreamSynchronize(st);
   crwork_free<R>(&w);
+  fx_ctx_free(&fx);
   if (s == HDCR_OK && !res.converged) {
     set_error("CR: not converged after %d iterations (|r|/|b| = %g)", res.iters, res.rel_resid);
     s = HDCR_ERR_NOT_CONVERGED;

@@ -15,6 +15,7 @@
 
 #include "host_io.cuh"
 #include "blas.cuh"
+#include "dwf_fx.cuh"
 #include "dwf_stencil.cuh"
 
 namespace hdcr {
@@ -255,6 +256,37 @@ int launch_convert(const void* in, int idt, void* out, int odt, long long n, cud
 // ===================================================================== C ABI
 using namespace hdcr;
 
+// an FP64 application on the integer pipe with scratch that holds at least one field, else in FP64
+static int apply_c128(const Geom& g, const hdcr_dwf_params* p, const void* U, const void* in, void* out, int nrhs,
+                      void* scratch, size_t bytes, cudaStream_t st) {
+  if (!fx_apply_fits(g, scratch, bytes)) return launch_g5dwf<double>(g, p->M5, p->mf, U, in, out, nrhs, st);
+  int slot;
+  stencil_timer_begin(0, g.V5 * nrhs, st, &slot);
+  const int s = launch_fx_apply(g, p->M5, p->mf, (const cpx<double>*)U, (const cpx<double>*)in, (cpx<double>*)out, nrhs,
+                                scratch, bytes, st);
+  stencil_timer_end(slot, st);
+  return s;
+}
+
+extern "C" size_t hdcr_apply_scratch_bytes(const hdcr_geom* gp, int dtype, int nrhs) {
+  Geom g;
+  if (make_geom(gp, &g) != HDCR_OK || dtype != HDCR_C128 || nrhs < 1 || !fx_ok(g)) return 0;
+  return fx_scratch_bytes(g, nrhs);
+}
+
+extern "C" int hdcr_apply_g5dwf_scratch(const hdcr_geom* gp, const hdcr_dwf_params* p, const void* U, const void* in,
+                                        void* out, int dtype, int nrhs, void* scratch, size_t scratch_bytes,
+                                        void* stream) {
+  if (dtype != HDCR_C128) return hdcr_apply_g5dwf(gp, p, U, in, out, dtype, nrhs, stream);
+  Geom g;
+  HDCR_TRY(make_geom(gp, &g));
+  if (!p || !U || !in || !out || nrhs < 1 || in == out) {
+    set_error("hdcr_apply_g5dwf_scratch: null pointer, nrhs < 1 or in and out overlapping");
+    return HDCR_ERR_BAD_ARG;
+  }
+  return apply_c128(g, p, U, in, out, nrhs, scratch, scratch_bytes, as_stream(stream));
+}
+
 extern "C" int hdcr_apply_g5dwf(const hdcr_geom* gp, const hdcr_dwf_params* p, const void* U,
                                 const void* in, void* out, int dtype, int nrhs, void* stream) {
   Geom g;
@@ -278,7 +310,19 @@ extern "C" int hdcr_apply_g5dwf(const hdcr_geom* gp, const hdcr_dwf_params* p, c
     stencil_timer_end(slot, as_stream(stream));
     return s;
   }
-  if (dtype == HDCR_C128) return launch_g5dwf<double>(g, p->M5, p->mf, U, in, out, nrhs, as_stream(stream));
+  if (dtype == HDCR_C128) {
+    cudaStream_t st = as_stream(stream);
+    const size_t one = fx_scratch_bytes(g, 1), all = fx_scratch_bytes(g, nrhs), most = (size_t)1 << 30;
+    const size_t bytes = all <= most ? all : one > most ? one : most;
+    void* scratch = nullptr;
+    if (!fx_ok(g) || cudaMallocAsync(&scratch, bytes, st) != cudaSuccess) {
+      cudaGetLastError();
+      scratch = nullptr;
+    }
+    const int s = apply_c128(g, p, U, in, out, nrhs, scratch, bytes, st);
+    if (scratch) cudaFreeAsync(scratch, st);
+    return s;
+  }
   if (dtype == HDCR_C64) return launch_g5dwf<float>(g, p->M5, p->mf, U, in, out, nrhs, as_stream(stream));
   set_error("hdcr_apply_g5dwf: unknown dtype %d", dtype);
   return HDCR_ERR_BAD_ARG;

@@ -1,0 +1,786 @@
+// Fine operator H = Gamma5 D_dwf in FP64 accuracy on the integer pipe (the format
+// and its error are described in dwf_fx.cuh).
+#include "dwf_fx.cuh"
+#include "dwf_stencil.cuh"
+
+namespace hdcr {
+
+typedef long long i64;
+typedef unsigned long long u64;
+
+constexpr int FX_UP = 6;  // a field's largest components: 2^58 <= |V| < 2^59; a link's one more
+
+// ------------------------------------------------------------------ encoding
+// (H, L) of V: H the nearest multiple of 2^30, L the rest as a float in units of it
+__device__ __forceinline__ int2 fx_limbs(i64 v) {
+  const i64 t = v + (1LL << 29);
+  const float l = (float)((int)((unsigned)t & 0x3fffffffu) - (1 << 29)) * 0x1p-30f;
+  return make_int2((int)(t >> 30), __float_as_int(l));
+}
+
+// V of one component of a group whose largest biased exponent is mx (in range), that exponent's
+// numbers scaled to 2^(52 + up) .. 2^(53 + up), rounded to nearest
+__device__ __forceinline__ i64 fx_fixed(double x, int mx, int up) {
+  const int hi = __double2hiint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  const int d = min(mx - e, 62);
+  const u64 m = ((u64)(unsigned)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(x)) << up;
+  const i64 v = (i64)((m + ((1ull << d) >> 1)) >> d);
+  return hi < 0 ? -v : v;
+}
+
+// the largest biased exponent << 20 (and lower mantissa bits) of N complex numbers, and in bit
+// 31 whether any is not zero
+template <int N>
+__device__ __forceinline__ unsigned fx_top(const cpx<double> (&x)[N]) {
+  unsigned top = 0, any = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const unsigned a = __double2hiint(x[i].re) & 0x7fffffff, b = __double2hiint(x[i].im) & 0x7fffffff;
+    top = max(top, max(a, b));
+    any |= a | b | __double2loint(x[i].re) | __double2loint(x[i].im);
+  }
+  return top | (any != 0 ? 0x80000000u : 0u);
+}
+
+// the exponent mark of a group with that top
+__device__ __forceinline__ int fx_mark(unsigned top, int emin, int emax) {
+  const int mx = (int)(top >> 20) & 0x7ff;
+  return !(top >> 31) ? 0 : mx < emin || mx > emax ? FX_RAW : mx;
+}
+
+// one number of a group with exponent mark ex
+__device__ __forceinline__ int4 fx_encode(cpx<double> x, int ex, int up) {
+  if (ex == FX_RAW)
+    return make_int4(__double2hiint(x.re), __double2loint(x.re), __double2hiint(x.im), __double2loint(x.im));
+  if (ex == 0) return make_int4(0, 0, 0, 0);
+  const int2 a = fx_limbs(fx_fixed(x.re, ex, up)), b = fx_limbs(fx_fixed(x.im, ex, up));
+  return make_int4(a.x, a.y, b.x, b.y);
+}
+
+// r 2^(be - 1086), be the biased exponent that a leading bit 63 would have, rounded to nearest
+__device__ __forceinline__ double fx_to_double(i64 r, int be) {
+  const u64 m = (u64)(r < 0 ? -r : r);
+  if (m == 0) return 0.0;
+  const int lz = __clzll((i64)m);
+  const u64 n = (m << lz) >> 1;  // leading bit 62
+  const u64 q = ((n + 0x1ff + ((n >> 10) & 1)) >> 10) + ((u64)(be - lz - 1) << 52);
+  return __longlong_as_double((i64)(q | ((u64)r & 0x8000000000000000ull)));
+}
+
+// the FP64 value of an encoded number of a field (scale 1051) or a link (1052)
+__device__ __forceinline__ double fx_value(int h, int l, int ex, int scale) {
+  if (ex == FX_RAW) return __hiloint2double(h, l);
+  return ldexp((double)h + (double)__int_as_float(l), ex - scale);
+}
+__device__ __forceinline__ cpx<double> fx_value(int4 w, int ex, int scale) {
+  return cpx<double>(fx_value(w.x, w.y, ex, scale), fx_value(w.z, w.w, ex, scale));
+}
+
+// One launch: the first fblocks CTAs encode a field's 5d sites, the others links.
+// Bound by the memory it streams (32 B per complex number): 16^4 x 16, 0.48 GB.
+__global__ void __launch_bounds__(128) fx_encode_kernel(int ls, i64 nsites, const cpx<double>* __restrict__ in,
+                                                        FxField f, int fblocks, i64 nlinks,
+                                                        const cpx<double>* __restrict__ U, FxLinks u) {
+  if ((int)blockIdx.x < fblocks) {
+    const i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nsites) return;
+    const i64 x4 = i / ls;
+    const i64 o = x4 * 12 * ls + (i - x4 * ls);
+    cpx<double> x[12];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) x[c] = ld(in + o + c * ls);
+    const int ex = fx_mark(fx_top(x), FX_SITE_MIN, FX_SITE_MAX);
+#pragma unroll
+    for (int c = 0; c < 12; ++c) f.v[o + c * ls] = fx_encode(x[c], ex, FX_UP);
+    f.ex[i] = ex;
+  } else {
+    const i64 i = (i64)(blockIdx.x - fblocks) * blockDim.x + threadIdx.x;
+    if (i >= nlinks) return;
+    cpx<double> x[9];
+#pragma unroll
+    for (int c = 0; c < 9; ++c) x[c] = ld(U + i * 9 + c);
+    const int ex = fx_mark(fx_top(x), FX_LINK_MIN, FX_LINK_MAX);
+#pragma unroll
+    for (int c = 0; c < 9; ++c) u.v[i * 9 + c] = fx_encode(x[c], ex, FX_UP + 1);
+    u.ex[i] = ex;
+  }
+}
+
+// ------------------------------------------------------------------- stencil
+// a real coefficient of the operator, encoded on the host
+struct FxCoef {
+  int h, ex;
+  float l;
+  double d;
+};
+
+struct FxParams {
+  FxCoef diag, one, mmf;  // 5 - M5, 1 (the s-hops' weight) and -mf (their weight across a wall)
+};
+
+__device__ __forceinline__ int4 ldi(const int4* p) { return __ldg(p); }
+
+// (row, lower component) tables of i sigma_k: component a of i sigma_k w is
+// sign * i^rot * w[1 - a or a]
+template <int K>
+struct ISigma {
+  static constexpr int idx(int a) { return K < 2 ? 1 - a : a; }
+  static constexpr int rot() { return K == 1 || K == 3 ? 0 : 1; }
+  // K = 0: (i w1, i w0); 1: (w1, -w0); 2: (i w0, -i w1); 3 (gamma_t): (-w0, -w1)
+  static constexpr int sign(int a) { return K == 0 ? 1 : K == 3 ? -1 : a == 0 ? 1 : -1; }
+};
+
+// u + S i^rot d
+__device__ __forceinline__ int4 fx_add(int4 u, int4 d, int S, int rot) {
+  const float ul = __int_as_float(u.y), um = __int_as_float(u.w), dl = __int_as_float(d.y), dm = __int_as_float(d.w);
+  if (rot == 0)
+    return S > 0 ? make_int4(u.x + d.x, __float_as_int(ul + dl), u.z + d.z, __float_as_int(um + dm))
+                 : make_int4(u.x - d.x, __float_as_int(ul - dl), u.z - d.z, __float_as_int(um - dm));
+  return S > 0 ? make_int4(u.x - d.z, __float_as_int(ul - dm), u.z + d.x, __float_as_int(um + dl))
+               : make_int4(u.x + d.z, __float_as_int(ul + dm), u.z - d.x, __float_as_int(um - dl));
+}
+
+__device__ __forceinline__ i64 mw(int a, int b, i64 c) { return c + (i64)a * b; }
+
+// acc -= one hop without its factor 1/2, each colour component of its two spins rounded to
+// nearest after a right shift by sh.  acc[spin][colour][re, im].
+template <int MU, int SIGN>
+__device__ __forceinline__ void fx_hop(const int4* __restrict__ Ul, const int4* __restrict__ nb, int ls, int sh,
+                                       bool flip, i64 (&acc)[4][3][2]) {
+  typedef ISigma<MU> T;
+  // the two spins of h = u -+ ..., their high limbs as integers and as floats, and their low limbs
+  int h[2][3][2];
+  float f[2][3][2], l[2][3][2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int4 u = ldi(nb + (3 * j + c) * ls), d = ldi(nb + (6 + 3 * T::idx(j) + c) * ls);
+      int4 w = fx_add(u, d, SIGN * T::sign(j), T::rot());
+      if (MU == 3 && flip)  // the antiperiodic boundary's factor -1
+        w = make_int4(-w.x, w.y ^ 0x80000000, -w.z, w.w ^ 0x80000000);
+      h[j][c][0] = w.x;
+      h[j][c][1] = w.z;
+      f[j][c][0] = (float)w.x;
+      f[j][c][1] = (float)w.z;
+      l[j][c][0] = __int_as_float(w.y);
+      l[j][c][1] = __int_as_float(w.w);
+    }
+  const i64 half = 1LL << (sh - 1);
+  const float down = __int_as_float((127 - sh) << 23);  // 2^-sh
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    int mr[3], mi[3];
+    float fr[3], fi[3], lr[3], li[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int4 m = ldi(Ul + (SIGN > 0 ? 3 * c + b : 3 * b + c));
+      mr[b] = m.x;
+      mi[b] = m.z;
+      fr[b] = (float)m.x;
+      fi[b] = (float)m.z;
+      lr[b] = __int_as_float(m.y);
+      li[b] = __int_as_float(m.w);
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      // re: m.re v.re -+ m.im v.im;  im: m.re v.im +- m.im v.re
+      i64 hr = half, hi = half;
+      float cr = 0.f, ci = 0.f;
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const int n = -mi[b];
+        hr = mw(SIGN > 0 ? n : mi[b], h[j][b][1], mw(mr[b], h[j][b][0], hr));
+        hi = mw(SIGN > 0 ? mi[b] : n, h[j][b][0], mw(mr[b], h[j][b][1], hi));
+        cr = fmaf(fr[b], l[j][b][0], fmaf(lr[b], f[j][b][0], cr));
+        ci = fmaf(fr[b], l[j][b][1], fmaf(lr[b], f[j][b][1], ci));
+        const float s = SIGN > 0 ? 1.f : -1.f;
+        cr = fmaf(-s * fi[b], l[j][b][1], fmaf(-s * li[b], f[j][b][1], cr));
+        ci = fmaf(s * fi[b], l[j][b][0], fmaf(s * li[b], f[j][b][0], ci));
+      }
+      const i64 pr = (hr >> sh) + __float2int_rn(cr * down), pi = (hi >> sh) + __float2int_rn(ci * down);
+      acc[j][c][0] -= pr;
+      acc[j][c][1] -= pi;
+      // lower = -+ i sigma h, subtracted: component a takes S i^rot of spin j = idx(a)
+      const int a = T::idx(j), S = MU == 3 ? SIGN : SIGN * T::sign(a);
+      if (T::rot() == 0) {
+        acc[2 + a][c][0] += S > 0 ? pr : -pr;
+        acc[2 + a][c][1] += S > 0 ? pi : -pi;
+      } else {
+        acc[2 + a][c][0] += S > 0 ? -pi : pi;
+        acc[2 + a][c][1] += S > 0 ? pr : -pr;
+      }
+    }
+  }
+}
+
+// k v rounded to nearest after a right shift by sh >= 0
+__device__ __forceinline__ i64 fx_mul(const FxCoef& k, int h, int l, int sh) {
+  const float c = fmaf((float)k.h, __int_as_float(l), k.l * (float)h);
+  return (mw(k.h, h, (1LL << sh) >> 1) >> sh) + __float2int_rn(c * __int_as_float((127 - sh) << 23));
+}
+
+// ------------------------------------------------ sites that need FP64 itself
+template <int MU, int SIGN>
+__device__ void fx_slow_hop(const Geom& g, const FxLinks& u, const FxField& in, int ls, int x4, int s, const int co[4],
+                            cpx<double> (&acc)[4][3]) {
+  int ph;
+  const int y4 = neighbour<MU, SIGN>(g, co, &ph);
+  const int l4 = MU * g.V4 + (SIGN > 0 ? x4 : y4);
+  const int le = u.ex[l4], fe = in.ex[y4 * ls + s];
+  cpx<double> m[9], v[12];
+  for (int i = 0; i < 9; ++i) m[i] = fx_value(u.v[(unsigned)(l4 * 9) + i], le, 1052);
+  for (int c = 0; c < 12; ++c) v[c] = fx_value(in.v[(unsigned)(y4 * 12 * ls + s) + c * ls], fe, 1051);
+  const double coef = -0.5 * ph;
+  for (int c = 0; c < 3; ++c) {
+    cpx<double> p[2];
+    for (int a = 0; a < 2; ++a) {
+      cpx<double> t(0.0, 0.0);
+      for (int b = 0; b < 3; ++b) {
+        const cpx<double> d = v[6 + 3 * ISigma<MU>::idx(a) + b];
+        const cpx<double> w = ISigma<MU>::rot() ? times_i(d) : d;
+        const double sg = SIGN * ISigma<MU>::sign(a);
+        const cpx<double> h(v[3 * a + b].re + sg * w.re, v[3 * a + b].im + sg * w.im);
+        t = SIGN > 0 ? cmadd(t, m[3 * c + b], h) : cjmadd(t, m[3 * b + c], h);
+      }
+      p[a] = t;
+      acc[a][c].re = fma(coef, t.re, acc[a][c].re);
+      acc[a][c].im = fma(coef, t.im, acc[a][c].im);
+    }
+    for (int a = 0; a < 2; ++a) {
+      const cpx<double> q = p[ISigma<MU>::idx(a)];
+      const cpx<double> w = ISigma<MU>::rot() ? times_i(q) : q;
+      const double cl = coef * (MU == 3 ? -SIGN : -SIGN * ISigma<MU>::sign(a));
+      acc[2 + a][c].re = fma(cl, w.re, acc[2 + a][c].re);
+      acc[2 + a][c].im = fma(cl, w.im, acc[2 + a][c].im);
+    }
+  }
+}
+
+// (D_dwf in)(x4, s) in FP64 arithmetic from the encoded operands
+__device__ void fx_slow_site(const Geom& g, const FxParams& p, const FxLinks& u, const FxField& in, int x4, int s,
+                             cpx<double> (&acc)[4][3]) {
+  const int ls = g.Ls;
+  int co[4];
+  x4_coords(g, x4, co);
+  const int sn = s + 1 == ls ? 0 : s + 1, sp = s == 0 ? ls - 1 : s - 1;
+  const double wn = s + 1 == ls ? p.mmf.d : 1.0, wp = s == 0 ? p.mmf.d : 1.0;
+  const int4* b = in.v + (unsigned)(x4 * 12 * ls);
+  const int* e = in.ex + (unsigned)(x4 * ls);
+  for (int c = 0; c < 12; ++c) {
+    const cpx<double> v = fx_value(b[c * ls + s], e[s], 1051);
+    const int so = c < 6 ? sp : sn;
+    const double w = c < 6 ? wp : wn;
+    const cpx<double> o = fx_value(b[c * ls + so], e[so], 1051);
+    acc[c / 3][c % 3] = cpx<double>(fma(-w, o.re, p.diag.d * v.re), fma(-w, o.im, p.diag.d * v.im));
+  }
+  fx_slow_hop<0, 1>(g, u, in, ls, x4, s, co, acc);
+  fx_slow_hop<0, -1>(g, u, in, ls, x4, s, co, acc);
+  fx_slow_hop<1, 1>(g, u, in, ls, x4, s, co, acc);
+  fx_slow_hop<1, -1>(g, u, in, ls, x4, s, co, acc);
+  fx_slow_hop<2, 1>(g, u, in, ls, x4, s, co, acc);
+  fx_slow_hop<2, -1>(g, u, in, ls, x4, s, co, acc);
+  fx_slow_hop<3, 1>(g, u, in, ls, x4, s, co, acc);
+  fx_slow_hop<3, -1>(g, u, in, ls, x4, s, co, acc);
+}
+
+// ------------------------------------------------------------------ the kernel
+// What a launch does with h = H in at each site
+constexpr int FX_OUT = 0;    // out = h
+constexpr int FX_ENC = 1;    // h encoded into enc
+constexpr int FX_BOTH = 2;   // out = h, h encoded into enc
+constexpr int FX_DOT = 3;    // out = h and Re <src, h> into *result
+constexpr int FX_RES = 4;    // out = src - h, also encoded into enc
+constexpr int FX_CHEB = 5;   // prev <- nx = 2 (a h + b cur) - prev, acc += ck nx, nx encoded into enc
+constexpr int FX_CHEB1 = 6;  // prev <- nx = a h + b cur, acc = c0 cur + ck nx, nx encoded into enc
+constexpr int FX_CHEBL = 7;  // acc += ck (2 (a h + b cur) - prev), acc encoded into enc
+struct FxEpilogue {
+  cpx<double>* out;
+  FxField enc;
+  const cpx<double>* src;
+  const cpx<double>* cur;
+  cpx<double>* prev;
+  cpx<double>* acc;
+  double a, b, ck, c0;
+  RedScratch rs;
+  double* result;
+};
+
+// one complex number of the epilogue: h in, the value to encode out.  The Chebyshev steps
+// are three FP64 multiply-adds a real, each a quarter of the clock that the whole stencil
+// takes per real on the integer and FP32 pipes.
+template <int MODE>
+__device__ __forceinline__ cpx<double> fx_epilogue(const FxEpilogue& ep, i64 o, cpx<double> h, double& dot) {
+  if (MODE == FX_OUT || MODE == FX_BOTH || MODE == FX_DOT) st(ep.out + o, h);
+  if (MODE == FX_DOT) {
+    const cpx<double> q = ld(ep.src + o);
+    dot = fma(q.re, h.re, fma(q.im, h.im, dot));
+  }
+  if (MODE == FX_RES) {
+    h = ld(ep.src + o) - h;
+    st(ep.out + o, h);
+  }
+  if (MODE == FX_CHEB || MODE == FX_CHEBL || MODE == FX_CHEB1) {
+    const cpx<double> cv = ld(ep.cur + o);
+    cpx<double> nx, av;
+    if (MODE == FX_CHEB1) {
+      nx.re = fma(ep.a, h.re, ep.b * cv.re);
+      nx.im = fma(ep.a, h.im, ep.b * cv.im);
+      av = cpx<double>(ep.c0 * cv.re, ep.c0 * cv.im);
+    } else {
+      const cpx<double> pv = ld(ep.prev + o);
+      const double a2 = 2.0 * ep.a, b2 = 2.0 * ep.b;
+      nx.re = fma(a2, h.re, fma(b2, cv.re, -pv.re));
+      nx.im = fma(a2, h.im, fma(b2, cv.im, -pv.im));
+      if (ep.acc) av = ld(ep.acc + o);
+    }
+    if (MODE != FX_CHEBL) st(ep.prev + o, nx);
+    if (ep.acc) {
+      av.re = fma(ep.ck, nx.re, av.re);
+      av.im = fma(ep.ck, nx.im, av.im);
+      st(ep.acc + o, av);
+    }
+    h = MODE == FX_CHEBL ? av : nx;
+  }
+  return h;
+}
+
+// A CTA's 4d sites: the box b[] of the lattice (n[] boxes in each direction), or ns
+// consecutive ones in the field's order when b[0] is 0
+struct FxTile {
+  int b[4], n[4];
+  int ns;     // 4d sites per tile
+  int tiles;  // tiles per field
+};
+
+constexpr int FX_THREADS = 256;  // (4d site, s) of a tile
+constexpr int FX_BLOCKS = 2;     // full tiles per SM
+constexpr int FX_MAX_SITES = FX_THREADS / 2;  // Ls >= 2
+
+// A site that reads an operand outside the format: the whole of its output.  Returns
+// its share of the dot product.
+template <int MODE>
+__device__ __noinline__ double fx_slow_output(Geom g, FxParams p, FxLinks u, FxField in, FxEpilogue ep, int r, int x4,
+                                              int s) {
+  cpx<double> a[4][3], w[12];
+  fx_slow_site(g, p, u, in, x4, s, a);
+  const int so = g.Ls - 1 - s;
+  const i64 o0 = ((i64)r * g.V4 + x4) * 12 * g.Ls + so;
+  double d = 0.0;
+  for (int c = 0; c < 12; ++c) {
+    const double sg = c < 6 ? 1.0 : -1.0;
+    w[c] = fx_epilogue<MODE>(ep, o0 + c * g.Ls, cpx<double>(sg * a[c / 3][c % 3].re, sg * a[c / 3][c % 3].im), d);
+  }
+  if (MODE != FX_OUT && MODE != FX_DOT && ep.enc.v) {
+    const int ex = fx_mark(fx_top(w), FX_SITE_MIN, FX_SITE_MAX);
+    for (int c = 0; c < 12; ++c) ep.enc.v[o0 + c * g.Ls] = fx_encode(w[c], ex, FX_UP);
+    ep.enc.ex[((i64)r * g.V4 + x4) * g.Ls + so] = ex;
+  }
+  return d;
+}
+
+__device__ __forceinline__ int fx_tile_site(const Geom& g, const FxTile& t, int tile, int i) {
+  if (t.b[0] == 0) return tile * t.ns + i;
+  int co[4];
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    const int q = i / t.b[mu], r = tile / t.n[mu];
+    co[mu] = (tile - r * t.n[mu]) * t.b[mu] + (i - q * t.b[mu]);
+    i = q;
+    tile = r;
+  }
+  return x4_index(g, co);
+}
+
+// entry of the tile's hop table for direction d = 2 mu + (1 for the backward hop):
+// the neighbour's x4 Ls, the link's first element, the link's exponent, 1 for a
+// factor -1 from the t boundary
+__device__ __forceinline__ int4 fx_hop_entry(const Geom& g, const FxLinks& u, int x4, int d) {
+  int co[4];
+  x4_coords(g, x4, co);
+  const int mu = d >> 1;
+  int c = 0, L = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (k == mu) {
+      c = co[k];
+      L = g.L[k];
+    }
+  const bool wrap = d & 1 ? c == 0 : c + 1 == L;
+  const int nc = d & 1 ? (wrap ? L - 1 : c - 1) : (wrap ? 0 : c + 1);
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (k == mu) co[k] = nc;
+  const int y4 = x4_index(g, co);
+  const int l4 = mu * g.V4 + (d & 1 ? y4 : x4);
+  return make_int4(y4 * g.Ls, l4 * 9, u.ex[l4], mu == 3 && wrap && g.bc_t < 0);
+}
+
+// the encoded form of r 2^(C - 2101) in a site whose numbers have at least lz leading sign-equal bits
+__device__ __forceinline__ int2 fx_renorm(i64 r, int lz) {
+  return fx_limbs(lz >= 5 ? r << (lz - 5) : (r + ((1LL << (5 - lz)) >> 1)) >> (5 - lz));
+}
+
+template <int LS>
+__device__ __forceinline__ void fx_site(const Geom& g, const FxParams& p, const FxLinks& u, const FxField& in,
+                                        const int4* tab, int x4, int s, int C, i64 (&acc)[4][3][2]) {
+  const int ls = ls_of<LS>(g);
+#pragma unroll
+  for (int c = 0; c < 12; ++c) acc[c / 3][c % 3][0] = acc[c / 3][c % 3][1] = 0;
+#pragma unroll 1
+  for (int d = 0; d < 8; ++d) {
+    const int4 t = tab[d];
+    const int sh = min(C - (t.z + __ldg(in.ex + t.x + s)) + 3, 61);
+    const int4* nb = in.v + (unsigned)(t.x * 12 + s);
+    const int4* Ul = u.v + (unsigned)t.y;
+    switch (d) {
+      case 0: fx_hop<0, 1>(Ul, nb, ls, sh, false, acc); break;
+      case 1: fx_hop<0, -1>(Ul, nb, ls, sh, false, acc); break;
+      case 2: fx_hop<1, 1>(Ul, nb, ls, sh, false, acc); break;
+      case 3: fx_hop<1, -1>(Ul, nb, ls, sh, false, acc); break;
+      case 4: fx_hop<2, 1>(Ul, nb, ls, sh, false, acc); break;
+      case 5: fx_hop<2, -1>(Ul, nb, ls, sh, false, acc); break;
+      case 6: fx_hop<3, 1>(Ul, nb, ls, sh, t.w != 0, acc); break;
+      default: fx_hop<3, -1>(Ul, nb, ls, sh, t.w != 0, acc); break;
+    }
+  }
+  // diagonal and fifth dimension: the upper spins couple to s - 1, the lower to s + 1
+  const int* e = in.ex + x4 * ls;
+  const int s0 = min(C - (p.diag.ex + __ldg(e + s)) + 2, 61);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const bool wall = h == 0 ? s == 0 : s + 1 == ls;
+    const int so = h == 0 ? (wall ? ls - 1 : s - 1) : (wall ? 0 : s + 1);
+    const FxCoef k = wall ? p.mmf : p.one;
+    const int s1 = min(C - (k.ex + __ldg(e + so)) + 2, 61);
+    const int4* self = in.v + (unsigned)((x4 * 12 + 6 * h) * ls);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      const int4 v = ldi(self + c * ls + s), w = ldi(self + c * ls + so);
+      acc[2 * h + c / 3][c % 3][0] += fx_mul(p.diag, v.x, v.y, s0) - fx_mul(k, w.x, w.y, s1);
+      acc[2 * h + c / 3][c % 3][1] += fx_mul(p.diag, v.z, v.w, s0) - fx_mul(k, w.z, w.w, s1);
+    }
+  }
+}
+
+// the exponent C of a site's terms: (D_dwf in)(x4, s) = sum 2^(C - 2101); FX_RAW / 2 or more
+// where an operand is not in the format
+template <int LS>
+__device__ __forceinline__ int fx_scale(const Geom& g, const FxParams& p, const FxField& in, const int4* tab, int x4,
+                                        int s) {
+  const int ls = ls_of<LS>(g);
+  const int* e = in.ex + x4 * ls;
+  const int wn = s + 1 == ls, wp = s == 0;
+  int C = max(p.diag.ex + __ldg(e + s), max((wn ? p.mmf.ex : p.one.ex) + __ldg(e + (wn ? 0 : s + 1)),
+                                            (wp ? p.mmf.ex : p.one.ex) + __ldg(e + (wp ? ls - 1 : s - 1)))) - 2;
+#pragma unroll
+  for (int d = 0; d < 8; ++d) C = max(C, tab[d].z + __ldg(in.ex + tab[d].x + s));
+  return C;
+}
+
+// Persistent CTAs over the tiles of all fields; a tile's hop table is built while the
+// one before is computed.
+template <int LS, int MODE>
+__global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) g5dwf_fx_kernel(Geom g, FxParams p, FxLinks u, FxField in,
+                                                                         FxEpilogue ep, FxTile t, int total) {
+  __shared__ int4 tabs[2][FX_MAX_SITES * 8];
+  __shared__ int sx4[2][FX_MAX_SITES];
+  const int ls = ls_of<LS>(g);
+  const int site = (int)threadIdx.x / ls, s = (int)threadIdx.x - site * ls;
+  auto fill = [&](int tile, int b) {
+    if (tile >= total) return;
+    const int t4 = tile % t.tiles;
+    for (int i = threadIdx.x; i < t.ns * 8; i += blockDim.x) {
+      const int x4 = fx_tile_site(g, t, t4, i >> 3);
+      if ((i & 7) == 0) sx4[b][i >> 3] = x4;
+      if (x4 < g.V4) tabs[b][i] = fx_hop_entry(g, u, x4, i & 7);
+    }
+  };
+  double acc_d[1] = {0.0};
+  fill(blockIdx.x, 0);
+  __syncthreads();
+  int b = 0;
+  for (int tile = blockIdx.x; tile < total; tile += gridDim.x, b ^= 1) {
+    const int r = tile / t.tiles;
+    const bool on = site < t.ns && sx4[b][min(site, t.ns - 1)] < g.V4;
+    if (on) {
+      const int x4 = sx4[b][site];
+      FxField f{in.v + (i64)r * 12 * g.V5, in.ex + (i64)r * g.V5};
+      const int4* tab = tabs[b] + site * 8;
+      const int C = fx_scale<LS>(g, p, f, tab, x4, s);
+      if (C < FX_RAW / 2) {
+        i64 v[4][3][2];
+        fx_site<LS>(g, p, u, f, tab, x4, s, C, v);
+        const i64 o0 = (i64)r * 12 * g.V5 + (unsigned)(x4 * 12 * ls + (ls - 1 - s));  // the R5 reflection
+#pragma unroll
+        for (int c = 6; c < 12; ++c)
+#pragma unroll
+          for (int k = 0; k < 2; ++k) v[c / 3][c % 3][k] = -v[c / 3][c % 3][k];  // gamma5
+        if (MODE == FX_ENC || MODE == FX_BOTH) {  // encoded from the integers
+          u64 any = 0;
+#pragma unroll
+          for (int i = 0; i < 24; ++i) {
+            const i64 q = v[i / 6][i / 2 % 3][i % 2];
+            any |= (u64)(q ^ (q >> 63));
+          }
+          const int lz = any ? __clzll((i64)any) : 64;
+          int ex = lz == 64 ? 0 : C - lz - 1015;
+          if (lz < 64 && (ex < FX_SITE_MIN || ex > FX_SITE_MAX)) ex = FX_RAW;
+#pragma unroll
+          for (int c = 0; c < 12; ++c) {
+            const i64 re = v[c / 3][c % 3][0], im = v[c / 3][c % 3][1];
+            int4 q = make_int4(0, 0, 0, 0);
+            if (ex == FX_RAW) {
+              q = fx_encode(cpx<double>(fx_to_double(re, C - 1015), fx_to_double(im, C - 1015)), FX_RAW, FX_UP);
+            } else if (ex != 0) {
+              const int2 a = fx_renorm(re, lz), d = fx_renorm(im, lz);
+              q = make_int4(a.x, a.y, d.x, d.y);
+            }
+            ep.enc.v[o0 + c * ls] = q;
+          }
+          ep.enc.ex[(i64)r * g.V5 + x4 * ls + (ls - 1 - s)] = ex;
+        }
+        if (MODE != FX_ENC) {
+          cpx<double> w[12];
+#pragma unroll
+          for (int c = 0; c < 12; ++c)
+            w[c] = fx_epilogue<MODE>(ep, o0 + c * ls, cpx<double>(fx_to_double(v[c / 3][c % 3][0], C - 1015),
+                                                                  fx_to_double(v[c / 3][c % 3][1], C - 1015)),
+                                     acc_d[0]);
+          if ((MODE == FX_RES || MODE == FX_CHEB || MODE == FX_CHEB1 || MODE == FX_CHEBL) && ep.enc.v) {
+            const int ex = fx_mark(fx_top(w), FX_SITE_MIN, FX_SITE_MAX);
+#pragma unroll
+            for (int c = 0; c < 12; ++c) ep.enc.v[o0 + c * ls] = fx_encode(w[c], ex, FX_UP);
+            ep.enc.ex[(i64)r * g.V5 + x4 * ls + (ls - 1 - s)] = ex;
+          }
+        }
+      } else {
+        acc_d[0] += fx_slow_output<MODE>(g, p, u, f, ep, r, x4, s);
+      }
+    }
+    fill(tile + gridDim.x, b ^ 1);
+    __syncthreads();
+  }
+  if (MODE == FX_DOT) {
+    double tot[1];
+    if (grid_reduce<1>(acc_d, ep.rs, tot)) *ep.result = tot[0];
+  }
+}
+
+// ---------------------------------------------------------------------- host
+static size_t up16(size_t b) { return (b + 15) & ~(size_t)15; }
+
+size_t fx_links_bytes(const Geom& g) { return (size_t)g.V4 * 36 * 16 + up16((size_t)g.V4 * 4 * 4); }
+size_t fx_field_bytes(const Geom& g, int nrhs) {
+  return (size_t)g.V5 * nrhs * 12 * 16 + up16((size_t)g.V5 * nrhs * 4);
+}
+FxLinks fx_links_at(const Geom& g, void* mem) {
+  FxLinks u;
+  u.v = (int4*)mem;
+  u.ex = (int*)(u.v + (size_t)g.V4 * 36);
+  return u;
+}
+FxField fx_field_at(const Geom& g, int nrhs, void* mem) {
+  FxField f;
+  f.v = (int4*)mem;
+  f.ex = (int*)(f.v + (size_t)g.V5 * nrhs * 12);
+  return f;
+}
+
+static FxCoef fx_coef(double x) {
+  FxCoef k{0, 0, 0.f, x};
+  if (x == 0.0) return k;
+  int e = 0;
+  const double m = frexp(x, &e);  // 0.5 <= |m| < 1, x = m 2^e: biased exponent e + 1022
+  if (!(fabs(m) < 1.0) || e + 1022 < FX_LINK_MIN || e + 1022 > FX_LINK_MAX) {
+    k.ex = FX_RAW;
+    return k;
+  }
+  const double y = ldexp(m, 30);
+  k.h = (int)rint(y);
+  k.l = (float)(y - k.h);
+  k.ex = e + 1022;
+  return k;
+}
+
+static FxParams fx_params(double M5, double mf) { return FxParams{fx_coef(5.0 - M5), fx_coef(1.0), fx_coef(-mf)}; }
+
+int launch_fx_encode(const Geom& g, const cpx<double>* in, int nrhs, const FxField& f, const cpx<double>* U,
+                     const FxLinks& u, cudaStream_t st) {
+  const i64 nsites = in ? g.V5 * nrhs : 0, nlinks = U ? (i64)g.V4 * 4 : 0;
+  const i64 fb = (nsites + 127) / 128, lb = (nlinks + 127) / 128;
+  if (fb + lb == 0) return HDCR_OK;
+  fx_encode_kernel<<<(unsigned)(fb + lb), 128, 0, st>>>(g.Ls, nsites, in, f, (int)fb, nlinks, U, u);
+  count_launch();
+  HDCR_LAUNCH_CHECK();
+  return HDCR_OK;
+}
+
+bool fx_ok(const Geom& g) { return g.Ls <= FX_THREADS; }
+
+// The tile with the fewest spinors read per 4d site (itself and the neighbours outside)
+// among the boxes that divide the lattice and fill the CTA's warps, or consecutive
+// sites when no box does better; smaller tiles when there would be less than two per SM.
+static FxTile fx_tile(const Geom& g, int nrhs) {
+  int most = FX_THREADS / g.Ls;
+  while (most > 1 && most * g.Ls > 32 && (i64)g.V4 * nrhs / most < 304) most = (most + 1) / 2;
+  if (most > g.V4) most = g.V4;
+  auto cost = [&](int ns, double reads) {
+    const int lanes = (ns * g.Ls + 31) / 32 * 32;
+    return (1.0 + 0.1 * reads) * lanes / (ns * g.Ls);
+  };
+  FxTile t{{0, 0, 0, 0}, {0, 0, 0, 0}, most, (g.V4 + most - 1) / most};
+  const int row = most < g.L[0] ? most : g.L[0];
+  double best = cost(most, 1.0 + 2.0 / row + (row < most ? 4.0 + 2.0 * row / most : 6.0));
+  for (int b3 = 1; b3 <= most && b3 <= g.L[3]; ++b3)
+    for (int b2 = 1; b3 * b2 <= most && b2 <= g.L[2]; ++b2)
+      for (int b1 = 1; b3 * b2 * b1 <= most && b1 <= g.L[1]; ++b1)
+        for (int b0 = 1; b3 * b2 * b1 * b0 <= most && b0 <= g.L[0]; ++b0) {
+          const int b[4] = {b0, b1, b2, b3};
+          double reads = 1.0;
+          bool ok = true;
+          for (int mu = 0; mu < 4; ++mu) {
+            ok = ok && g.L[mu] % b[mu] == 0;
+            reads += b[mu] == g.L[mu] ? 0.0 : 2.0 / b[mu];
+          }
+          if (!ok || cost(b0 * b1 * b2 * b3, reads) >= best) continue;
+          best = cost(b0 * b1 * b2 * b3, reads);
+          t.ns = b0 * b1 * b2 * b3;
+          t.tiles = g.V4 / t.ns;
+          for (int mu = 0; mu < 4; ++mu) {
+            t.b[mu] = b[mu];
+            t.n[mu] = g.L[mu] / b[mu];
+          }
+        }
+  return t;
+}
+
+template <int MODE>
+static int fx_launch(const Geom& g, double M5, double mf, const FxLinks& u, const FxField& in, const FxEpilogue& ep,
+                     int nrhs, cudaStream_t st) {
+  const FxParams p = fx_params(M5, mf);
+  const FxTile t = fx_tile(g, nrhs);
+  const int total = t.tiles * nrhs;
+  const int threads = (t.ns * g.Ls + 31) / 32 * 32;
+  int sms = 0, dev = 0;
+  HDCR_CUDA_TRY(cudaGetDevice(&dev));
+  HDCR_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int fit = sms * (FX_BLOCKS * FX_THREADS / threads);  // CTAs resident at once
+  const int most = fit < RED_MAX_BLOCKS ? fit : RED_MAX_BLOCKS;
+  const int grid = total < most ? total : most;
+  HDCR_DISPATCH_LS(g.Ls, (g5dwf_fx_kernel<LSC, MODE><<<grid, threads, 0, st>>>(g, p, u, in, ep, t, total)));
+  HDCR_LAUNCH_CHECK();
+  return HDCR_OK;
+}
+
+int launch_fx_g5dwf(const Geom& g, double M5, double mf, const FxLinks& u, const FxField& in, cpx<double>* out,
+                    int nrhs, cudaStream_t st, const FxField* enc) {
+  FxEpilogue ep{};
+  ep.out = out;
+  if (enc) ep.enc = *enc;
+  if (!out) return fx_launch<FX_ENC>(g, M5, mf, u, in, ep, nrhs, st);
+  if (enc) return fx_launch<FX_BOTH>(g, M5, mf, u, in, ep, nrhs, st);
+  return fx_launch<FX_OUT>(g, M5, mf, u, in, ep, nrhs, st);
+}
+
+int launch_fx_g5dwf_res(const Geom& g, double M5, double mf, const FxLinks& u, const FxField& in,
+                        const cpx<double>* src, cpx<double>* out, const FxField* enc, int nrhs, cudaStream_t st) {
+  FxEpilogue ep{};
+  ep.src = src;
+  ep.out = out;
+  if (enc) ep.enc = *enc;
+  return fx_launch<FX_RES>(g, M5, mf, u, in, ep, nrhs, st);
+}
+
+int launch_fx_g5dwf_cheb(const Geom& g, double M5, double mf, const FxLinks& u, const FxField& in, const FxChebStep& c,
+                         const FxField& enc, int nrhs, cudaStream_t st) {
+  FxEpilogue ep{};
+  ep.enc = enc;
+  ep.cur = c.cur;
+  ep.prev = c.prev;
+  ep.acc = c.acc;
+  ep.a = c.a;
+  ep.b = c.b;
+  ep.ck = c.ck;
+  ep.c0 = c.c0;
+  if (c.first) return fx_launch<FX_CHEB1>(g, M5, mf, u, in, ep, nrhs, st);
+  if (c.last) return fx_launch<FX_CHEBL>(g, M5, mf, u, in, ep, nrhs, st);
+  return fx_launch<FX_CHEB>(g, M5, mf, u, in, ep, nrhs, st);
+}
+
+int launch_fx_g5dwf_dot(const Geom& g, double M5, double mf, const FxLinks& u, const FxField& in,
+                        const cpx<double>* in64, cpx<double>* out, RedScratch rs, double* result, cudaStream_t st) {
+  FxEpilogue ep{};
+  ep.out = out;
+  ep.src = in64;
+  ep.rs = rs;
+  ep.result = result;
+  return fx_launch<FX_DOT>(g, M5, mf, u, in, ep, 1, st);
+}
+
+size_t fx_scratch_bytes(const Geom& g, int nrhs) { return fx_links_bytes(g) + fx_field_bytes(g, nrhs); }
+
+bool fx_apply_fits(const Geom& g, const void* scratch, size_t bytes) {
+  return fx_ok(g) && scratch && ((uintptr_t)scratch & 15) == 0 && bytes >= fx_scratch_bytes(g, 1);
+}
+
+int launch_fx_apply(const Geom& g, double M5, double mf, const cpx<double>* U, const cpx<double>* in,
+                    cpx<double>* out, int nrhs, void* scratch, size_t bytes, cudaStream_t st) {
+  int fit = nrhs;
+  while (fit > 1 && fx_scratch_bytes(g, fit) > bytes) --fit;
+  const FxLinks u = fx_links_at(g, scratch);
+  for (int r = 0; r < nrhs; r += fit) {
+    const int m = nrhs - r < fit ? nrhs - r : fit;
+    const FxField f = fx_field_at(g, m, (char*)scratch + fx_links_bytes(g));
+    const i64 o = (i64)r * 12 * g.V5;
+    HDCR_TRY(launch_fx_encode(g, in + o, m, f, r == 0 ? U : nullptr, u, st));
+    HDCR_TRY(launch_fx_g5dwf(g, M5, mf, u, f, out + o, m, st));
+  }
+  return HDCR_OK;
+}
+
+void fx_ctx_alloc(FxCtx* c, const Geom& g, int nrhs) {
+  *c = FxCtx();
+  if (!fx_ok(g)) return;
+  const size_t lb = fx_links_bytes(g), fb = fx_field_bytes(g, nrhs);
+  if (cudaMalloc(&c->mem, lb + 2 * fb) != cudaSuccess) {
+    cudaGetLastError();
+    c->mem = nullptr;
+    return;
+  }
+  c->u = fx_links_at(g, c->mem);
+  c->e0 = fx_field_at(g, nrhs, (char*)c->mem + lb);
+  c->e1 = fx_field_at(g, nrhs, (char*)c->mem + lb + fb);
+}
+
+void fx_ctx_free(FxCtx* c) {
+  if (c->mem) cudaFree(c->mem);
+  *c = FxCtx();
+}
+
+int fx_ctx_links(const FxCtx& c, const Geom& g, const cpx<double>* U, cudaStream_t st) {
+  return c.mem ? launch_fx_encode(g, nullptr, 0, c.e0, U, c.u, st) : HDCR_OK;
+}
+
+int fx_ctx_apply(const FxCtx& c, const Geom& g, double M5, double mf, const cpx<double>* in, cpx<double>* out, int nrhs,
+                 cudaStream_t st) {
+  int slot;
+  stencil_timer_begin(0, g.V5 * nrhs, st, &slot);
+  int s = launch_fx_encode(g, in, nrhs, c.e0, nullptr, c.u, st);
+  if (s == HDCR_OK) s = launch_fx_g5dwf(g, M5, mf, c.u, c.e0, out, nrhs, st);
+  stencil_timer_end(slot, st);
+  return s;
+}
+
+int fx_ctx_apply_dot(const FxCtx& c, const Geom& g, double M5, double mf, const cpx<double>* in, cpx<double>* out,
+                     RedScratch rs, double* result, cudaStream_t st) {
+  int slot;
+  stencil_timer_begin(0, g.V5, st, &slot);
+  int s = launch_fx_encode(g, in, 1, c.e0, nullptr, c.u, st);
+  if (s == HDCR_OK) s = launch_fx_g5dwf_dot(g, M5, mf, c.u, c.e0, in, out, rs, result, st);
+  stencil_timer_end(slot, st);
+  return s;
+}
+
+}  // namespace hdcr

@@ -116,6 +116,7 @@ struct SolveCache {
   std::vector<double> cheb_c;
   RedBuffers rb{};       // outer reductions; scal: [0..127] MGS coefficients, 128.. scalars
   cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  FxCtx fx;              // encoded links and fields of the FP64 applications
   CRGraph cgraph;        // the coarse CR's iterations between host checks, replayed every V-cycle
 };
 
@@ -141,6 +142,7 @@ void solve_cache_free(SolveCache* c) {
   if (c->inner == HDCR_C128) free_inner<double>(c);
   if (c->inner == HDCR_C64) free_inner<float>(c);
   cr_graph_free(&c->cgraph);
+  fx_ctx_free(&c->fx);
   if (c->mem) cudaFree(c->mem);
   red_buffers_free(&c->rb);
   for (int i = 0; i < 6; ++i)
@@ -198,6 +200,7 @@ static int alloc_cache(const hdcr_coarse* co, int restart, SolveCache** out) {
     solve_cache_free(c);  // frees whatever part was allocated
     return s;
   }
+  if (!co->cf) fx_ctx_alloc(&c->fx, co->g, 1);
   *out = c;
   return HDCR_OK;
 }
@@ -257,12 +260,45 @@ static int coarse_solve(const hdcr_coarse* co, SolveCache* c, const hdcr_solve_p
   return HDCR_OK;
 }
 
+// out = r - H z (its encoded form left in e1 when ``enc``); in FP64 without the FP64 pipe z is
+// encoded first unless ``zin`` holds it already, and the subtraction rides in the application
+template <typename R>
+static int residual(const FineOp<R>& H, SolveCache* c, const cpx<R>* r, const cpx<R>* z, const FxField* zin, bool enc,
+                    cpx<R>* out, cudaStream_t st) {
+  if constexpr (sizeof(R) == 8) {
+    if (H.fixed()) {
+      const FxField& in = zin ? *zin : H.fx->e0;
+      if (!zin) HDCR_TRY(launch_fx_encode(H.g, z, H.nrhs, in, nullptr, H.fx->u, st));
+      int slot;
+      stencil_timer_begin(0, H.g.V5 * H.nrhs, st, &slot);
+      const int s = launch_fx_g5dwf_res(H.g, H.M5, H.mf, H.fx->u, in, r, out, enc ? &H.fx->e1 : nullptr, H.nrhs, st);
+      stencil_timer_end(slot, st);
+      return s;
+    }
+  }
+  cpx<R>* t1 = (cpx<R>*)c->t1;
+  HDCR_TRY(H.apply(z, t1, st));
+  sub_kernel<R><<<num_blocks(c->fs, 256, 4096), 256, 0, st>>>(r, t1, out, c->fs); count_launch();
+  HDCR_LAUNCH_CHECK();
+  return HDCR_OK;
+}
+
+// e = S t2 after residual(..., enc = true, t2): from its encoded form where there is one
+template <typename R>
+static int smooth_residual(const FineOp<R>& H, SolveCache* c, const hdcr_solve_params* prm, const cpx<R>* t2, cpx<R>* e,
+                           VStats* vs, cudaStream_t st) {
+  if constexpr (sizeof(R) == 8)
+    if (H.fixed() && prm->smoother_kind == HDCR_SMOOTHER_CHEBYSHEV)
+      return cheb_smoother_fx(H, H.fx->e1, H.fx->e0, e, c->cheb_c, prm->cheb_lo, prm->cheb_hi,
+                              *(ChebWork<double>*)c->chw, st, &vs->fine);
+  return smooth<R>(H, c, prm, t2, e, vs, st);
+}
+
 // z = B r in precision R (r, z in R)
 template <typename R>
 static int vcycle(const hdcr_coarse* co, const FineOp<R>& H, SolveCache* c, const hdcr_solve_params* prm,
                   const cpx<R>* r, cpx<R>* z, VStats* vs, cudaStream_t st) {
   const long long fs = c->fs;
-  cpx<R>* t1 = (cpx<R>*)c->t1;
   cpx<R>* t2 = (cpx<R>*)c->t2;
   cpx<R>* e = (cpx<R>*)c->e;
   const int nb = num_blocks(fs, 256, 4096);
@@ -275,12 +311,10 @@ static int vcycle(const hdcr_coarse* co, const FineOp<R>& H, SolveCache* c, cons
     HDCR_TRY(coarse_solve<R>(co, c, prm, vs, st));
     HDCR_TRY(launch_prolong<R>(co->sub, (const cpx<R>*)c->c_sol, (const cpx<R>*)nullptr, z, 1, st));
     HDCR_CUDA_TRY(cudaEventRecord(c->ev[3], st));
-    HDCR_TRY(H.apply(z, t1, st));
+    HDCR_TRY(residual<R>(H, c, r, z, nullptr, true, t2, st));
     vs->fine++;
-    sub_kernel<R><<<nb, 256, 0, st>>>(r, t1, t2, fs); count_launch();
-    HDCR_LAUNCH_CHECK();
     HDCR_CUDA_TRY(cudaEventRecord(c->ev[4], st));
-    HDCR_TRY(smooth<R>(H, c, prm, t2, e, vs, st));
+    HDCR_TRY(smooth_residual<R>(H, c, prm, t2, e, vs, st));
     add_kernel<R><<<nb, 256, 0, st>>>(z, e, fs); count_launch();
     HDCR_LAUNCH_CHECK();
     HDCR_CUDA_TRY(cudaEventRecord(c->ev[5], st));
@@ -291,22 +325,20 @@ static int vcycle(const hdcr_coarse* co, const FineOp<R>& H, SolveCache* c, cons
   HDCR_TRY(smooth<R>(H, c, prm, r, z, vs, st));
   HDCR_CUDA_TRY(cudaEventRecord(c->ev[1], st));
   // r1 = r - H z1;  z2 = z1 + P A^{-1} P^dag r1
-  HDCR_TRY(H.apply(z, t1, st));
+  // (the Chebyshev smoother leaves z encoded in e1)
+  const FxField* zin = H.fixed() && prm->smoother_kind == HDCR_SMOOTHER_CHEBYSHEV ? &H.fx->e1 : nullptr;
+  HDCR_TRY(residual<R>(H, c, r, z, zin, false, t2, st));
   vs->fine++;
-  sub_kernel<R><<<nb, 256, 0, st>>>(r, t1, t2, fs); count_launch();
-  HDCR_LAUNCH_CHECK();
   HDCR_CUDA_TRY(cudaEventRecord(c->ev[2], st));
   HDCR_TRY(launch_restrict<R>(co->sub, t2, (cpx<R>*)c->c_rhs, 1, st));
   HDCR_TRY(coarse_solve<R>(co, c, prm, vs, st));
   HDCR_TRY(launch_prolong<R>(co->sub, (const cpx<R>*)c->c_sol, z, z, 1, st));
   HDCR_CUDA_TRY(cudaEventRecord(c->ev[3], st));
   // r2 = r - H z2;  z = z2 + S r2
-  HDCR_TRY(H.apply(z, t1, st));
+  HDCR_TRY(residual<R>(H, c, r, z, nullptr, true, t2, st));
   vs->fine++;
-  sub_kernel<R><<<nb, 256, 0, st>>>(r, t1, t2, fs); count_launch();
-  HDCR_LAUNCH_CHECK();
   HDCR_CUDA_TRY(cudaEventRecord(c->ev[4], st));
-  HDCR_TRY(smooth<R>(H, c, prm, t2, e, vs, st));
+  HDCR_TRY(smooth_residual<R>(H, c, prm, t2, e, vs, st));
   add_kernel<R><<<nb, 256, 0, st>>>(z, e, fs); count_launch();
   HDCR_LAUNCH_CHECK();
   HDCR_CUDA_TRY(cudaEventRecord(c->ev[5], st));
@@ -321,6 +353,8 @@ static int solve_impl(const hdcr_coarse* co, SolveCache* c, const void* U, const
   const int nb = num_blocks(fs, 256, 4096);
   FineOp<double> H64{co->g, co->M5, co->mf, (const cpx<double>*)U};
   H64.cf = co->cf;
+  H64.fx = &c->fx;
+  HDCR_TRY(fx_ctx_links(c->fx, co->g, (const cpx<double>*)U, st));
   const cpx<R>* Uin = (const cpx<R>*)U;
   if (sizeof(R) != 8) {
     HDCR_TRY(launch_convert(U, HDCR_C128, c->U_in, HDCR_C64, (long long)co->g.V4 * 36, st));
@@ -328,6 +362,7 @@ static int solve_impl(const hdcr_coarse* co, SolveCache* c, const void* U, const
   }
   FineOp<R> Hin{co->g, co->M5, co->mf, Uin};
   Hin.cf = co->cf;
+  Hin.fx = &c->fx;
   if (prm->smoother_kind == HDCR_SMOOTHER_CHEBYSHEV)
     c->cheb_c = cheb_inverse_coeffs(prm->cheb_lo, prm->cheb_hi, prm->smoother_order);
   double* scal = c->rb.scal;    // [0, 2*restart): MGS coefficients; 128: |w|^2; 130: a; 132: |r|^2; 133: |b|^2

@@ -164,6 +164,7 @@ struct MultiCache {
   void *c_rhs = nullptr, *c_sol = nullptr;                                            // nrhs coarse vectors
   void* U_in = nullptr;                                                               // links, inner precision
   void* chw = nullptr;                                                                // ChebWork<R> over nrhs
+  FxCtx fx;                 // encoded links and fields of the FP64 applications
   double* sc = nullptr;     // nrhs x SC device scalars
   double2* part = nullptr;  // nrhs x MB_BLOCKS partial sums
   double* rr = nullptr;     // nrhs x 2: |r_r|^2 (stride 2)
@@ -199,6 +200,7 @@ static void multi_cache_free(MultiCache* c) {
   if (c->exec) cudaGraphExecDestroy(c->exec);
   if (c->cap) cudaStreamDestroy(c->cap);
   if (c->host) cudaFreeHost(c->host);
+  fx_ctx_free(&c->fx);
   if (c->mem) cudaFree(c->mem);
   delete c;
 }
@@ -257,6 +259,7 @@ static int multi_alloc(const hdcr_coarse* co, int nrhs, int restart, MultiCache*
     multi_cache_free(c);
     return s;
   }
+  fx_ctx_alloc(&c->fx, co->g, nrhs);
   *out = c;
   return HDCR_OK;
 }
@@ -361,12 +364,15 @@ static int solve_multi_impl(const hdcr_coarse* co, MultiCache* c, const void* U,
   const int nb = num_blocks(N, 256, 8192);
   const dim3 gb(num_blocks(fs, 256, MB_BLOCKS * 4), nrhs);
   FineOp<double> H64{co->g, co->M5, co->mf, (const cpx<double>*)U, nrhs};
+  H64.fx = &c->fx;
+  HDCR_TRY(fx_ctx_links(c->fx, co->g, (const cpx<double>*)U, st));
   const cpx<R>* Uin = (const cpx<R>*)U;
   if (sizeof(R) != 8) {
     HDCR_TRY(launch_convert(U, HDCR_C128, c->U_in, HDCR_C64, (long long)co->g.V4 * 36, st));
     Uin = (const cpx<R>*)c->U_in;
   }
   FineOp<R> Hin{co->g, co->M5, co->mf, Uin, nrhs};
+  Hin.fx = &c->fx;
   c->cheb_c = cheb_inverse_coeffs(prm->cheb_lo, prm->cheb_hi, prm->smoother_order);
   double* sc = c->sc;
   const int SC = c->SC;

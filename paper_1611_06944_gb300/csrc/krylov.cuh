@@ -3,7 +3,7 @@
 // no host synchronisation.
 #pragma once
 
-#include "blas.cuh"
+#include "dwf_fx.cuh"
 
 namespace hdcr {
 
@@ -30,13 +30,21 @@ struct FineOp {
   // set: the continued-fraction operator of Section 3 (its N components where the
   // domain-wall operator has s) instead of Gamma5 D_dwf; mf is then unused
   const CFCoef* cf = nullptr;
+  // FP64 domain-wall operator only: set (with memory) to run without the FP64 pipe; its links
+  // are encoded by the solver (fx_ctx_links)
+  const FxCtx* fx = nullptr;
+  bool fixed() const { return sizeof(R) == 8 && !cf && fx && fx->mem; }
   long long n() const { return g.V5 * 12 * nrhs; }  // complex entries of one vector
   int apply(const cpx<R>* in, cpx<R>* out, cudaStream_t st) const {
     if (cf) return launch_cf<R>(g, M5, *cf, U, in, out, nrhs, RedScratch{nullptr, nullptr}, nullptr, st);
+    if constexpr (sizeof(R) == 8)
+      if (fixed()) return fx_ctx_apply(*fx, g, M5, mf, in, out, nrhs, st);
     return launch_g5dwf<R>(g, M5, mf, U, in, out, nrhs, st);
   }
   int apply_dot(const cpx<R>* in, cpx<R>* out, RedScratch rs, double* res, cudaStream_t st) const {
     if (cf) return launch_cf<R>(g, M5, *cf, U, in, out, 1, rs, res, st);
+    if constexpr (sizeof(R) == 8)
+      if (fixed()) return fx_ctx_apply_dot(*fx, g, M5, mf, in, out, rs, res, st);
     return launch_g5dwf_dot<R>(g, M5, mf, U, in, out, rs, res, st);
   }
 };

@@ -1,0 +1,167 @@
+"""The FP64 operator in fixed point (dwf_fx.cu): its error against extended precision, every
+form a call can take (scratch for all fields, for one, for none), operands outside the
+format, and the fused epilogues of the solver against the oracle's V-cycle."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import synth
+from oracle import dwf, multigrid as mg
+from gpu_util import dev, host, links, natural, planes, relerr
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def hd():
+    import paper_1611_06944_gb300 as hd
+    return hd
+
+
+def apply_with(hd, lat, U, psi, scratch_fields, mf=0.01):
+    """H psi through the C entry with scratch for that many fields (0: the FP64 kernel)."""
+    g, p = lat.c_geom(), hd._params(1.8, mf)
+    n = psi.numel() // (12 * lat.V5)
+    size = hd._L.hdcr_apply_scratch_bytes(hd.C_ref(g), 0, scratch_fields) if scratch_fields else 0
+    scratch = torch.empty(size, dtype=torch.uint8, device="cuda")
+    out = torch.empty_like(psi)
+    s = hd._L.hdcr_apply_g5dwf_scratch(hd.C_ref(g), hd.C_ref(p), U.data_ptr(), psi.data_ptr(), out.data_ptr(), 0, n,
+                                       scratch.data_ptr() if size else None, size,
+                                       ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert s == 0
+    return out
+
+
+def apply_extended(U, psi, mf, bc):
+    """dwf.apply_H in extended precision (numpy longdouble), its pieces rewritten without BLAS."""
+    U, p = U.astype(np.clongdouble), psi.astype(np.clongdouble)
+    G = [g.astype(np.clongdouble) for g in dwf.GAMMA]
+    one = np.eye(4, dtype=np.clongdouble)
+
+    def colour(M, v):
+        return (M[..., None, None, :, :] * v[..., None, :]).sum(-1)
+
+    def spin(S, v):
+        return (S[:, :, None] * v[..., None, :, :]).sum(-2)
+
+    D = np.longdouble(5.0 - 1.8) * p
+    nxt, prv = np.roll(p, -1, -3), np.roll(p, 1, -3)
+    nxt[..., -1, :, :] *= -np.longdouble(mf)
+    prv[..., 0, :, :] *= -np.longdouble(mf)
+    D[..., 2:, :] -= nxt[..., 2:, :]
+    D[..., :2, :] -= prv[..., :2, :]
+    for mu in range(4):
+        fwd = spin(one - G[mu], colour(U[mu], dwf.shift_fermion(p, mu, +1, bc)))
+        dag = np.conj(np.swapaxes(dwf.shift_links(U[mu], mu, -1), -1, -2))
+        bwd = spin(one + G[mu], colour(dag, dwf.shift_fermion(p, mu, -1, bc)))
+        D = D - np.longdouble(0.5) * (fwd + bwd)
+    out = D[..., ::-1, :, :].copy()
+    out[..., 2:, :] *= -1
+    return out
+
+
+# tiles that divide the lattice and that do not, partial warps, Ls from 2 to the largest a
+# tile takes (256) and one beyond it (the FP64 kernel)
+SHAPES = [((4, 4, 4, 4), 8, 1), ((3, 5, 2, 6), 5, -1), ((7, 3, 5, 2), 16, 1), ((4, 2, 2, 4), 2, -1),
+          ((5, 3, 1, 7), 3, 1), ((2, 2, 3, 2), 33, -1), ((2, 1, 2, 2), 256, 1), ((2, 1, 2, 2), 258, -1)]
+
+
+@pytest.mark.parametrize("L,Ls,bc", SHAPES)
+@pytest.mark.parametrize("wall", [False, True])
+def test_error_is_not_above_the_fp64_kernels(hd, L, Ls, bc, wall):
+    U = synth.gauge_field(L, 0.5, 5000)
+    psi = synth.gaussian_fermion(L, Ls, 5001, count=3)
+    if wall:  # decaying into the fifth dimension
+        s = np.arange(Ls)
+        psi = psi * np.exp(-0.5 * np.minimum(s, Ls - 1 - s))[:, None, None]
+    lat = hd.Lattice(L, Ls, bc)
+    Ud, pd = dev(links(U)), dev(planes(psi))
+    want = np.stack([apply_extended(U, p, 0.01, bc) for p in psi])
+
+    def err(t):
+        d = natural(host(t), L, Ls) - want
+        return float(np.sqrt((np.abs(d) ** 2).sum() / (np.abs(want) ** 2).sum()))
+
+    fp64 = err(apply_with(hd, lat, Ud, pd, 0))
+    full = hd.apply_g5dwf(lat, Ud, pd, 1.8, 0.01)
+    # 1.1e-16 measured on every shape, 1.5e-16 for the FP64 kernel
+    assert err(full) <= fp64 <= 2.5e-16
+    for k in (3, 2, 1):
+        assert torch.equal(apply_with(hd, lat, Ud, pd, k), full)
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), 1e200, 1e-250, 5e-324, 0.0])
+def test_operands_outside_the_format(hd, value):
+    """A site that holds such a value (one component, or a whole site of it) and a link that is
+    not finite: finite results as the FP64 kernel's, infinities and NaN where it has them."""
+    L, Ls, bc = (4, 3, 2, 4), 6, -1
+    lat = hd.Lattice(L, Ls, bc)
+    U0 = dev(links(synth.gauge_field(L, 0.5, 5100)))
+    p0 = dev(planes(synth.gaussian_fermion(L, Ls, 5101)))
+    for what in ("component", "site", "link", "all"):
+        U, psi = U0.clone(), p0.clone()
+        if what == "component":
+            psi[5, 3, 2] = value
+        elif what == "site":
+            psi[5, :, 2] = value
+        elif what == "all":
+            psi[:] = value
+        else:
+            U[1, 7, 0, 1] = value
+        a = torch.view_as_real(apply_with(hd, lat, U, psi, 1))
+        b = torch.view_as_real(apply_with(hd, lat, U, psi, 0))
+        assert torch.equal(torch.isnan(a), torch.isnan(b))
+        assert torch.equal(torch.isposinf(a), torch.isposinf(b)) and torch.equal(torch.isneginf(a), torch.isneginf(b))
+        f = torch.isfinite(b)
+        # per element against the sum of the magnitudes of what a site adds up (24 terms of |psi| <= 10 where
+        # no large value is read): a site next to 1e200 only to its own scale
+        scale = b.abs().masked_fill(~f, 0).reshape(lat.V4, 12, Ls, 2).amax(dim=(1, 3), keepdim=True).expand(
+            lat.V4, 12, Ls, 2).reshape(b.shape).clamp_min(1.0 if what != "all" else 0.0)
+        assert bool(((a - b).abs()[f] <= 4e-15 * scale[f] + 1e-322).all())
+
+
+def test_coefficients_outside_the_format(hd):
+    L, Ls = (2, 3, 2, 2), 4
+    lat = hd.Lattice(L, Ls)
+    U = dev(links(synth.gauge_field(L, 0.5, 5200)))
+    psi = dev(planes(synth.gaussian_fermion(L, Ls, 5201)))
+    for mf in (0.0, 1.0, 1e-60, 1e60):
+        a, b = apply_with(hd, lat, U, psi, 1, mf), apply_with(hd, lat, U, psi, 0, mf)
+        assert relerr(host(a), host(b)) <= 4e-16
+
+
+@pytest.mark.parametrize("cycle", ["symmetric", "post"])
+@pytest.mark.parametrize("order", [1, 2, 3])
+def test_short_smoothers_match_the_oracle(hd, order, cycle):
+    """One outer iteration with smoothers whose recurrence ends in its first, second and third
+    step: each has an epilogue of its own."""
+    L, Ls, block, M5, mf = (4, 4, 4, 4), 6, (2, 2, 2, 2), 1.8, 0.05
+    U = synth.gauge_field(L, 0.3, 5300)
+    b = synth.gaussian_fermion(L, Ls, 5301)
+    vec = synth.gaussian_fermion(L, Ls, 5302, count=8)
+    lat = hd.Lattice(L, Ls)
+    Ud, bd = dev(links(U)), dev(planes(b))
+    sub = hd.subspace_from_vectors(lat, block, dev(planes(vec)))
+    co = hd.build_coarse_op(sub, Ud, M5, mf)
+    x = torch.zeros_like(bd)
+    hd.hdcr_solve_into(co, Ud, bd, x, tol=1e-14, max_outer=1, restart=1, smoother_order=order, coarse_solver="cr",
+                       coarse_tol=1e-13, coarse_max=20000, cycle=cycle)
+    p = mg.HDCRParams(M5=M5, mf=mf, bc_t=1)
+    osub = mg.basis_from_vectors(mg.Geometry(L, Ls, block), vec)
+    A = mg.coarse_op(U, osub, M5, mf, 1)
+    D = mg.coarse_dense(A, osub.geom)
+
+    def S(r):
+        return mg.chebyshev_smoother(U, r, p, 1.0, 64.0, order)
+
+    def Q(c):
+        return np.linalg.solve(D, c.reshape(-1)).reshape(c.shape)
+
+    z = mg.vcycle(U, osub, A, b, p, S=S, Qc=Q, cycle=cycle)
+    w = dwf.apply_H(U, z, M5, mf, 1)
+    want = np.vdot(w, b) / np.vdot(w, w).real * z
+    # the coarse solve's tolerance over the smallest coarse eigenvalue bounds the difference
+    assert relerr(natural(host(x), L, Ls), want) <= 1e-9
