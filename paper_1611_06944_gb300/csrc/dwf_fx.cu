@@ -260,7 +260,7 @@ __device__ void fx_slow_hop(const Geom& g, const FxLinks& u, const FxField& in, 
 
 // (D_dwf in)(x4, s) in FP64 arithmetic from the encoded operands
 __device__ void fx_slow_site(const Geom& g, const FxParams& p, const FxLinks& u, const FxField& in, int x4, int s,
-                             cpx<double> (&acc)[4][3]) {
+                             bool local, cpx<double> (&acc)[4][3]) {
   const int ls = g.Ls;
   int co[4];
   x4_coords(g, x4, co);
@@ -269,6 +269,8 @@ __device__ void fx_slow_site(const Geom& g, const FxParams& p, const FxLinks& u,
   const int4* b = in.v + (unsigned)(x4 * 12 * ls);
   const int* e = in.ex + (unsigned)(x4 * ls);
   for (int c = 0; c < 12; ++c) {
+    acc[c / 3][c % 3] = cpx<double>(0.0, 0.0);
+    if (!local) continue;
     const cpx<double> v = fx_value(b[c * ls + s], e[s], 1051);
     const int so = c < 6 ? sp : sn;
     const double w = c < 6 ? wp : wn;
@@ -295,6 +297,12 @@ constexpr int FX_RES = 4;    // out = src - h, also encoded into enc
 constexpr int FX_CHEB = 5;   // prev <- nx = 2 (a h + b cur) - prev, acc += ck nx, nx encoded into enc
 constexpr int FX_CHEB1 = 6;  // prev <- nx = a h + b cur, acc = c0 cur + ck nx, nx encoded into enc
 constexpr int FX_CHEBL = 7;  // acc += ck (2 (a h + b cur) - prev), acc encoded into enc
+// the red-black launches: the 4d hops alone, h = D_hop in on the sites of one parity
+constexpr int FX_RB = 8;      // out = h
+// w = M5 v - h, v = src: out = w, |w|^2 into *result and Gamma5 w encoded into enc; with dag
+// v = Gamma5 src and out = Gamma5 w
+constexpr int FX_RBS = 9;
+constexpr bool fx_reduces(int mode) { return mode == FX_DOT || mode == FX_RBS; }
 struct FxEpilogue {
   cpx<double>* out;
   FxField enc;
@@ -303,6 +311,7 @@ struct FxEpilogue {
   cpx<double>* prev;
   cpx<double>* acc;
   double a, b, ck, c0;
+  int dag;
   RedScratch rs;
   double* result;
 };
@@ -346,9 +355,50 @@ __device__ __forceinline__ cpx<double> fx_epilogue(const FxEpilogue& ep, i64 o, 
   return h;
 }
 
+// The output of the red-black launches at one site from h = (D_hop in)(x4, s)
+template <int MODE>
+__device__ __forceinline__ void fx_rb_output(const Geom& g, const FxEpilogue& ep, int ls, int x4, int s,
+                                             cpx<double> (&h)[12], double& dot) {
+  const unsigned site = (unsigned)(x4 * 12 * ls);
+  if (MODE == FX_RB) {
+#pragma unroll
+    for (int c = 0; c < 12; ++c) st(ep.out + site + c * ls + s, h[c]);
+    return;
+  }
+  const int sr = ls - 1 - s;
+  // M5 couples the upper spins to s - 1 and the lower to s + 1, with -mf across the wall
+  const int sp = s == 0 ? ls - 1 : s - 1, sn = s + 1 == ls ? 0 : s + 1;
+  const double kp = s == 0 ? ep.c0 : -1.0, kn = s + 1 == ls ? ep.c0 : -1.0;
+#pragma unroll
+  for (int c = 0; c < 12; ++c) {
+    const int so = c < 6 ? sp : sn;
+    const double k = c < 6 ? kp : kn;
+    cpx<double> v = ld(ep.src + site + c * ls + (ep.dag ? sr : s));
+    cpx<double> w = ld(ep.src + site + c * ls + (ep.dag ? ls - 1 - so : so));
+    const double sg = ep.dag && c >= 6 ? -1.0 : 1.0;  // Gamma5
+    h[c].re = fma(sg * k, w.re, fma(sg * ep.a, v.re, -h[c].re));
+    h[c].im = fma(sg * k, w.im, fma(sg * ep.a, v.im, -h[c].im));
+    if (ep.dag) {
+      st(ep.out + site + c * ls + sr, cpx<double>(sg * h[c].re, sg * h[c].im));
+    } else {
+      st(ep.out + site + c * ls + s, h[c]);
+      dot = fma(h[c].re, h[c].re, fma(h[c].im, h[c].im, dot));
+      if (c >= 6) h[c] = cpx<double>(-h[c].re, -h[c].im);
+    }
+  }
+  if (!ep.dag) {
+    const int ex = fx_mark(fx_top(h), FX_SITE_MIN, FX_SITE_MAX);
+#pragma unroll
+    for (int c = 0; c < 12; ++c) ep.enc.v[site + c * ls + sr] = fx_encode(h[c], ex, FX_UP);
+    ep.enc.ex[x4 * ls + sr] = ex;
+  }
+}
+
 // A CTA's 4d sites: the box b[] of the lattice (n[] boxes in each direction), or ns
-// consecutive ones in the field's order when b[0] is 0
+// consecutive ones in the field's order when b[0] is 0.  rb: of the sites of parity par,
+// numbered with half the x extent.
 struct FxTile {
+  int rb, par;
   int b[4], n[4];
   int ns;     // 4d sites per tile
   int tiles;  // tiles per field
@@ -364,7 +414,13 @@ template <int MODE>
 __device__ __noinline__ double fx_slow_output(Geom g, FxParams p, FxLinks u, FxField in, FxEpilogue ep, int r, int x4,
                                               int s) {
   cpx<double> a[4][3], w[12];
-  fx_slow_site(g, p, u, in, x4, s, a);
+  fx_slow_site(g, p, u, in, x4, s, MODE < FX_RB, a);
+  if (MODE >= FX_RB) {
+    double dot = 0.0;
+    for (int c = 0; c < 12; ++c) w[c] = a[c / 3][c % 3];
+    fx_rb_output<MODE>(g, ep, g.Ls, x4, s, w, dot);
+    return dot;
+  }
   const int so = g.Ls - 1 - s;
   const i64 o0 = ((i64)r * g.V4 + x4) * 12 * g.Ls + so;
   double d = 0.0;
@@ -381,15 +437,27 @@ __device__ __noinline__ double fx_slow_output(Geom g, FxParams p, FxLinks u, FxF
 }
 
 __device__ __forceinline__ int fx_tile_site(const Geom& g, const FxTile& t, int tile, int i) {
-  if (t.b[0] == 0) return tile * t.ns + i;
   int co[4];
+  if (t.b[0] == 0) {
+    const int h = tile * t.ns + i;
+    if (!t.rb) return h;
+    if (h >= g.V4 / 2) return g.V4;
+    int r = h / (g.L[0] / 2);
+    co[0] = h - r * (g.L[0] / 2);
+    co[1] = r % g.L[1];
+    r /= g.L[1];
+    co[2] = r % g.L[2];
+    co[3] = r / g.L[2];
+  } else {
 #pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
-    const int q = i / t.b[mu], r = tile / t.n[mu];
-    co[mu] = (tile - r * t.n[mu]) * t.b[mu] + (i - q * t.b[mu]);
-    i = q;
-    tile = r;
+    for (int mu = 0; mu < 4; ++mu) {
+      const int q = i / t.b[mu], r = tile / t.n[mu];
+      co[mu] = (tile - r * t.n[mu]) * t.b[mu] + (i - q * t.b[mu]);
+      i = q;
+      tile = r;
+    }
   }
+  if (t.rb) co[0] = 2 * co[0] + ((t.par + co[1] + co[2] + co[3]) & 1);
   return x4_index(g, co);
 }
 
@@ -422,7 +490,7 @@ __device__ __forceinline__ int2 fx_renorm(i64 r, int lz) {
   return fx_limbs(lz >= 5 ? r << (lz - 5) : (r + ((1LL << (5 - lz)) >> 1)) >> (5 - lz));
 }
 
-template <int LS>
+template <int LS, int MODE>
 __device__ __forceinline__ void fx_site(const Geom& g, const FxParams& p, const FxLinks& u, const FxField& in,
                                         const int4* tab, int x4, int s, int C, i64 (&acc)[4][3][2]) {
   const int ls = ls_of<LS>(g);
@@ -445,6 +513,7 @@ __device__ __forceinline__ void fx_site(const Geom& g, const FxParams& p, const 
       default: fx_hop<3, -1>(Ul, nb, ls, sh, t.w != 0, acc); break;
     }
   }
+  if (MODE >= FX_RB) return;
   // diagonal and fifth dimension: the upper spins couple to s - 1, the lower to s + 1
   const int* e = in.ex + x4 * ls;
   const int s0 = min(C - (p.diag.ex + __ldg(e + s)) + 2, 61);
@@ -466,13 +535,14 @@ __device__ __forceinline__ void fx_site(const Geom& g, const FxParams& p, const 
 
 // the exponent C of a site's terms: (D_dwf in)(x4, s) = sum 2^(C - 2101); FX_RAW / 2 or more
 // where an operand is not in the format
-template <int LS>
+template <int LS, int MODE>
 __device__ __forceinline__ int fx_scale(const Geom& g, const FxParams& p, const FxField& in, const int4* tab, int x4,
                                         int s) {
   const int ls = ls_of<LS>(g);
   const int* e = in.ex + x4 * ls;
   const int wn = s + 1 == ls, wp = s == 0;
-  int C = max(p.diag.ex + __ldg(e + s), max((wn ? p.mmf.ex : p.one.ex) + __ldg(e + (wn ? 0 : s + 1)),
+  int C = 0;
+  if (MODE < FX_RB) C = max(p.diag.ex + __ldg(e + s), max((wn ? p.mmf.ex : p.one.ex) + __ldg(e + (wn ? 0 : s + 1)),
                                             (wp ? p.mmf.ex : p.one.ex) + __ldg(e + (wp ? ls - 1 : s - 1)))) - 2;
 #pragma unroll
   for (int d = 0; d < 8; ++d) C = max(C, tab[d].z + __ldg(in.ex + tab[d].x + s));
@@ -508,13 +578,13 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) g5dwf_fx_kernel(Geom g,
       const int x4 = sx4[b][site];
       FxField f{in.v + (i64)r * 12 * g.V5, in.ex + (i64)r * g.V5};
       const int4* tab = tabs[b] + site * 8;
-      const int C = fx_scale<LS>(g, p, f, tab, x4, s);
+      const int C = fx_scale<LS, MODE>(g, p, f, tab, x4, s);
       if (C < FX_RAW / 2) {
         i64 v[4][3][2];
-        fx_site<LS>(g, p, u, f, tab, x4, s, C, v);
+        fx_site<LS, MODE>(g, p, u, f, tab, x4, s, C, v);
         const i64 o0 = (i64)r * 12 * g.V5 + (unsigned)(x4 * 12 * ls + (ls - 1 - s));  // the R5 reflection
 #pragma unroll
-        for (int c = 6; c < 12; ++c)
+        for (int c = MODE < FX_RB ? 6 : 12; c < 12; ++c)
 #pragma unroll
           for (int k = 0; k < 2; ++k) v[c / 3][c % 3][k] = -v[c / 3][c % 3][k];  // gamma5
         if (MODE == FX_ENC || MODE == FX_BOTH) {  // encoded from the integers
@@ -541,7 +611,13 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) g5dwf_fx_kernel(Geom g,
           }
           ep.enc.ex[(i64)r * g.V5 + x4 * ls + (ls - 1 - s)] = ex;
         }
-        if (MODE != FX_ENC) {
+        if (MODE >= FX_RB) {
+          cpx<double> w[12];
+#pragma unroll
+          for (int c = 0; c < 12; ++c)
+            w[c] = cpx<double>(fx_to_double(v[c / 3][c % 3][0], C - 1015), fx_to_double(v[c / 3][c % 3][1], C - 1015));
+          fx_rb_output<MODE>(g, ep, ls, x4, s, w, acc_d[0]);
+        } else if (MODE != FX_ENC) {
           cpx<double> w[12];
 #pragma unroll
           for (int c = 0; c < 12; ++c)
@@ -562,7 +638,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) g5dwf_fx_kernel(Geom g,
     fill(tile + gridDim.x, b ^ 1);
     __syncthreads();
   }
-  if (MODE == FX_DOT) {
+  if (fx_reduces(MODE) && ep.result) {
     double tot[1];
     if (grid_reduce<1>(acc_d, ep.rs, tot)) *ep.result = tot[0];
   }
@@ -622,7 +698,12 @@ bool fx_ok(const Geom& g) { return g.Ls <= FX_THREADS; }
 // The tile with the fewest spinors read per 4d site (itself and the neighbours outside)
 // among the boxes that divide the lattice and fill the CTA's warps, or consecutive
 // sites when no box does better; smaller tiles when there would be less than two per SM.
-static FxTile fx_tile(const Geom& g, int nrhs) {
+static FxTile fx_tile(const Geom& full, int nrhs, bool rb) {
+  Geom g = full;
+  if (rb) {
+    g.L[0] /= 2;
+    g.V4 /= 2;
+  }
   int most = FX_THREADS / g.Ls;
   while (most > 1 && most * g.Ls > 32 && (i64)g.V4 * nrhs / most < 304) most = (most + 1) / 2;
   if (most > g.V4) most = g.V4;
@@ -630,7 +711,7 @@ static FxTile fx_tile(const Geom& g, int nrhs) {
     const int lanes = (ns * g.Ls + 31) / 32 * 32;
     return (1.0 + 0.1 * reads) * lanes / (ns * g.Ls);
   };
-  FxTile t{{0, 0, 0, 0}, {0, 0, 0, 0}, most, (g.V4 + most - 1) / most};
+  FxTile t{rb, 0, {0, 0, 0, 0}, {0, 0, 0, 0}, most, (g.V4 + most - 1) / most};
   const int row = most < g.L[0] ? most : g.L[0];
   double best = cost(most, 1.0 + 2.0 / row + (row < most ? 4.0 + 2.0 * row / most : 6.0));
   for (int b3 = 1; b3 <= most && b3 <= g.L[3]; ++b3)
@@ -658,9 +739,10 @@ static FxTile fx_tile(const Geom& g, int nrhs) {
 
 template <int MODE>
 static int fx_launch(const Geom& g, double M5, double mf, const FxLinks& u, const FxField& in, const FxEpilogue& ep,
-                     int nrhs, cudaStream_t st) {
+                     int nrhs, cudaStream_t st, int par = 0) {
   const FxParams p = fx_params(M5, mf);
-  const FxTile t = fx_tile(g, nrhs);
+  FxTile t = fx_tile(g, nrhs, MODE >= FX_RB);
+  t.par = par;
   const int total = t.tiles * nrhs;
   const int threads = (t.ns * g.Ls + 31) / 32 * 32;
   int sms = 0, dev = 0;
@@ -682,6 +764,125 @@ int launch_fx_g5dwf(const Geom& g, double M5, double mf, const FxLinks& u, const
   if (!out) return fx_launch<FX_ENC>(g, M5, mf, u, in, ep, nrhs, st);
   if (enc) return fx_launch<FX_BOTH>(g, M5, mf, u, in, ep, nrhs, st);
   return fx_launch<FX_OUT>(g, M5, mf, u, in, ep, nrhs, st);
+}
+
+int launch_fx_rb_hop(const Geom& g, const FxLinks& u, const FxField& in, cpx<double>* out, int par, cudaStream_t st) {
+  FxEpilogue ep{};
+  ep.out = out;
+  return fx_launch<FX_RB>(g, 0.0, 0.0, u, in, ep, 1, st, par);
+}
+
+int launch_fx_rb_schur(const Geom& g, double diag, double mf, const FxLinks& u, const FxField& in,
+                       const cpx<double>* src, cpx<double>* out, bool dag, const FxField& enc, RedScratch rs,
+                       double* norm2, int par, cudaStream_t st) {
+  FxEpilogue ep{};
+  ep.src = src;
+  ep.out = out;
+  ep.enc = enc;
+  ep.a = diag;
+  ep.c0 = mf;
+  ep.dag = dag;
+  ep.rs = rs;
+  ep.result = dag ? nullptr : norm2;
+  return fx_launch<FX_RBS>(g, 0.0, 0.0, u, in, ep, 1, st, par);
+}
+
+// M5^{-1} on the sites of one parity (rbcg.cu describes it), the result encoded: a CTA's rows
+// over s are brought into shared memory in runs, each is substituted by one thread, and a site's
+// 12 rows are encoded together.  FP64 substitution, 3 FP64 instructions a real.
+__global__ void __launch_bounds__(128) fx_rb_m5inv_kernel(Geom g, int ns, const cpx<double>* __restrict__ in, FxField out,
+                                                          int par, double a, double mf) {
+  extern __shared__ cpx<double> rows[];  // [ns * 12][Ls + 1]
+  __shared__ int sx4[64];
+  const int ls = g.Ls, pitch = ls + 1, half = g.V4 / 2;
+  FxTile t{1, par, {0, 0, 0, 0}, {0, 0, 0, 0}, ns, 0};
+  if ((int)threadIdx.x < ns) sx4[threadIdx.x] = fx_tile_site(g, t, blockIdx.x, threadIdx.x);
+  __syncthreads();
+  const int n = min(ns, half - (int)blockIdx.x * ns);  // sites here
+  for (int i = threadIdx.x; i < n * 12 * ls; i += blockDim.x) {
+    const int row = i / ls, s = i - row * ls;
+    rows[row * pitch + s] = in[(unsigned)((sx4[row / 12] * 12 + row % 12) * ls + s)];
+  }
+  __syncthreads();
+  const double ia = 1.0 / a;
+  double aLs = 1.0;  // a^{-Ls}
+  for (int s = 0; s < ls; ++s) aLs *= ia;
+  const double f = mf / (1.0 + mf * aLs);
+  for (int row = threadIdx.x; row < n * 12; row += blockDim.x) {
+    cpx<double>* y = rows + row * pitch;
+    const bool upper = row % 12 < 6;  // substitution from s = 0 up, else from Ls - 1 down
+    const int s0 = upper ? 0 : ls - 1, d = upper ? 1 : -1;
+    cpx<double> z(0.0, 0.0);
+    for (int k = 0, s = s0; k < ls; ++k, s += d) {
+      z = cpx<double>(ia * (y[s].re + z.re), ia * (y[s].im + z.im));
+      y[s] = z;
+    }
+    const cpx<double> gam = f * z;
+    double w = ia;
+    for (int k = 0, s = s0; k < ls; ++k, s += d) {
+      y[s] = cpx<double>(fma(-w, gam.re, y[s].re), fma(-w, gam.im, y[s].im));
+      w *= ia;
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n * ls; i += blockDim.x) {
+    const int site = i / ls, s = i - site * ls;
+    cpx<double> x[12];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) x[c] = rows[(site * 12 + c) * pitch + s];
+    const int ex = fx_mark(fx_top(x), FX_SITE_MIN, FX_SITE_MAX);
+#pragma unroll
+    for (int c = 0; c < 12; ++c) out.v[(unsigned)((sx4[site] * 12 + c) * ls + s)] = fx_encode(x[c], ex, FX_UP);
+    out.ex[sx4[site] * ls + s] = ex;
+  }
+}
+
+int launch_fx_rb_m5inv(const Geom& g, const cpx<double>* in, const FxField& out, int par, double a, double mf,
+                       cudaStream_t st) {
+  int ns = 128 / g.Ls;
+  ns = ns < 1 ? 1 : ns > 32 ? 32 : ns;
+  const size_t smem = sizeof(cpx<double>) * (size_t)ns * 12 * (g.Ls + 1);
+  HDCR_CUDA_TRY(cudaFuncSetAttribute(fx_rb_m5inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  fx_rb_m5inv_kernel<<<(g.V4 / 2 + ns - 1) / ns, 128, smem, st>>>(g, ns, in, out, par, a, mf);
+  count_launch();
+  HDCR_LAUNCH_CHECK();
+  return HDCR_OK;
+}
+
+// p <- r + beta p on the sites of one parity (beta = rr[k ^ 1] / rr[k], 0 where rr[k] is 0), encoded;
+// r null: p as it is
+__global__ void __launch_bounds__(128) fx_rb_p_kernel(Geom g, const cpx<double>* __restrict__ r, cpx<double>* __restrict__ p,
+                                                      FxField out, int par, const double* rr, int k) {
+  const int ls = g.Ls;
+  const i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= g.V5 / 2) return;
+  const int h = (int)(i / ls), s = (int)(i - (i64)h * ls);
+  const FxTile t{1, par, {0, 0, 0, 0}, {0, 0, 0, 0}, 1, 0};
+  const int x4 = fx_tile_site(g, t, h, 0);
+  const double beta = r && rr[k] > 0.0 ? rr[k ^ 1] / rr[k] : 0.0;
+  cpx<double> x[12];
+#pragma unroll
+  for (int c = 0; c < 12; ++c) {
+    const unsigned o = (unsigned)((x4 * 12 + c) * ls + s);
+    x[c] = p[o];
+    if (r) {
+      const cpx<double> v = r[o];
+      x[c] = cpx<double>(fma(beta, x[c].re, v.re), fma(beta, x[c].im, v.im));
+      p[o] = x[c];
+    }
+  }
+  const int ex = fx_mark(fx_top(x), FX_SITE_MIN, FX_SITE_MAX);
+#pragma unroll
+  for (int c = 0; c < 12; ++c) out.v[(unsigned)((x4 * 12 + c) * ls + s)] = fx_encode(x[c], ex, FX_UP);
+  out.ex[x4 * ls + s] = ex;
+}
+
+int launch_fx_rb_p(const Geom& g, const cpx<double>* r, cpx<double>* p, const FxField& out, int par, const double* rr,
+                   int k, cudaStream_t st) {
+  fx_rb_p_kernel<<<num_blocks(g.V5 / 2, 128), 128, 0, st>>>(g, r, p, out, par, rr, k);
+  count_launch();
+  HDCR_LAUNCH_CHECK();
+  return HDCR_OK;
 }
 
 int launch_fx_g5dwf_res(const Geom& g, double M5, double mf, const FxLinks& u, const FxField& in,

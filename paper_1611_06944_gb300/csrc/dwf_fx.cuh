@@ -83,6 +83,20 @@ int launch_fx_g5dwf_cheb(const Geom& g, double M5, double mf, const FxLinks& u, 
 int launch_fx_g5dwf_dot(const Geom& g, double M5, double mf, const FxLinks& u, const FxField& in,
                         const cpx<double>* in64, cpx<double>* out, RedScratch rs, double* result, cudaStream_t st);
 
+// Red-black pieces on the sites of parity par (every extent even; 4d sites of the other
+// parity are read).  hop: out = D_hop in.  schur, with in = M5^{-1} D_hop v encoded:
+// w = M5 v - D_hop in; out = w, |w|^2 into *norm2 and Gamma5 w encoded into enc, or with dag
+// v = Gamma5 src and out = Gamma5 w (norm2 and enc unused).  m5inv: M5^{-1} in, encoded.
+// p: p <- r + (rr[k ^ 1] / rr[k]) p (r null: p unchanged), p encoded.
+int launch_fx_rb_hop(const Geom& g, const FxLinks& u, const FxField& in, cpx<double>* out, int par, cudaStream_t st);
+int launch_fx_rb_schur(const Geom& g, double diag, double mf, const FxLinks& u, const FxField& in,
+                       const cpx<double>* src, cpx<double>* out, bool dag, const FxField& enc, RedScratch rs,
+                       double* norm2, int par, cudaStream_t st);
+int launch_fx_rb_m5inv(const Geom& g, const cpx<double>* in, const FxField& out, int par, double a, double mf,
+                       cudaStream_t st);
+int launch_fx_rb_p(const Geom& g, const cpx<double>* r, cpx<double>* p, const FxField& out, int par, const double* rr,
+                   int k, cudaStream_t st);
+
 // What a solver keeps for FP64 applications of H on nrhs fields: the encoded links and two
 // encoded field vectors.  Without memory for it mem stays null and H runs on the FP64 pipe.
 struct FxCtx {

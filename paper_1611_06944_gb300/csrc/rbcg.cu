@@ -168,17 +168,22 @@ struct RBDev {
   double pad[3];
 };
 
-// x += alpha p; t -= alpha q; r -= alpha Ap with alpha = rr[k] / qq; |r|^2 -> rr[k^1], |t|^2 -> tt
+// x += alpha p; t -= alpha q; r -= alpha Ap with alpha = rr[k] / qq on the odd sites;
+// |r|^2 -> rr[k^1], |t|^2 -> tt
 __global__ void __launch_bounds__(RED_THREADS) rb_update_kernel(cpx<double>* __restrict__ x,
                                                                 const cpx<double>* __restrict__ p,
                                                                 cpx<double>* __restrict__ t,
                                                                 const cpx<double>* __restrict__ q,
                                                                 cpx<double>* __restrict__ r,
-                                                                const cpx<double>* __restrict__ Ap, long long n,
+                                                                const cpx<double>* __restrict__ Ap, Geom g,
                                                                 RBDev* d, int k, RedScratch rs) {
   const double alpha = d->qq > 0.0 ? d->rr[k] / d->qq : 0.0;
   double acc[2] = {0.0, 0.0};
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+  const unsigned per = 12u * (unsigned)g.Ls, n = (unsigned)(g.V4 / 2) * per;
+  for (unsigned j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    const unsigned h = j / per;
+    int co[4];
+    const unsigned i = (unsigned)rb_site(g, (int)h, 1, co) * per + (j - h * per);
     const cpx<double> pv = p[i], qv = q[i], av = Ap[i];
     cpx<double> xv = x[i], tv = t[i], rv = r[i];
     xv.re += alpha * pv.re;
@@ -285,6 +290,8 @@ static int rb_solve_impl(const Geom& g, const hdcr_dwf_params* prm, const cpx<do
     cudaFree(w.mem);
     return s;
   }
+  FxCtx fx;  // the iterations' hops in fixed point; without memory for it they run on the FP64 pipe
+  fx_ctx_alloc(&fx, g, 1);
   RBOp S{g, 5.0 - prm->M5, prm->mf, U, &w};
   RBDev* d = w.dev();
   RedScratch rs = w.rb.rs;
@@ -312,19 +319,38 @@ static int rb_solve_impl(const Geom& g, const hdcr_dwf_params* prm, const cpx<do
       set_error("red-black CGNE: non-finite right-hand side");
       return HDCR_ERR_NONFINITE;
     }
+    if (fx.mem) {
+      HDCR_TRY(fx_ctx_links(fx, g, U, st));
+      HDCR_TRY(launch_fx_rb_p(g, nullptr, w.p, fx.e0, 1, d->rr, 0, st));
+    }
     const double stop2 = tol * tol * ee;
     converged = ee == 0.0 || ring[0] <= stop2;
     constexpr int CHECK = 4;
     for (int k = 0; !converged && k < max_iter; ++k) {
       const int par = k & 1;
-      HDCR_TRY(S.schur(w.p, w.q, st));
-      HDCR_TRY(launch_norm2<double>(w.q, n, rs, &d->qq, st));
-      HDCR_TRY(S.schur_dag(w.q, w.Ap, st));
-      rb_update_kernel<<<red_blocks(n), RED_THREADS, 0, st>>>(w.xo, w.p, w.t, w.q, w.r, w.Ap, n, d, par, rs);
-      count_launch();
-      rb_p_kernel<<<nb, 256, 0, st>>>(w.r, w.p, n, d, par);
+      if (fx.mem) {
+        // q = S p from p encoded in e0, with |q|^2 and Gamma5 q encoded there in its place; Ap = S^dag q
+        HDCR_TRY(launch_fx_rb_hop(g, fx.u, fx.e0, w.a, 0, st));
+        HDCR_TRY(launch_fx_rb_m5inv(g, w.a, fx.e1, 0, S.a, S.mf, st));
+        HDCR_TRY(launch_fx_rb_schur(g, S.a, S.mf, fx.u, fx.e1, w.p, w.q, false, fx.e0, rs, &d->qq, 1, st));
+        HDCR_TRY(launch_fx_rb_hop(g, fx.u, fx.e0, w.a, 0, st));
+        HDCR_TRY(launch_fx_rb_m5inv(g, w.a, fx.e1, 0, S.a, S.mf, st));
+        HDCR_TRY(launch_fx_rb_schur(g, S.a, S.mf, fx.u, fx.e1, w.q, w.Ap, true, fx.e0, rs, nullptr, 1, st));
+      } else {
+        HDCR_TRY(S.schur(w.p, w.q, st));
+        HDCR_TRY(launch_norm2<double>(w.q, n, rs, &d->qq, st));
+        HDCR_TRY(S.schur_dag(w.q, w.Ap, st));
+      }
+      rb_update_kernel<<<red_blocks(n / 2), RED_THREADS, 0, st>>>(w.xo, w.p, w.t, w.q, w.r, w.Ap, g, d, par, rs);
       count_launch();
       HDCR_LAUNCH_CHECK();
+      if (fx.mem) {
+        HDCR_TRY(launch_fx_rb_p(g, w.r, w.p, fx.e0, 1, d->rr, par, st));
+      } else {
+        rb_p_kernel<<<nb, 256, 0, st>>>(w.r, w.p, n, d, par);
+        count_launch();
+        HDCR_LAUNCH_CHECK();
+      }
       iters = k + 1;
       if (iters % CHECK == 0 || iters == max_iter) {
         HDCR_CUDA_TRY(cudaMemcpyAsync(ring, &d->tt, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -354,6 +380,7 @@ static int rb_solve_impl(const Geom& g, const hdcr_dwf_params* prm, const cpx<do
   s = body();
   cudaStreamSynchronize(st);
   red_buffers_free(&w.rb);
+  fx_ctx_free(&fx);
   cudaFree(w.mem);
   if (s == HDCR_OK && !converged) {
     set_error("red-black CGNE: not converged after %d iterations (|r|/|b| = %g)", iters, rel);

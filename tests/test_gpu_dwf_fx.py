@@ -165,3 +165,13 @@ def test_short_smoothers_match_the_oracle(hd, order, cycle):
     want = np.vdot(w, b) / np.vdot(w, w).real * z
     # the coarse solve's tolerance over the smallest coarse eigenvalue bounds the difference
     assert relerr(natural(host(x), L, Ls), want) <= 1e-9
+
+
+@pytest.mark.parametrize("L,Ls,bc", [((4, 6, 2, 8), 7, -1), ((2, 2, 4, 2), 33, 1), ((6, 4, 2, 2), 2, -1)])
+def test_red_black_shapes(hd, L, Ls, bc):
+    """CGNE's fixed-point hops on half lattices whose boxes do not fill a tile, odd and long Ls."""
+    U, b, mf = synth.gauge_field(L, 0.4, 5400), synth.gaussian_fermion(L, Ls, 5401), 0.1
+    x, st = hd.cgne_rb_solve(hd.Lattice(L, Ls, bc), dev(links(U)), dev(planes(b)), 1.8, mf, tol=1e-10)
+    r = b - dwf.apply_H(U, natural(host(x), L, Ls), 1.8, mf, bc)
+    # the Schur residual stops at 1e-10; the reconstruction adds rounding times the condition number
+    assert np.linalg.norm(r) <= 2e-10 * np.linalg.norm(b)
