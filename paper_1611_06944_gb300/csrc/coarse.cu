@@ -18,6 +18,8 @@
 //   leg -mu: H is Hermitian, so A[a][-mu] = (A[a - mu][+mu])^dag.
 // On a coarse extent of 2 the legs +mu and -mu reach the same coarse site and
 // are both kept.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <vector>
 
@@ -414,7 +416,12 @@ __global__ void __launch_bounds__(RED_THREADS) restrict_kernel(Geom g, BlockGeom
                                                                cpx<R>* __restrict__ coarse, int nvec,
                                                                bool table) {
   extern __shared__ int sx4[];  // the block's 4d sites (bvol of them), when ``table``
-  const int a = blockIdx.x;
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  __shared__ double part[2 * RP_KC];
+  __shared__ double warp_sum[2 * RP_KC][RED_THREADS / 32 + 1];
+  static_assert(RP_KC == 8, "the reduction gives each pair of lanes one of 16 values");
+  const int a = blockIdx.x / S;
   const int k0 = blockIdx.y * RP_KC;
   const int r = blockIdx.z;
   const long long fs = g.V5 * 12;
@@ -435,7 +442,7 @@ __global__ void __launch_bounds__(RED_THREADS) restrict_kernel(Geom g, BlockGeom
   // table lookup
   const int per = 12 * g.Ls;
   const int nel = bg.bvol * per;
-  for (int e = threadIdx.x; e < nel; e += RED_THREADS) {
+  for (int e = rank * RED_THREADS + threadIdx.x; e < nel; e += S * RED_THREADS) {
     const int site = e / per;
     const unsigned x4 = table ? (unsigned)sx4[site] : (unsigned)(block_site(g, bg, a, (long long)site * g.Ls) / g.Ls);
     const unsigned off = x4 * (unsigned)per + (unsigned)(e - site * per);
@@ -453,13 +460,36 @@ __global__ void __launch_bounds__(RED_THREADS) restrict_kernel(Geom g, BlockGeom
   double acc[2 * RP_KC];
 #pragma unroll
   for (int i = 0; i < 2 * RP_KC; ++i) acc[i] = (double)tacc[i];
-  block_reduce<2 * RP_KC>(acc);
-  if (threadIdx.x == 0) {
+  // a lane ends with one value's sum over its pairs of lanes: 16 FP64 additions a thread where a
+  // reduction of each value would take 80, which at 2 FP64 operations per clock and SM cost
+  // more than the products of a small block
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int i = 0; i < RP_KC; ++i)
-      if (k0 + i < nvec)
-        coarse[((long long)r * bg.Vc + a) * nvec + k0 + i] = cpx<R>((R)acc[2 * i], (R)acc[2 * i + 1]);
+  for (int w = RP_KC; w >= 1; w >>= 1) {
+    const bool up = lane & (2 * w);  // lane bits 4, 3, 2, 1 choose the half of the values that stays
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const double keep = up ? acc[i + w] : acc[i], send = up ? acc[i] : acc[i + w];
+      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * w);
+    }
   }
+  acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+  if (!(lane & 1)) warp_sum[lane >> 1][threadIdx.x >> 5] = acc[0];
+  __syncthreads();
+  if (threadIdx.x < 2 * RP_KC) {
+    double x = 0.0;
+#pragma unroll
+    for (int w = 0; w < RED_THREADS / 32; ++w) x += warp_sum[threadIdx.x][w];
+    part[threadIdx.x] = x;
+  }
+  cluster.sync();
+  const int i = threadIdx.x;
+  if (rank == 0 && i < 2 * RP_KC && k0 + i / 2 < nvec) {  // the CTAs' sums in their order
+    double x = 0.0;
+    for (int q = 0; q < S; ++q) x += *cluster.map_shared_rank(part + i, q);
+    reinterpret_cast<R*>(coarse + ((long long)r * bg.Vc + a) * nvec + k0)[i] = (R)x;
+  }
+  cluster.sync();  // a CTA's sums stay until they are read
 }
 
 // fine = fine_in + sum_k phi_k c[a][k]   (fine_in may be null)
@@ -486,16 +516,36 @@ __global__ void prolong_kernel(Geom g, BlockGeom bg, const cpx<R>* __restrict__ 
 }
 
 // ---------------------------------------------------------------- launchers
+// CTAs that share a block's restriction as a cluster: more while there are fewer than four per
+// SM and each still has four rounds of its threads.  With 2^3 x 4 coarse sites (8^3 x 16, 16
+// vectors, FP32) a block per CTA left most of the chip idle: 129 us a launch.
+static int restrict_cluster(long long ctas, long long rounds) {
+  int S = 1;
+  while (S < 8 && ctas * S < 4 * 152 && rounds >= 8 * S) S *= 2;
+  return S;
+}
+
 template <typename R>
 int launch_restrict(const hdcr_subspace* sub, const cpx<R>* fine, cpx<R>* coarse, int nrhs, cudaStream_t st) {
-  dim3 grid(sub->bg.Vc, (sub->nvec + RP_KC - 1) / RP_KC, nrhs);
-  // the table of the block's 4d sites in shared memory when it fits (48 KB), else
+  const int chunks = (sub->nvec + RP_KC - 1) / RP_KC;
+  const int S = restrict_cluster((long long)sub->bg.Vc * chunks * nrhs, sub->bg.K5 * 12 / RED_THREADS);
+  // the table of the block's 4d sites in shared memory when it fits (44 KB), else
   // the sites are worked out per element
-  const bool table = sub->bg.bvol <= 12 * 1024;
-  const size_t smem = table ? sizeof(int) * (size_t)sub->bg.bvol : 0;
-  restrict_kernel<R><<<grid, RED_THREADS, smem, st>>>(sub->g, sub->bg, (const cpx<R>*)sub->vecs, fine, coarse,
-                                                      sub->nvec, table); count_launch();
-  HDCR_LAUNCH_CHECK();
+  const bool table = sub->bg.bvol <= 11 * 1024;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(sub->bg.Vc * S, chunks, nrhs);
+  cfg.blockDim = dim3(RED_THREADS);
+  cfg.dynamicSmemBytes = table ? sizeof(int) * (size_t)sub->bg.bvol : 0;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = S;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  HDCR_CUDA_TRY(cudaLaunchKernelEx(&cfg, restrict_kernel<R>, sub->g, sub->bg, (const cpx<R>*)sub->vecs, fine, coarse,
+                                   sub->nvec, table));
+  count_launch();
   return HDCR_OK;
 }
 
