@@ -16,6 +16,7 @@ Tensor layouts (see ``include/hdcr.h``):
 from __future__ import annotations
 
 import ctypes
+import functools
 from dataclasses import dataclass
 
 import torch
@@ -31,7 +32,9 @@ class _LazyLib:
     def __getattr__(self, name):
         if _LazyLib._handle is None:
             _LazyLib._handle = _lib.load()
-        return getattr(_LazyLib._handle, name)
+        fn = getattr(_LazyLib._handle, name)
+        self.__dict__[name] = fn  # found without this method from now on
+        return fn
 
 
 _L = _LazyLib()
@@ -135,14 +138,22 @@ class Lattice:
     Ls: int
     bc_t: int = 1
 
-    @property
+    @functools.cached_property
     def V4(self) -> int:
         Lx, Ly, Lz, Lt = self.L
         return Lx * Ly * Lz * Lt
 
-    @property
+    @functools.cached_property
     def V5(self) -> int:
         return self.V4 * self.Ls
+
+    @functools.cached_property
+    def _scratch(self) -> tuple:
+        """(bytes of links, bytes a field) of an FP64 application's scratch, (0, 0) for none."""
+        g = self.c_geom()
+        one = _L.hdcr_apply_scratch_bytes(C_ref(g), _lib.HDCR_C128, 1)
+        two = _L.hdcr_apply_scratch_bytes(C_ref(g), _lib.HDCR_C128, 2)
+        return one, two - one
 
     def c_geom(self) -> _lib.hdcr_geom:
         g = _lib.hdcr_geom()
@@ -172,8 +183,12 @@ def _dev(t: torch.Tensor, name: str, host_ok: bool = False) -> int:
 
 
 def _stream(stream=None) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():  # calls on host tensors alone
+        torch.cuda.init()
+    # torch.cuda.current_stream().cuda_stream without building a Stream object
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _params(M5: float, mf: float) -> _lib.hdcr_dwf_params:
@@ -182,9 +197,10 @@ def _params(M5: float, mf: float) -> _lib.hdcr_dwf_params:
 
 def _nfields(lat: Lattice, t: torch.Tensor, name: str) -> int:
     per = 12 * lat.V5
-    if t.numel() == 0 or t.numel() % per:
+    n, rest = divmod(t.numel(), per)
+    if n == 0 or rest:
         raise ValueError(f"{name} has {t.numel()} entries, not a multiple of 12*V5 = {per}")
-    return t.numel() // per
+    return n
 
 
 def apply_g5dwf(lat: Lattice, U: torch.Tensor, psi: torch.Tensor, M5: float, mf: float,
@@ -199,7 +215,7 @@ def apply_g5dwf(lat: Lattice, U: torch.Tensor, psi: torch.Tensor, M5: float, mf:
     g = lat.c_geom()
     p = _params(M5, mf)
     args = (C_ref(g), C_ref(p), _dev(U, "U"), _dev(psi, "psi"), _dev(out, "out"), _code(psi), n)
-    scratch = _apply_scratch(g, psi, n, stream)
+    scratch = _apply_scratch(lat, psi, n, stream) if psi.dtype == torch.complex128 else None
     if scratch is None:
         _check(_L.hdcr_apply_g5dwf(*args, _stream(stream)), "apply_g5dwf")
     else:
@@ -211,21 +227,19 @@ def apply_g5dwf(lat: Lattice, U: torch.Tensor, psi: torch.Tensor, M5: float, mf:
 _SCRATCH_MAX = 1 << 30  # most scratch bytes an application over many fields asks torch for
 
 
-def _apply_scratch(g, psi, n, stream):
+def _apply_scratch(lat, psi, n, stream):
     """Scratch of an FP64 application from torch's allocator, allocated on the stream that
     uses it; None where the library allocates what it can itself: under stream capture, and
     when torch is out of memory."""
-    if psi.dtype != torch.complex128:
+    one, field = lat._scratch
+    if one == 0 or torch._C._cuda_isCurrentStreamCapturing():
         return None
-    one = _L.hdcr_apply_scratch_bytes(C_ref(g), _lib.HDCR_C128, 1)
-    size = max(one, min(_L.hdcr_apply_scratch_bytes(C_ref(g), _lib.HDCR_C128, n), _SCRATCH_MAX))
-    if torch.cuda.is_current_stream_capturing():
-        return None
+    size = max(one, min(one + (n - 1) * field, _SCRATCH_MAX))
     try:
         if stream is None:
             return torch.empty(size, dtype=torch.uint8, device=psi.device)
         with torch.cuda.stream(stream):
-            if torch.cuda.is_current_stream_capturing():
+            if torch._C._cuda_isCurrentStreamCapturing():
                 return None
             return torch.empty(size, dtype=torch.uint8, device=psi.device)
     except torch.OutOfMemoryError:

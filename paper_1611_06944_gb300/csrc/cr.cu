@@ -299,7 +299,7 @@ static int cr_solve_impl(const Geom& g, const hdcr_dwf_params* p, const void* U,
   CRConfig cfg;
   cfg.tol = tol;
   cfg.max_iter = max_iter;
-  cfg.check_every = sizeof(R) == 8 ? 2 : 8;
+  cfg.check_every = 8;
   CRGraph graph;  // the iterations between host checks replay from one CUDA graph
   cfg.graph = &graph;
   CRResult res;
