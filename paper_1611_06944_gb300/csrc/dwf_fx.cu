@@ -1,81 +1,9 @@
 // Fine operator H = Gamma5 D_dwf in FP64 accuracy on the integer pipe (the format
 // and its error are described in dwf_fx.cuh).
-#include "dwf_fx.cuh"
 #include "dwf_stencil.cuh"
+#include "fx_device.cuh"
 
 namespace hdcr {
-
-typedef long long i64;
-typedef unsigned long long u64;
-
-constexpr int FX_UP = 6;  // a field's largest components: 2^58 <= |V| < 2^59; a link's one more
-
-// ------------------------------------------------------------------ encoding
-// (H, L) of V: H the nearest multiple of 2^30, L the rest as a float in units of it
-__device__ __forceinline__ int2 fx_limbs(i64 v) {
-  const i64 t = v + (1LL << 29);
-  const float l = (float)((int)((unsigned)t & 0x3fffffffu) - (1 << 29)) * 0x1p-30f;
-  return make_int2((int)(t >> 30), __float_as_int(l));
-}
-
-// V of one component of a group whose largest biased exponent is mx (in range), that exponent's
-// numbers scaled to 2^(52 + up) .. 2^(53 + up), rounded to nearest
-__device__ __forceinline__ i64 fx_fixed(double x, int mx, int up) {
-  const int hi = __double2hiint(x);
-  const int e = (hi >> 20) & 0x7ff;
-  const int d = min(mx - e, 62);
-  const u64 m = ((u64)(unsigned)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(x)) << up;
-  const i64 v = (i64)((m + ((1ull << d) >> 1)) >> d);
-  return hi < 0 ? -v : v;
-}
-
-// the largest biased exponent << 20 (and lower mantissa bits) of N complex numbers, and in bit
-// 31 whether any is not zero
-template <int N>
-__device__ __forceinline__ unsigned fx_top(const cpx<double> (&x)[N]) {
-  unsigned top = 0, any = 0;
-#pragma unroll
-  for (int i = 0; i < N; ++i) {
-    const unsigned a = __double2hiint(x[i].re) & 0x7fffffff, b = __double2hiint(x[i].im) & 0x7fffffff;
-    top = max(top, max(a, b));
-    any |= a | b | __double2loint(x[i].re) | __double2loint(x[i].im);
-  }
-  return top | (any != 0 ? 0x80000000u : 0u);
-}
-
-// the exponent mark of a group with that top
-__device__ __forceinline__ int fx_mark(unsigned top, int emin, int emax) {
-  const int mx = (int)(top >> 20) & 0x7ff;
-  return !(top >> 31) ? 0 : mx < emin || mx > emax ? FX_RAW : mx;
-}
-
-// one number of a group with exponent mark ex
-__device__ __forceinline__ int4 fx_encode(cpx<double> x, int ex, int up) {
-  if (ex == FX_RAW)
-    return make_int4(__double2hiint(x.re), __double2loint(x.re), __double2hiint(x.im), __double2loint(x.im));
-  if (ex == 0) return make_int4(0, 0, 0, 0);
-  const int2 a = fx_limbs(fx_fixed(x.re, ex, up)), b = fx_limbs(fx_fixed(x.im, ex, up));
-  return make_int4(a.x, a.y, b.x, b.y);
-}
-
-// r 2^(be - 1086), be the biased exponent that a leading bit 63 would have, rounded to nearest
-__device__ __forceinline__ double fx_to_double(i64 r, int be) {
-  const u64 m = (u64)(r < 0 ? -r : r);
-  if (m == 0) return 0.0;
-  const int lz = __clzll((i64)m);
-  const u64 n = (m << lz) >> 1;  // leading bit 62
-  const u64 q = ((n + 0x1ff + ((n >> 10) & 1)) >> 10) + ((u64)(be - lz - 1) << 52);
-  return __longlong_as_double((i64)(q | ((u64)r & 0x8000000000000000ull)));
-}
-
-// the FP64 value of an encoded number of a field (scale 1051) or a link (1052)
-__device__ __forceinline__ double fx_value(int h, int l, int ex, int scale) {
-  if (ex == FX_RAW) return __hiloint2double(h, l);
-  return ldexp((double)h + (double)__int_as_float(l), ex - scale);
-}
-__device__ __forceinline__ cpx<double> fx_value(int4 w, int ex, int scale) {
-  return cpx<double>(fx_value(w.x, w.y, ex, scale), fx_value(w.z, w.w, ex, scale));
-}
 
 // One launch: the first fblocks CTAs encode a field's 5d sites, the others links.
 // Bound by the memory it streams (32 B per complex number): 16^4 x 16, 0.48 GB.
@@ -140,8 +68,6 @@ __device__ __forceinline__ int4 fx_add(int4 u, int4 d, int S, int rot) {
   return S > 0 ? make_int4(u.x - d.z, __float_as_int(ul - dm), u.z + d.x, __float_as_int(um + dl))
                : make_int4(u.x + d.z, __float_as_int(ul + dm), u.z - d.x, __float_as_int(um - dl));
 }
-
-__device__ __forceinline__ i64 mw(int a, int b, i64 c) { return c + (i64)a * b; }
 
 // acc -= one hop without its factor 1/2, each colour component of its two spins rounded to
 // nearest after a right shift by sh.  acc[spin][colour][re, im].
@@ -407,6 +333,11 @@ struct FxTile {
 constexpr int FX_THREADS = 256;  // (4d site, s) of a tile
 constexpr int FX_BLOCKS = 2;     // full tiles per SM
 constexpr int FX_MAX_SITES = FX_THREADS / 2;  // Ls >= 2
+constexpr int FX_SPLIT_SITES = 32;  // (4d site, s) of a tile whose sites are split over four warps
+// Launches of at most this many 5d sites split them: encoding and operator, whole sites
+// and split, took 17.3 and 9.3 us at 4^4 x 8 (2048 sites), 24.7 and 20.4 at 18,900, the same at
+// 32,768, and 59.9 and 70.8 at 131,072
+constexpr long long FX_SPLIT_MAX = 24576;
 
 // A site that reads an operand outside the format: the whole of its output.  Returns
 // its share of the dot product.
@@ -490,14 +421,16 @@ __device__ __forceinline__ int2 fx_renorm(i64 r, int lz) {
   return fx_limbs(lz >= 5 ? r << (lz - 5) : (r + ((1LL << (5 - lz)) >> 1)) >> (5 - lz));
 }
 
+// part < 0: the whole site; else direction part's two hops, and with parts 0 and 1 one chirality
+// of the fifth-dimension part
 template <int LS, int MODE>
 __device__ __forceinline__ void fx_site(const Geom& g, const FxParams& p, const FxLinks& u, const FxField& in,
-                                        const int4* tab, int x4, int s, int C, i64 (&acc)[4][3][2]) {
+                                        const int4* tab, int x4, int s, int C, i64 (&acc)[4][3][2], int part = -1) {
   const int ls = ls_of<LS>(g);
 #pragma unroll
   for (int c = 0; c < 12; ++c) acc[c / 3][c % 3][0] = acc[c / 3][c % 3][1] = 0;
 #pragma unroll 1
-  for (int d = 0; d < 8; ++d) {
+  for (int d = part < 0 ? 0 : 2 * part; d < (part < 0 ? 8 : 2 * part + 2); ++d) {
     const int4 t = tab[d];
     const int sh = min(C - (t.z + __ldg(in.ex + t.x + s)) + 3, 61);
     const int4* nb = in.v + (unsigned)(t.x * 12 + s);
@@ -519,6 +452,7 @@ __device__ __forceinline__ void fx_site(const Geom& g, const FxParams& p, const 
   const int s0 = min(C - (p.diag.ex + __ldg(e + s)) + 2, 61);
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
+    if (part >= 0 && part != h) continue;
     const bool wall = h == 0 ? s == 0 : s + 1 == ls;
     const int so = h == 0 ? (wall ? ls - 1 : s - 1) : (wall ? 0 : s + 1);
     const FxCoef k = wall ? p.mmf : p.one;
@@ -644,6 +578,66 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) g5dwf_fx_kernel(Geom g,
   }
 }
 
+// The same for launches that would leave most of the chip idle: the four directions of a site go
+// to the four warps of a CTA, whose sums (exact, so in any order) meet in shared memory, and each
+// warp finishes a quarter of the components.  A thread's chain is a quarter as long.
+template <int LS, int MODE>
+__global__ void __launch_bounds__(4 * FX_SPLIT_SITES, 4) g5dwf_fx_split_kernel(Geom g, FxParams p, FxLinks u, FxField in,
+                                                                              FxEpilogue ep, FxTile t, int total) {
+  __shared__ int4 tabs[FX_SPLIT_SITES / 2 * 8];
+  __shared__ int sx4[FX_SPLIT_SITES / 2];
+  __shared__ i64 sum[24][4][FX_SPLIT_SITES];
+  const int ls = ls_of<LS>(g);
+  const int part = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int site = lane / ls, s = lane - site * ls;
+  double acc_d[1] = {0.0};
+  for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
+    const int r = tile / t.tiles, t4 = tile - r * t.tiles;
+    for (int i = threadIdx.x; i < t.ns * 8; i += blockDim.x) {
+      const int x4 = fx_tile_site(g, t, t4, i >> 3);
+      if ((i & 7) == 0) sx4[i >> 3] = x4;
+      if (x4 < g.V4) tabs[i] = fx_hop_entry(g, u, x4, i & 7);
+    }
+    __syncthreads();
+    const int x4 = site < t.ns ? sx4[site] : g.V4;
+    const bool on = x4 < g.V4;
+    FxField f{in.v + (i64)r * 12 * g.V5, in.ex + (i64)r * g.V5};
+    int C = FX_RAW;
+    if (on) C = fx_scale<LS, MODE>(g, p, f, tabs + site * 8, x4, s);
+    const bool fx = C < FX_RAW / 2;
+    if (fx) {
+      i64 v[4][3][2];
+      fx_site<LS, MODE>(g, p, u, f, tabs + site * 8, x4, s, C, v, part);
+#pragma unroll
+      for (int i = 0; i < 24; ++i) sum[i][part][lane] = v[i / 6][i / 2 % 3][i % 2];
+    }
+    __syncthreads();
+    if (fx) {
+      const i64 o0 = (i64)r * 12 * g.V5 + (unsigned)(x4 * 12 * ls + (ls - 1 - s));  // the R5 reflection
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const int c = 3 * part + j;
+        i64 v[2] = {0, 0};
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) v[k] += sum[2 * c + k][q][lane];
+          if (part >= 2) v[k] = -v[k];  // gamma5
+        }
+        fx_epilogue<MODE>(ep, o0 + c * ls, cpx<double>(fx_to_double(v[0], C - 1015), fx_to_double(v[1], C - 1015)),
+                          acc_d[0]);
+      }
+    } else if (on && part == 0) {
+      acc_d[0] += fx_slow_output<MODE>(g, p, u, f, ep, r, x4, s);
+    }
+    __syncthreads();
+  }
+  if (fx_reduces(MODE)) {
+    double tot[1];
+    if (grid_reduce<1>(acc_d, ep.rs, tot)) *ep.result = tot[0];
+  }
+}
+
 // ---------------------------------------------------------------------- host
 static size_t up16(size_t b) { return (b + 15) & ~(size_t)15; }
 
@@ -698,14 +692,14 @@ bool fx_ok(const Geom& g) { return g.Ls <= FX_THREADS; }
 // The tile with the fewest spinors read per 4d site (itself and the neighbours outside)
 // among the boxes that divide the lattice and fill the CTA's warps, or consecutive
 // sites when no box does better; smaller tiles when there would be less than two per SM.
-static FxTile fx_tile(const Geom& full, int nrhs, bool rb) {
+static FxTile fx_tile(const Geom& full, int nrhs, bool rb, int threads) {
   Geom g = full;
   if (rb) {
     g.L[0] /= 2;
     g.V4 /= 2;
   }
-  int most = FX_THREADS / g.Ls;
-  while (most > 1 && most * g.Ls > 32 && (i64)g.V4 * nrhs / most < 304) most = (most + 1) / 2;
+  int most = threads / g.Ls;
+  while (threads == FX_THREADS && most > 1 && most * g.Ls > 32 && (i64)g.V4 * nrhs / most < 304) most = (most + 1) / 2;
   if (most > g.V4) most = g.V4;
   auto cost = [&](int ns, double reads) {
     const int lanes = (ns * g.Ls + 31) / 32 * 32;
@@ -714,18 +708,18 @@ static FxTile fx_tile(const Geom& full, int nrhs, bool rb) {
   FxTile t{rb, 0, {0, 0, 0, 0}, {0, 0, 0, 0}, most, (g.V4 + most - 1) / most};
   const int row = most < g.L[0] ? most : g.L[0];
   double best = cost(most, 1.0 + 2.0 / row + (row < most ? 4.0 + 2.0 * row / most : 6.0));
-  for (int b3 = 1; b3 <= most && b3 <= g.L[3]; ++b3)
-    for (int b2 = 1; b3 * b2 <= most && b2 <= g.L[2]; ++b2)
-      for (int b1 = 1; b3 * b2 * b1 <= most && b1 <= g.L[1]; ++b1)
+  for (int b3 = 1; b3 <= most && b3 <= g.L[3]; ++b3) {
+    if (g.L[3] % b3) continue;
+    for (int b2 = 1; b3 * b2 <= most && b2 <= g.L[2]; ++b2) {
+      if (g.L[2] % b2) continue;
+      for (int b1 = 1; b3 * b2 * b1 <= most && b1 <= g.L[1]; ++b1) {
+        if (g.L[1] % b1) continue;
         for (int b0 = 1; b3 * b2 * b1 * b0 <= most && b0 <= g.L[0]; ++b0) {
+          if (g.L[0] % b0) continue;
           const int b[4] = {b0, b1, b2, b3};
           double reads = 1.0;
-          bool ok = true;
-          for (int mu = 0; mu < 4; ++mu) {
-            ok = ok && g.L[mu] % b[mu] == 0;
-            reads += b[mu] == g.L[mu] ? 0.0 : 2.0 / b[mu];
-          }
-          if (!ok || cost(b0 * b1 * b2 * b3, reads) >= best) continue;
+          for (int mu = 0; mu < 4; ++mu) reads += b[mu] == g.L[mu] ? 0.0 : 2.0 / b[mu];
+          if (cost(b0 * b1 * b2 * b3, reads) >= best) continue;
           best = cost(b0 * b1 * b2 * b3, reads);
           t.ns = b0 * b1 * b2 * b3;
           t.tiles = g.V4 / t.ns;
@@ -734,6 +728,9 @@ static FxTile fx_tile(const Geom& full, int nrhs, bool rb) {
             t.n[mu] = g.L[mu] / b[mu];
           }
         }
+      }
+    }
+  }
   return t;
 }
 
@@ -741,13 +738,23 @@ template <int MODE>
 static int fx_launch(const Geom& g, double M5, double mf, const FxLinks& u, const FxField& in, const FxEpilogue& ep,
                      int nrhs, cudaStream_t st, int par = 0) {
   const FxParams p = fx_params(M5, mf);
-  FxTile t = fx_tile(g, nrhs, MODE >= FX_RB);
-  t.par = par;
-  const int total = t.tiles * nrhs;
-  const int threads = (t.ns * g.Ls + 31) / 32 * 32;
   int sms = 0, dev = 0;
   HDCR_CUDA_TRY(cudaGetDevice(&dev));
   HDCR_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  if constexpr (MODE == FX_OUT || MODE == FX_DOT) {
+    if (g.Ls <= FX_SPLIT_SITES && g.V5 * nrhs <= FX_SPLIT_MAX) {
+      const FxTile t = fx_tile(g, nrhs, false, FX_SPLIT_SITES);
+      const int total = t.tiles * nrhs, most = sms * 4;
+      HDCR_DISPATCH_LS(g.Ls, (g5dwf_fx_split_kernel<LSC, MODE><<<total < most ? total : most, 4 * FX_SPLIT_SITES, 0, st>>>(
+                                 g, p, u, in, ep, t, total)));
+      HDCR_LAUNCH_CHECK();
+      return HDCR_OK;
+    }
+  }
+  FxTile t = fx_tile(g, nrhs, MODE >= FX_RB, FX_THREADS);
+  t.par = par;
+  const int total = t.tiles * nrhs;
+  const int threads = (t.ns * g.Ls + 31) / 32 * 32;
   const int fit = sms * (FX_BLOCKS * FX_THREADS / threads);  // CTAs resident at once
   const int most = fit < RED_MAX_BLOCKS ? fit : RED_MAX_BLOCKS;
   const int grid = total < most ? total : most;
