@@ -409,23 +409,43 @@ __global__ void __launch_bounds__(RED_THREADS) cdot_re_kernel(const cpx<R>* __re
 // ------------------------------------------------------------ restrict / prolong
 constexpr int RP_KC = 8;  // basis vectors per restrict CTA
 
-template <typename R>
+// Elements e and e + 1 of a field when V is 2 (one 16-byte load of two FP32 complex numbers), else e
+template <typename R, int V>
+struct Elems {
+  cpx<R> x[V];
+};
+template <typename R, int V>
+__device__ __forceinline__ Elems<R, V> ld_elems(const cpx<R>* p) {
+  Elems<R, V> q;
+  if constexpr (V == 2) {
+    const float4 f = __ldg(reinterpret_cast<const float4*>(p));
+    q.x[0] = cpx<R>(f.x, f.y);
+    q.x[1] = cpx<R>(f.z, f.w);
+  } else {
+    q.x[0] = ld(p);
+  }
+  return q;
+}
+
+// NR fields at once (gridDim.z groups of them), so that the basis is read once for all: at
+// 8^3 x 16 x 8 with 24 vectors 12 fields took 392 us one by one.
+template <typename R, int V, int NR>
 __global__ void __launch_bounds__(RED_THREADS) restrict_kernel(Geom g, BlockGeom bg,
                                                                const cpx<R>* __restrict__ phi,
                                                                const cpx<R>* __restrict__ fine,
-                                                               cpx<R>* __restrict__ coarse, int nvec,
+                                                               cpx<R>* __restrict__ coarse, int nvec, int nrhs,
                                                                bool table) {
   extern __shared__ int sx4[];  // the block's 4d sites (bvol of them), when ``table``
   cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
   const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-  __shared__ double part[2 * RP_KC];
+  __shared__ double part[NR][2 * RP_KC];
   __shared__ double warp_sum[2 * RP_KC][RED_THREADS / 32 + 1];
   static_assert(RP_KC == 8, "the reduction gives each pair of lanes one of 16 values");
   const int a = blockIdx.x / S;
   const int k0 = blockIdx.y * RP_KC;
-  const int r = blockIdx.z;
+  const int r0 = blockIdx.z * NR;
   const long long fs = g.V5 * 12;
-  const cpx<R>* v = fine + (long long)r * fs;
+  const cpx<R>* v = fine + (long long)r0 * fs;
   if (table) {
     for (int i = threadIdx.x; i < bg.bvol; i += RED_THREADS)
       sx4[i] = (int)(block_site(g, bg, a, (long long)i * g.Ls) / g.Ls);
@@ -434,85 +454,127 @@ __global__ void __launch_bounds__(RED_THREADS) restrict_kernel(Geom g, BlockGeom
   // each thread sums its elements in R (FP32 for an FP32 basis: the result is
   // stored in FP32, and FP64 arithmetic would bind the kernel to the slow FP64
   // pipe); the threads' partial sums are added in FP64
-  R tacc[2 * RP_KC];
+  R tacc[NR][2 * RP_KC];
 #pragma unroll
-  for (int i = 0; i < 2 * RP_KC; ++i) tacc[i] = (R)0;
+  for (int r = 0; r < NR; ++r)
+#pragma unroll
+    for (int i = 0; i < 2 * RP_KC; ++i) tacc[r][i] = (R)0;
   // elements in the order (4d site of the block, component, s): one 4d site's 12 Ls
   // elements are contiguous in the field, so the index is one 32-bit division and a
   // table lookup
-  const int per = 12 * g.Ls;
+  const int per = 12 * g.Ls / V;
   const int nel = bg.bvol * per;
   for (int e = rank * RED_THREADS + threadIdx.x; e < nel; e += S * RED_THREADS) {
     const int site = e / per;
     const unsigned x4 = table ? (unsigned)sx4[site] : (unsigned)(block_site(g, bg, a, (long long)site * g.Ls) / g.Ls);
-    const unsigned off = x4 * (unsigned)per + (unsigned)(e - site * per);
-    const cpx<R> q = ld(v + off);
+    const unsigned off = (x4 * (unsigned)per + (unsigned)(e - site * per)) * V;
+    Elems<R, V> q[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+      if (NR == 1 || r0 + r < nrhs) q[r] = ld_elems<R, V>(v + r * fs + off);
 #pragma unroll
     for (int i = 0; i < RP_KC; ++i) {
       if (k0 + i < nvec) {
-        const cpx<R> p = ld(phi + (long long)(k0 + i) * fs + off);
-        // conj(p) q accumulated with four FMAs
-        tacc[2 * i] = fma(p.re, q.re, fma(p.im, q.im, tacc[2 * i]));
-        tacc[2 * i + 1] = fma(p.re, q.im, fma(-p.im, q.re, tacc[2 * i + 1]));
+        const Elems<R, V> p = ld_elems<R, V>(phi + (long long)(k0 + i) * fs + off);
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+          if (NR == 1 || r0 + r < nrhs)
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+              // conj(p) q accumulated with four FMAs
+              const cpx<R> x = p.x[j], y = q[r].x[j];
+              tacc[r][2 * i] = fma(x.re, y.re, fma(x.im, y.im, tacc[r][2 * i]));
+              tacc[r][2 * i + 1] = fma(x.re, y.im, fma(-x.im, y.re, tacc[r][2 * i + 1]));
+            }
       }
     }
   }
-  double acc[2 * RP_KC];
 #pragma unroll
-  for (int i = 0; i < 2 * RP_KC; ++i) acc[i] = (double)tacc[i];
-  // a lane ends with one value's sum over its pairs of lanes: 16 FP64 additions a thread where a
-  // reduction of each value would take 80, which at 2 FP64 operations per clock and SM cost
-  // more than the products of a small block
-  const int lane = threadIdx.x & 31;
+  for (int r = 0; r < NR; ++r) {
+    double acc[2 * RP_KC];
 #pragma unroll
-  for (int w = RP_KC; w >= 1; w >>= 1) {
-    const bool up = lane & (2 * w);  // lane bits 4, 3, 2, 1 choose the half of the values that stays
+    for (int i = 0; i < 2 * RP_KC; ++i) acc[i] = (double)tacc[r][i];
+    // a lane ends with one value's sum over its pairs of lanes: 16 FP64 additions a thread where a
+    // reduction of each value would take 80, which at 2 FP64 operations per clock and SM cost
+    // more than the products of a small block
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int i = 0; i < w; ++i) {
-      const double keep = up ? acc[i + w] : acc[i], send = up ? acc[i] : acc[i + w];
-      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * w);
+    for (int w = RP_KC; w >= 1; w >>= 1) {
+      const bool up = lane & (2 * w);  // lane bits 4, 3, 2, 1 choose the half of the values that stays
+#pragma unroll
+      for (int i = 0; i < w; ++i) {
+        const double keep = up ? acc[i + w] : acc[i], send = up ? acc[i] : acc[i + w];
+        acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * w);
+      }
     }
-  }
-  acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
-  if (!(lane & 1)) warp_sum[lane >> 1][threadIdx.x >> 5] = acc[0];
-  __syncthreads();
-  if (threadIdx.x < 2 * RP_KC) {
-    double x = 0.0;
+    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+    if (!(lane & 1)) warp_sum[lane >> 1][threadIdx.x >> 5] = acc[0];
+    __syncthreads();
+    if (threadIdx.x < 2 * RP_KC) {
+      double x = 0.0;
 #pragma unroll
-    for (int w = 0; w < RED_THREADS / 32; ++w) x += warp_sum[threadIdx.x][w];
-    part[threadIdx.x] = x;
+      for (int w = 0; w < RED_THREADS / 32; ++w) x += warp_sum[threadIdx.x][w];
+      part[r][threadIdx.x] = x;
+    }
+    __syncthreads();
   }
   cluster.sync();
-  const int i = threadIdx.x;
-  if (rank == 0 && i < 2 * RP_KC && k0 + i / 2 < nvec) {  // the CTAs' sums in their order
+  const int i = threadIdx.x % (2 * RP_KC), r = threadIdx.x / (2 * RP_KC);
+  if (rank == 0 && r < NR && r0 + r < nrhs && k0 + i / 2 < nvec) {  // the CTAs' sums in their order
     double x = 0.0;
-    for (int q = 0; q < S; ++q) x += *cluster.map_shared_rank(part + i, q);
-    reinterpret_cast<R*>(coarse + ((long long)r * bg.Vc + a) * nvec + k0)[i] = (R)x;
+    for (int q = 0; q < S; ++q) x += *cluster.map_shared_rank(&part[r][i], q);
+    reinterpret_cast<R*>(coarse + ((long long)(r0 + r) * bg.Vc + a) * nvec + k0)[i] = (R)x;
   }
   cluster.sync();  // a CTA's sums stay until they are read
 }
 
-// fine = fine_in + sum_k phi_k c[a][k]   (fine_in may be null)
-template <typename R>
+// fine = fine_in + sum_k phi_k c[a][k]   (fine_in may be null), NR fields at once
+template <typename R, int V, int NR>
 __global__ void prolong_kernel(Geom g, BlockGeom bg, const cpx<R>* __restrict__ phi,
-                               const cpx<R>* __restrict__ coarse, const cpx<R>* __restrict__ fine_in,
-                               cpx<R>* __restrict__ fine, int nvec, int nrhs) {
+                               const cpx<R>* __restrict__ coarse, const cpx<R>* fine_in,
+                               cpx<R>* fine, int nvec, int nrhs) {
   const long long fs = g.V5 * 12;
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= fs * nrhs) return;
-  const int r = (int)(idx / fs);
-  const long long e = idx - (long long)r * fs;   // element (x4*12 + c)*Ls + s
-  const int x4 = (int)(e / (12LL * g.Ls));
+  const long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * V;  // element (x4*12 + c)*Ls + s
+  if (e >= fs) return;
+  const int x4 = (int)((unsigned)e / (12u * (unsigned)g.Ls));
   int co[4];
   x4_coords(g, x4, co);
   int ac[4];
   for (int mu = 0; mu < 4; ++mu) ac[mu] = co[mu] / bg.b[mu];
   const int a = ((ac[3] * bg.Lc[2] + ac[2]) * bg.Lc[1] + ac[1]) * bg.Lc[0] + ac[0];
-  const cpx<R>* cf = coarse + ((long long)r * bg.Vc + a) * nvec;
-  cpx<R> acc((R)0, (R)0);
-  if (fine_in) acc = ld(fine_in + idx);
-  for (int k = 0; k < nvec; ++k) acc = cmadd(acc, ld(phi + (long long)k * fs + e), ld(cf + k));
-  st(fine + idx, acc);
+  const long long cs = (long long)bg.Vc * nvec;
+  for (int r0 = blockIdx.y * NR; r0 < nrhs; r0 += gridDim.y * NR) {
+    const cpx<R>* cf = coarse + r0 * cs + (long long)a * nvec;
+    Elems<R, V> acc[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+#pragma unroll
+      for (int j = 0; j < V; ++j) acc[r].x[j] = cpx<R>((R)0, (R)0);
+      if (fine_in && r0 + r < nrhs) {
+#pragma unroll
+        for (int j = 0; j < V; ++j) acc[r].x[j] = fine_in[(r0 + r) * fs + e + j];
+      }
+    }
+    for (int k = 0; k < nvec; ++k) {
+      const Elems<R, V> p = ld_elems<R, V>(phi + (long long)k * fs + e);
+#pragma unroll
+      for (int r = 0; r < NR; ++r)
+        if (NR == 1 || r0 + r < nrhs) {
+          const cpx<R> c = ld(cf + r * cs + k);
+#pragma unroll
+          for (int j = 0; j < V; ++j) acc[r].x[j] = cmadd(acc[r].x[j], p.x[j], c);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+      if (r0 + r < nrhs) {
+        cpx<R>* o = fine + (r0 + r) * fs + e;
+        if constexpr (V == 2)
+          *reinterpret_cast<float4*>(o) = make_float4(acc[r].x[0].re, acc[r].x[0].im, acc[r].x[1].re, acc[r].x[1].im);
+        else
+          st(o, acc[r].x[0]);
+      }
+  }
 }
 
 // ---------------------------------------------------------------- launchers
@@ -525,15 +587,22 @@ static int restrict_cluster(long long ctas, long long rounds) {
   return S;
 }
 
-template <typename R>
-int launch_restrict(const hdcr_subspace* sub, const cpx<R>* fine, cpx<R>* coarse, int nrhs, cudaStream_t st) {
-  const int chunks = (sub->nvec + RP_KC - 1) / RP_KC;
-  const int S = restrict_cluster((long long)sub->bg.Vc * chunks * nrhs, sub->bg.K5 * 12 / RED_THREADS);
+constexpr int RP_NR = 4;  // FP32 fields that share a pass over the basis
+
+// two FP32 elements a load: even Ls (elements of a site pair up) and 16-byte aligned fields
+static bool rp_pairs(const hdcr_subspace* sub, const void* a, const void* b) {
+  return sub->g.Ls % 2 == 0 && ((((uintptr_t)sub->vecs) | ((uintptr_t)a) | ((uintptr_t)b)) & 15) == 0;
+}
+
+template <typename R, int V, int NR>
+static int restrict_launch(const hdcr_subspace* sub, const cpx<R>* fine, cpx<R>* coarse, int nrhs, cudaStream_t st) {
+  const int chunks = (sub->nvec + RP_KC - 1) / RP_KC, groups = (nrhs + NR - 1) / NR;
+  const int S = restrict_cluster((long long)sub->bg.Vc * chunks * groups, sub->bg.K5 * 12 / V / RED_THREADS);
   // the table of the block's 4d sites in shared memory when it fits (44 KB), else
   // the sites are worked out per element
   const bool table = sub->bg.bvol <= 11 * 1024;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(sub->bg.Vc * S, chunks, nrhs);
+  cfg.gridDim = dim3(sub->bg.Vc * S, chunks, groups);
   cfg.blockDim = dim3(RED_THREADS);
   cfg.dynamicSmemBytes = table ? sizeof(int) * (size_t)sub->bg.bvol : 0;
   cfg.stream = st;
@@ -543,20 +612,49 @@ int launch_restrict(const hdcr_subspace* sub, const cpx<R>* fine, cpx<R>* coarse
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  HDCR_CUDA_TRY(cudaLaunchKernelEx(&cfg, restrict_kernel<R>, sub->g, sub->bg, (const cpx<R>*)sub->vecs, fine, coarse,
-                                   sub->nvec, table));
+  HDCR_CUDA_TRY(cudaLaunchKernelEx(&cfg, restrict_kernel<R, V, NR>, sub->g, sub->bg, (const cpx<R>*)sub->vecs, fine,
+                                   coarse, sub->nvec, nrhs, table));
   count_launch();
+  return HDCR_OK;
+}
+
+template <typename R>
+int launch_restrict(const hdcr_subspace* sub, const cpx<R>* fine, cpx<R>* coarse, int nrhs, cudaStream_t st) {
+  if constexpr (sizeof(R) == 4) {
+    const bool two = rp_pairs(sub, fine, fine);
+    if (nrhs == 1)
+      return two ? restrict_launch<R, 2, 1>(sub, fine, coarse, 1, st) : restrict_launch<R, 1, 1>(sub, fine, coarse, 1, st);
+    return two ? restrict_launch<R, 2, RP_NR>(sub, fine, coarse, nrhs, st)
+               : restrict_launch<R, 1, RP_NR>(sub, fine, coarse, nrhs, st);
+  } else {
+    return restrict_launch<R, 1, 1>(sub, fine, coarse, nrhs, st);  // bound by the FP64 pipe, not by the basis
+  }
+}
+
+template <typename R, int V, int NR>
+static int prolong_launch(const hdcr_subspace* sub, const cpx<R>* coarse, const cpx<R>* fine_in, cpx<R>* fine,
+                          int nrhs, cudaStream_t st) {
+  const int groups = (nrhs + NR - 1) / NR;
+  const dim3 grid(num_blocks(sub->g.V5 * 12 / V, 256), groups < 65535 ? groups : 65535);
+  prolong_kernel<R, V, NR><<<grid, 256, 0, st>>>(sub->g, sub->bg, (const cpx<R>*)sub->vecs, coarse, fine_in, fine,
+                                                 sub->nvec, nrhs); count_launch();
+  HDCR_LAUNCH_CHECK();
   return HDCR_OK;
 }
 
 template <typename R>
 int launch_prolong(const hdcr_subspace* sub, const cpx<R>* coarse, const cpx<R>* fine_in, cpx<R>* fine,
                    int nrhs, cudaStream_t st) {
-  const long long n = sub->g.V5 * 12 * nrhs;
-  prolong_kernel<R><<<num_blocks(n, 256), 256, 0, st>>>(sub->g, sub->bg, (const cpx<R>*)sub->vecs, coarse,
-                                                        fine_in, fine, sub->nvec, nrhs); count_launch();
-  HDCR_LAUNCH_CHECK();
-  return HDCR_OK;
+  if constexpr (sizeof(R) == 4) {
+    const bool two = rp_pairs(sub, fine_in, fine);
+    if (nrhs == 1)
+      return two ? prolong_launch<R, 2, 1>(sub, coarse, fine_in, fine, 1, st)
+                 : prolong_launch<R, 1, 1>(sub, coarse, fine_in, fine, 1, st);
+    return two ? prolong_launch<R, 2, RP_NR>(sub, coarse, fine_in, fine, nrhs, st)
+               : prolong_launch<R, 1, RP_NR>(sub, coarse, fine_in, fine, nrhs, st);
+  } else {
+    return prolong_launch<R, 1, 1>(sub, coarse, fine_in, fine, nrhs, st);
+  }
 }
 
 template <typename R>

@@ -1,5 +1,6 @@
-"""Restriction over clusters of CTAs: error against extended precision over block shapes, vector
-counts and field profiles, with the prolongation beside it."""
+"""Restriction over clusters of CTAs and several fields a pass, and the prolongation: error
+against extended precision over block shapes, vector
+counts, numbers of fields, odd and even Ls and field profiles."""
 import numpy as np
 import pytest
 
@@ -27,10 +28,10 @@ def blocks(a, L, Ls, block):
 
 
 # blocks of less than a round of a CTA's threads, not a multiple of them, and many rounds; clusters of
-# 1, 2 and 8 CTAs; vector counts around the 8 of a CTA
+# 1, 2 and 8 CTAs; vector counts around the 8 of a CTA; numbers of fields around the 4 of a pass
 CASES = [((4, 4, 4, 4), 6, (2, 2, 2, 2), 2, 1, True), ((6, 3, 9, 6), 5, (3, 1, 3, 3), 8, 2, False),
          ((8, 4, 4, 4), 16, (4, 2, 2, 2), 10, 1, True), ((8, 8, 8, 8), 8, (4, 4, 4, 4), 34, 1, False),
-         ((4, 4, 4, 4), 24, (2, 2, 2, 2), 18, 3, True)]
+         ((4, 4, 4, 4), 24, (2, 2, 2, 2), 18, 5, True), ((4, 4, 4, 4), 7, (2, 2, 2, 2), 6, 4, False)]
 
 
 @pytest.mark.parametrize("L,Ls,block,nvec,nrhs,wall", CASES)
