@@ -35,59 +35,119 @@ __global__ void add_kernel(cpx<R>* __restrict__ y, const cpx<R>* __restrict__ x,
     st(y + i, ld(y + i) + ld(x + i));
 }
 
-// w -= beta wj;  z -= beta zj   (beta complex, device)
-__global__ void axpy2_neg_kernel(cpx<double>* __restrict__ w, const cpx<double>* __restrict__ wj,
-                                 cpx<double>* __restrict__ z, const cpx<double>* __restrict__ zj, long long n,
-                                 const double* __restrict__ beta) {
-  const double br = beta[0], bi = beta[1];
+// The outer flexible GCR keeps its directions as the preconditioner left them and its images
+// w_i orthogonal but not normalised: with beta_ji = <w_j, w> / |w_j|^2 of the i-th image,
+//     H z_i = w_i + sum_j<i beta_ji w_j,   r -= a_i w_i,   a_i = <w_i, r> / |w_i|^2,
+// and at the end of a cycle x += sum_i y_i z_i with y_i + sum_k>i beta_ik y_k = a_i.  The
+// modified Gram-Schmidt steps are those of the normalised form; the z updates (as many
+// as the w updates: half of the outer iteration's FP64 work), the scaling of both and
+// the x update of every iteration are not made.  A step's update and the next one's inner
+// product share a pass: at 16^3 x 32 x 16 the vector work of an iteration with 3.5
+// earlier images took 3.5 ms of FP64 pipe and memory in seven kinds of pass.
+
+// beta <- <u, v> / n2, into the double pair ``out``
+__device__ __forceinline__ void store_ratio(double re, double im, double n2, double* out) {
+  const double s = n2 > 0.0 ? 1.0 / n2 : 0.0;
+  out[0] = re * s;
+  out[1] = im * s;
+}
+
+__global__ void __launch_bounds__(RED_THREADS) gs_dot_kernel(const cpx<double>* __restrict__ u,
+                                                             const cpx<double>* __restrict__ v, long long n,
+                                                             const double* __restrict__ n2, RedScratch rs,
+                                                             double* beta) {
+  double acc[2] = {0.0, 0.0};
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
-    const cpx<double> a = wj[i], c = zj[i];
-    cpx<double> u = w[i], v = z[i];
-    u.re = fma(-br, a.re, fma(bi, a.im, u.re));
-    u.im = fma(-br, a.im, fma(-bi, a.re, u.im));
-    v.re = fma(-br, c.re, fma(bi, c.im, v.re));
-    v.im = fma(-br, c.im, fma(-bi, c.re, v.im));
-    w[i] = u;
-    z[i] = v;
+    const cpx<double> a = ld(u + i), b = ld(v + i);
+    acc[0] = fma(a.re, b.re, fma(a.im, b.im, acc[0]));
+    acc[1] = fma(a.re, b.im, fma(-a.im, b.re, acc[1]));
+  }
+  double tot[2];
+  if (grid_reduce<2>(acc, rs, tot)) store_ratio(tot[0], tot[1], *n2, beta);
+}
+
+// w -= beta wj (wj null: w as it is), then
+//   LAST = false: beta_next <- <wn, w> / *n2n
+//   LAST = true:  *n2 <- |w|^2,  a <- <w, r> / |w|^2     (wn = r)
+template <bool LAST>
+__global__ void __launch_bounds__(RED_THREADS) gs_step_kernel(cpx<double>* __restrict__ w,
+                                                              const cpx<double>* __restrict__ wj,
+                                                              const double* __restrict__ beta,
+                                                              const cpx<double>* __restrict__ wn, long long n,
+                                                              double* n2, RedScratch rs, double* out) {
+  const double br = wj ? beta[0] : 0.0, bi = wj ? beta[1] : 0.0;
+  double acc[3] = {0.0, 0.0, 0.0};
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    cpx<double> u = w[i];
+    if (wj) {
+      const cpx<double> a = ld(wj + i);
+      u.re = fma(-br, a.re, fma(bi, a.im, u.re));
+      u.im = fma(-br, a.im, fma(-bi, a.re, u.im));
+      w[i] = u;
+    }
+    const cpx<double> q = ld(wn + i);
+    if (LAST) {  // <w, r>
+      acc[0] = fma(u.re, q.re, fma(u.im, q.im, acc[0]));
+      acc[1] = fma(u.re, q.im, fma(-u.im, q.re, acc[1]));
+      acc[2] = fma(u.re, u.re, fma(u.im, u.im, acc[2]));
+    } else {
+      acc[0] = fma(q.re, u.re, fma(q.im, u.im, acc[0]));
+      acc[1] = fma(q.re, u.im, fma(-q.im, u.re, acc[1]));
+    }
+  }
+  double tot[3];
+  if (grid_reduce<3>(acc, rs, tot)) {
+    if (LAST) *n2 = tot[2];
+    store_ratio(tot[0], tot[1], *n2, out);
   }
 }
 
-// w /= |w|, z /= |w|
-__global__ void scale2_kernel(cpx<double>* __restrict__ w, cpx<double>* __restrict__ z, long long n,
-                              const double* __restrict__ n2) {
-  const double s = *n2 > 0.0 ? 1.0 / sqrt(*n2) : 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const cpx<double> a = w[i], c = z[i];
-    w[i] = cpx<double>(a.re * s, a.im * s);
-    z[i] = cpx<double>(c.re * s, c.im * s);
-  }
-}
-
-// x += a z;  r -= a w;  |r|^2 -> *rr
-__global__ void __launch_bounds__(RED_THREADS) fgcr_update_kernel(cpx<double>* __restrict__ x,
-                                                                  const cpx<double>* __restrict__ z,
-                                                                  cpx<double>* __restrict__ r,
-                                                                  const cpx<double>* __restrict__ w, long long n,
-                                                                  const double* __restrict__ a, RedScratch rs,
-                                                                  double* rr) {
+// r -= a w;  |r|^2 -> *rr
+__global__ void __launch_bounds__(RED_THREADS) fgcr_residual_kernel(cpx<double>* __restrict__ r,
+                                                                    const cpx<double>* __restrict__ w, long long n,
+                                                                    const double* __restrict__ a, RedScratch rs,
+                                                                    double* rr) {
   const double ar = a[0], ai = a[1];
   double acc[1] = {0.0};
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
-    const cpx<double> zv = z[i], wv = w[i];
-    cpx<double> xv = x[i], rv = r[i];
-    xv.re = fma(ar, zv.re, fma(-ai, zv.im, xv.re));
-    xv.im = fma(ar, zv.im, fma(ai, zv.re, xv.im));
+    const cpx<double> wv = ld(w + i);
+    cpx<double> rv = r[i];
     rv.re = fma(-ar, wv.re, fma(ai, wv.im, rv.re));
     rv.im = fma(-ar, wv.im, fma(-ai, wv.re, rv.im));
-    x[i] = xv;
     r[i] = rv;
-    acc[0] = fma((double)rv.re, (double)rv.re, fma((double)rv.im, (double)rv.im, acc[0]));
+    acc[0] = fma(rv.re, rv.re, fma(rv.im, rv.im, acc[0]));
   }
   double tot[1];
   if (grid_reduce<1>(acc, rs, tot)) *rr = tot[0];
+}
+
+// y from a by back substitution over the first m columns; beta_ji at B[2 (i restart + j)]
+__global__ void fgcr_coef_kernel(const double* __restrict__ B, const double* __restrict__ a, double* y, int m,
+                                 int restart) {
+  for (int i = m - 1; i >= 0; --i) {
+    double re = a[2 * i], im = a[2 * i + 1];
+    for (int k = i + 1; k < m; ++k) {
+      const double br = B[2 * (k * restart + i)], bi = B[2 * (k * restart + i) + 1];
+      re -= br * y[2 * k] - bi * y[2 * k + 1];
+      im -= br * y[2 * k + 1] + bi * y[2 * k];
+    }
+    y[2 * i] = re;
+    y[2 * i + 1] = im;
+  }
+}
+
+// x += sum_i<m y_i z_i, z_i at Z + i n
+__global__ void fgcr_solution_kernel(cpx<double>* __restrict__ x, const cpx<double>* __restrict__ Z, long long n,
+                                     const double* __restrict__ y, int m) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    cpx<double> v = x[i];
+    for (int k = 0; k < m; ++k) v = cmadd(v, cpx<double>(y[2 * k], y[2 * k + 1]), ld(Z + k * n + i));
+    x[i] = v;
+  }
 }
 
 // ------------------------------------------------------------------ workspace
@@ -114,7 +174,8 @@ struct SolveCache {
   void* cw = nullptr;    // CRWork<R> of the coarse solve
   void* chw = nullptr;   // ChebWork<R> of the Chebyshev smoother
   std::vector<double> cheb_c;
-  RedBuffers rb{};       // outer reductions; scal: [0..127] MGS coefficients, 128.. scalars
+  double* B = nullptr;   // restart^2 complex beta, then restart each of complex a, complex y, |w|^2
+  RedBuffers rb{};       // outer reductions and scalars
   cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   FxCtx fx;              // encoded links and fields of the FP64 applications
   CRGraph cgraph;        // the coarse CR's iterations between host checks, replayed every V-cycle
@@ -158,7 +219,8 @@ static int alloc_cache(const hdcr_coarse* co, int restart, SolveCache** out) {
   c->fs = co->g.V5 * 12;
   c->cs = (long long)co->bg.Vc * co->nvec;
   const size_t f64 = sizeof(cpx<double>) * c->fs, fin = sizeof(cpx<R>) * c->fs, cin = sizeof(cpx<R>) * c->cs;
-  const size_t bytes = f64 * (2 * restart + 2) + fin * 5 + cin * 2 + sizeof(cpx<R>) * (size_t)co->g.V4 * 36 + 1024;
+  const size_t bytes = f64 * (2 * restart + 2) + fin * 5 + cin * 2 + sizeof(cpx<R>) * (size_t)co->g.V4 * 36 +
+                       sizeof(double) * restart * (2 * restart + 5) + 2048;
   cudaError_t e = cudaMalloc(&c->mem, bytes);
   if (e != cudaSuccess) {
     delete c;
@@ -183,6 +245,7 @@ static int alloc_cache(const hdcr_coarse* co, int restart, SolveCache** out) {
   c->c_rhs = take(cin);
   c->c_sol = take(cin);
   c->U_in = take(sizeof(cpx<R>) * (size_t)co->g.V4 * 36);
+  c->B = (double*)take(sizeof(double) * restart * (2 * restart + 5));
   int s = red_buffers_alloc(&c->rb, 192);
   CRWork<R>* sw = new CRWork<R>();
   CRWork<R>* cw = new CRWork<R>();
@@ -365,7 +428,12 @@ static int solve_impl(const hdcr_coarse* co, SolveCache* c, const void* U, const
   Hin.fx = &c->fx;
   if (prm->smoother_kind == HDCR_SMOOTHER_CHEBYSHEV)
     c->cheb_c = cheb_inverse_coeffs(prm->cheb_lo, prm->cheb_hi, prm->smoother_order);
-  double* scal = c->rb.scal;    // [0, 2*restart): MGS coefficients; 128: |w|^2; 130: a; 132: |r|^2; 133: |b|^2
+  double* scal = c->rb.scal;    // 132: |r|^2; 133: |b|^2
+  const int m = c->restart;     // columns that the workspace holds (at least prm->restart)
+  double* B = c->B;
+  double* ac = B + 2 * m * m;
+  double* yc = ac + 2 * m;
+  double* wn2 = yc + 2 * m;
   RedScratch rs = c->rb.rs;
   double* ring = pinned_ring();
   if (!ring) {
@@ -392,8 +460,8 @@ static int solve_impl(const hdcr_coarse* co, SolveCache* c, const void* U, const
   const double tol2 = prm->tol * prm->tol * bb;
   bool converged = bb == 0.0 || rr <= tol2;
   while (!converged && iters < prm->max_outer) {
-    int i = 0;
-    for (; i < prm->restart && iters < prm->max_outer; ++i) {
+    int done = 0;  // iterations of this cycle that x takes
+    for (int i = 0; i < prm->restart && iters < prm->max_outer; ++i) {
       cpx<double>* z = c->Z + (long long)i * fs;
       cpx<double>* w = c->W + (long long)i * fs;
       // z = B r
@@ -404,20 +472,22 @@ static int solve_impl(const hdcr_coarse* co, SolveCache* c, const void* U, const
         HDCR_TRY(vcycle<R>(co, Hin, c, prm, (const cpx<R>*)c->r_in, (cpx<R>*)c->z_in, &vs, st));
         HDCR_TRY(launch_convert(c->z_in, HDCR_C64, z, HDCR_C128, fs, st));
       }
-      // w = H z, orthogonalised against the earlier w_j (same coefficients on z)
+      // w = H z, orthogonalised against the earlier w_j;  r -= a w
       HDCR_TRY(H64.apply(z, w, st));
       fine64++;
-      for (int j = 0; j < i; ++j) {
-        HDCR_TRY(launch_cdot<double>(c->W + (long long)j * fs, w, fs, rs, scal + 2 * j, st));
-        axpy2_neg_kernel<<<nb, 256, 0, st>>>(w, c->W + (long long)j * fs, z, c->Z + (long long)j * fs, fs,
-                                             scal + 2 * j); count_launch();
-        HDCR_LAUNCH_CHECK();
+      const int nr = red_blocks(fs);
+      double* col = B + 2 * (size_t)i * m;
+      if (i > 0) {
+        gs_dot_kernel<<<nr, RED_THREADS, 0, st>>>(c->W, w, fs, wn2, rs, col); count_launch();
       }
-      HDCR_TRY(launch_norm2<double>(w, fs, rs, scal + 128, st));
-      scale2_kernel<<<nb, 256, 0, st>>>(w, z, fs, scal + 128); count_launch();
-      HDCR_LAUNCH_CHECK();
-      HDCR_TRY(launch_cdot<double>(w, c->r, fs, rs, scal + 130, st));
-      fgcr_update_kernel<<<red_blocks(fs), RED_THREADS, 0, st>>>(x, z, c->r, w, fs, scal + 130, rs, scal + 132); count_launch();
+      for (int j = 0; j + 1 < i; ++j) {
+        gs_step_kernel<false><<<nr, RED_THREADS, 0, st>>>(w, c->W + (long long)j * fs, col + 2 * j,
+                                                          c->W + (long long)(j + 1) * fs, fs, wn2 + j + 1, rs,
+                                                          col + 2 * (j + 1)); count_launch();
+      }
+      gs_step_kernel<true><<<nr, RED_THREADS, 0, st>>>(w, i > 0 ? c->W + (long long)(i - 1) * fs : nullptr,
+                                                       col + 2 * (i - 1), c->r, fs, wn2 + i, rs, ac + 2 * i); count_launch();
+      fgcr_residual_kernel<<<nr, RED_THREADS, 0, st>>>(c->r, w, fs, ac + 2 * i, rs, scal + 132); count_launch();
       HDCR_LAUNCH_CHECK();
       HDCR_CUDA_TRY(cudaMemcpyAsync(ring, scal + 132, sizeof(double), cudaMemcpyDeviceToHost, st));
       HDCR_CUDA_TRY(cudaStreamSynchronize(st));
@@ -432,7 +502,14 @@ static int solve_impl(const hdcr_coarse* co, SolveCache* c, const void* U, const
         status = HDCR_ERR_NONFINITE;
         break;
       }
+      done = i + 1;
       if (rr <= tol2) break;
+    }
+    // x += Z y over the cycle's iterations (the one that met a non-finite residual left out)
+    if (done > 0) {
+      fgcr_coef_kernel<<<1, 1, 0, st>>>(B, ac, yc, done, m); count_launch();
+      fgcr_solution_kernel<<<nb, 256, 0, st>>>(x, c->Z, fs, yc, done); count_launch();
+      HDCR_LAUNCH_CHECK();
     }
     if (status != HDCR_OK) break;
     // true residual (restart or convergence check)

@@ -79,63 +79,124 @@ __global__ void __launch_bounds__(MB_THREADS) mdot_final_kernel(const double2* _
   }
 }
 
-// w_r -= beta_r wj_r;  z_r -= beta_r zj_r   (beta_r = sc[r * ss], complex)
-__global__ void maxpy2_neg_kernel(cpx<double>* __restrict__ w, const cpx<double>* __restrict__ wj,
-                                  cpx<double>* __restrict__ z, const cpx<double>* __restrict__ zj, long long n,
-                                  const double* __restrict__ sc, int ss) {
+// The outer iteration of the single solve (unnormalised images, directions as they are, the
+// solution at the end of a cycle: hdcr.cu), for every right-hand side r: its scalars are at
+// sc + r ss.
+//
+// w_r -= beta_r wj_r (wj null: w as it is), then partial sums of
+//   LAST = false: <wn_r, w_r> into part
+//   LAST = true:  <w_r, wn_r> into part and |w_r|^2 into part2
+template <bool LAST>
+__global__ void __launch_bounds__(MB_THREADS) mgs_step_kernel(cpx<double>* __restrict__ w,
+                                                              const cpx<double>* __restrict__ wj,
+                                                              const double* __restrict__ beta, int ss,
+                                                              const cpx<double>* __restrict__ wn, long long n,
+                                                              double2* __restrict__ part, double2* __restrict__ part2) {
   const long long off = (long long)blockIdx.y * n;
-  const double br = sc[blockIdx.y * ss], bi = sc[blockIdx.y * ss + 1];
+  const double br = wj ? beta[blockIdx.y * ss] : 0.0, bi = wj ? beta[blockIdx.y * ss + 1] : 0.0;
+  double a = 0.0, b = 0.0, n2 = 0.0, zero = 0.0;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
-    const cpx<double> a = wj[off + i], c = zj[off + i];
-    cpx<double> u = w[off + i], v = z[off + i];
-    u.re = fma(-br, a.re, fma(bi, a.im, u.re));
-    u.im = fma(-br, a.im, fma(-bi, a.re, u.im));
-    v.re = fma(-br, c.re, fma(bi, c.im, v.re));
-    v.im = fma(-br, c.im, fma(-bi, c.re, v.im));
-    w[off + i] = u;
-    z[off + i] = v;
+    cpx<double> u = w[off + i];
+    if (wj) {
+      const cpx<double> c = wj[off + i];
+      u.re = fma(-br, c.re, fma(bi, c.im, u.re));
+      u.im = fma(-br, c.im, fma(-bi, c.re, u.im));
+      w[off + i] = u;
+    }
+    const cpx<double> q = wn[off + i];
+    if (LAST) {
+      a = fma(u.re, q.re, fma(u.im, q.im, a));
+      b = fma(u.re, q.im, fma(-u.im, q.re, b));
+      n2 = fma(u.re, u.re, fma(u.im, u.im, n2));
+    } else {
+      a = fma(q.re, u.re, fma(q.im, u.im, a));
+      b = fma(q.re, u.im, fma(-q.im, u.re, b));
+    }
+  }
+  block_sum2(a, b);
+  if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = make_double2(a, b);
+  if (LAST) {
+    __syncthreads();
+    block_sum2(n2, zero);
+    if (threadIdx.x == 0) part2[blockIdx.y * gridDim.x + blockIdx.x] = make_double2(n2, 0.0);
   }
 }
 
-// w_r /= |w_r|, z_r /= |w_r|   (|w_r|^2 = sc[r * ss])
-__global__ void mscale2_kernel(cpx<double>* __restrict__ w, cpx<double>* __restrict__ z, long long n,
-                               const double* __restrict__ sc, int ss) {
-  const long long off = (long long)blockIdx.y * n;
-  const double n2 = sc[blockIdx.y * ss];
-  const double s = n2 > 0.0 ? 1.0 / sqrt(n2) : 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const cpx<double> a = w[off + i], c = z[off + i];
-    w[off + i] = cpx<double>(a.re * s, a.im * s);
-    z[off + i] = cpx<double>(c.re * s, c.im * s);
+// out_r <- (sum of part) / |.|^2 with |.|^2 at n2_r, summed from part2 first when that is set (grid: nrhs)
+__global__ void __launch_bounds__(MB_THREADS) mgs_final_kernel(const double2* __restrict__ part,
+                                                               const double2* __restrict__ part2, int nblk,
+                                                               double* n2, double* out, int ss) {
+  double a = 0.0, b = 0.0, c = 0.0, zero = 0.0;
+  for (int t = threadIdx.x; t < nblk; t += blockDim.x) {
+    const double2 p = part[blockIdx.x * nblk + t];
+    a += p.x;
+    b += p.y;
+    if (part2) c += part2[blockIdx.x * nblk + t].x;
+  }
+  block_sum2(a, b);
+  if (part2) {
+    __syncthreads();
+    block_sum2(c, zero);
+  }
+  if (threadIdx.x == 0) {
+    double* q = n2 + (long long)blockIdx.x * ss;
+    if (part2) *q = c;
+    const double s = *q > 0.0 ? 1.0 / *q : 0.0;
+    out[(long long)blockIdx.x * ss] = a * s;
+    out[(long long)blockIdx.x * ss + 1] = b * s;
   }
 }
 
-// x_r += a_r z_r;  r_r -= a_r w_r;  partial |r_r|^2 into part (a_r = sc[r * ss])
-__global__ void __launch_bounds__(MB_THREADS) mfgcr_update_kernel(cpx<double>* __restrict__ x,
-                                                                  const cpx<double>* __restrict__ z,
-                                                                  cpx<double>* __restrict__ r,
-                                                                  const cpx<double>* __restrict__ w, long long n,
-                                                                  const double* __restrict__ sc, int ss,
-                                                                  double2* __restrict__ part) {
+// r_r -= a_r w_r;  partial |r_r|^2 into part
+__global__ void __launch_bounds__(MB_THREADS) mfgcr_residual_kernel(cpx<double>* __restrict__ r,
+                                                                    const cpx<double>* __restrict__ w, long long n,
+                                                                    const double* __restrict__ sc, int ss,
+                                                                    double2* __restrict__ part) {
   const long long off = (long long)blockIdx.y * n;
   const double ar = sc[blockIdx.y * ss], ai = sc[blockIdx.y * ss + 1];
   double acc = 0.0, zero = 0.0;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
-    const cpx<double> zv = z[off + i], wv = w[off + i];
-    cpx<double> xv = x[off + i], rv = r[off + i];
-    xv.re = fma(ar, zv.re, fma(-ai, zv.im, xv.re));
-    xv.im = fma(ar, zv.im, fma(ai, zv.re, xv.im));
+    const cpx<double> wv = w[off + i];
+    cpx<double> rv = r[off + i];
     rv.re = fma(-ar, wv.re, fma(ai, wv.im, rv.re));
     rv.im = fma(-ar, wv.im, fma(-ai, wv.re, rv.im));
-    x[off + i] = xv;
     r[off + i] = rv;
-    acc = fma((double)rv.re, (double)rv.re, fma((double)rv.im, (double)rv.im, acc));
+    acc = fma(rv.re, rv.re, fma(rv.im, rv.im, acc));
   }
   block_sum2(acc, zero);
   if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = make_double2(acc, 0.0);
+}
+
+// y_r from a_r and beta_r over the first m columns (grid: nrhs)
+__global__ void mfgcr_coef_kernel(double* sc, int ss, int restart, int m) {
+  const double* B = sc + (long long)blockIdx.x * ss;
+  const double* a = B + 2 * restart * restart;
+  double* y = sc + (long long)blockIdx.x * ss + 2 * restart * restart + 2 * restart;
+  for (int i = m - 1; i >= 0; --i) {
+    double re = a[2 * i], im = a[2 * i + 1];
+    for (int k = i + 1; k < m; ++k) {
+      const double br = B[2 * (k * restart + i)], bi = B[2 * (k * restart + i) + 1];
+      re -= br * y[2 * k] - bi * y[2 * k + 1];
+      im -= br * y[2 * k + 1] + bi * y[2 * k];
+    }
+    y[2 * i] = re;
+    y[2 * i + 1] = im;
+  }
+}
+
+// x_r += sum_i<m y_ri z_ri, z_ri at Z + i N + r n
+__global__ void mfgcr_solution_kernel(cpx<double>* __restrict__ x, const cpx<double>* __restrict__ Z, long long n,
+                                      long long N, const double* __restrict__ y, int ss, int m) {
+  const long long off = (long long)blockIdx.y * n;
+  const double* yr = y + (long long)blockIdx.y * ss;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    cpx<double> v = x[off + i];
+    for (int k = 0; k < m; ++k) v = cmadd(v, cpx<double>(yr[2 * k], yr[2 * k + 1]), Z[k * N + off + i]);
+    x[off + i] = v;
+  }
 }
 
 template <typename R>
@@ -166,7 +227,7 @@ struct MultiCache {
   void* chw = nullptr;                                                                // ChebWork<R> over nrhs
   FxCtx fx;                 // encoded links and fields of the FP64 applications
   double* sc = nullptr;     // nrhs x SC device scalars
-  double2* part = nullptr;  // nrhs x MB_BLOCKS partial sums
+  double2* part = nullptr;  // 2 x nrhs x MB_BLOCKS partial sums
   double* rr = nullptr;     // nrhs x 2: |r_r|^2 (stride 2)
   double* bb = nullptr;     // nrhs x 2: |b_r|^2
   double* host = nullptr;   // pinned, 2 * nrhs
@@ -214,11 +275,11 @@ static int multi_alloc(const hdcr_coarse* co, int nrhs, int restart, MultiCache*
   c->fs = co->g.V5 * 12;
   c->N = c->fs * nrhs;
   c->cs = (long long)co->bg.Vc * co->nvec;
-  c->SC = 2 * restart + 8;
+  c->SC = 2 * restart * restart + 5 * restart;  // beta, a, y, |w|^2
   const size_t f64 = sizeof(cpx<double>) * (size_t)c->N, fin = sizeof(cpx<R>) * (size_t)c->N;
   const size_t cin = sizeof(cpx<R>) * (size_t)(c->cs * nrhs);
   const size_t bytes = f64 * (2 * (size_t)restart + 2) + fin * 5 + cin * 2 + sizeof(cpx<R>) * (size_t)co->g.V4 * 36 +
-                       sizeof(double) * (size_t)(nrhs * c->SC + 4 * nrhs) + sizeof(double2) * nrhs * MB_BLOCKS +
+                       sizeof(double) * (size_t)(nrhs * c->SC + 4 * nrhs) + 2 * sizeof(double2) * nrhs * MB_BLOCKS +
                        16 * 256;
   cudaError_t e = cudaMalloc(&c->mem, bytes);
   if (e != cudaSuccess) {
@@ -247,7 +308,7 @@ static int multi_alloc(const hdcr_coarse* co, int nrhs, int restart, MultiCache*
   c->sc = (double*)take(sizeof(double) * (size_t)nrhs * c->SC);
   c->rr = (double*)take(sizeof(double) * 2 * nrhs);
   c->bb = (double*)take(sizeof(double) * 2 * nrhs);
-  c->part = (double2*)take(sizeof(double2) * nrhs * MB_BLOCKS);
+  c->part = (double2*)take(2 * sizeof(double2) * nrhs * MB_BLOCKS);
   int s = HDCR_OK;
   if (cudaMallocHost(&c->host, sizeof(double) * 2 * nrhs) != cudaSuccess) s = HDCR_ERR_NO_MEMORY;
   ChebWork<R>* chw = new ChebWork<R>();
@@ -376,7 +437,7 @@ static int solve_multi_impl(const hdcr_coarse* co, MultiCache* c, const void* U,
   c->cheb_c = cheb_inverse_coeffs(prm->cheb_lo, prm->cheb_hi, prm->smoother_order);
   double* sc = c->sc;
   const int SC = c->SC;
-  const int I_N2 = 2 * c->restart, I_A = 2 * c->restart + 2;
+  const int I_A = 2 * c->restart * c->restart, I_Y = I_A + 2 * c->restart, I_N2 = I_Y + 2 * c->restart;
   // r = b - H x, |b_r|^2, |r_r|^2
   HDCR_TRY(H64.apply(x, c->tmp, st));
   msub_kernel<double><<<nb, 256, 0, st>>>(b, c->tmp, c->r, N);
@@ -408,8 +469,8 @@ static int solve_multi_impl(const hdcr_coarse* co, MultiCache* c, const void* U,
   bool have_graph = graph_ok;
   int fine64 = 1, fine_in = 0, iters = 0, restarts = 0, status = HDCR_OK;
   while (!converged && iters < prm->max_outer) {
-    int i = 0;
-    for (; i < prm->restart && iters < prm->max_outer; ++i) {
+    int done = 0;  // iterations of this cycle that x takes
+    for (int i = 0; i < prm->restart && iters < prm->max_outer; ++i) {
       cpx<double>* z = c->Z + (long long)i * N;
       cpx<double>* w = c->W + (long long)i * N;
       // z = B r (the first V-cycle of a solve runs eagerly, which also tunes the stencil tiles)
@@ -436,21 +497,27 @@ static int solve_multi_impl(const hdcr_coarse* co, MultiCache* c, const void* U,
       } else {
         HDCR_TRY(launch_convert(c->z_in, HDCR_C64, z, HDCR_C128, N, st));
       }
-      // w = H z, orthogonalised against the earlier w_j (same coefficients on z), per right-hand side
+      // w = H z, orthogonalised against the earlier w_j;  r -= a w, per right-hand side
       HDCR_TRY(H64.apply(z, w, st));
       fine64++;
-      for (int j = 0; j < i; ++j) {
-        mdot(c->W + (long long)j * N, w, fs, nrhs, c->part, sc + 2 * j, SC, st);
-        maxpy2_neg_kernel<<<gb, 256, 0, st>>>(w, c->W + (long long)j * N, z, c->Z + (long long)j * N, fs, sc + 2 * j,
-                                              SC);
+      const dim3 grid(MB_BLOCKS, nrhs);
+      double2* part2 = c->part + (size_t)nrhs * MB_BLOCKS;
+      double* col = sc + 2 * (size_t)i * c->restart;
+      auto final = [&](double2* p2, double* n2, double* out) {
+        mgs_final_kernel<<<nrhs, MB_THREADS, 0, st>>>(c->part, p2, MB_BLOCKS, n2, out, SC);
         count_launch();
-        HDCR_LAUNCH_CHECK();
+      };
+      for (int j = -1; j + 1 < i; ++j) {  // (the first only takes <w_0, w>)
+        mgs_step_kernel<false><<<grid, MB_THREADS, 0, st>>>(w, j < 0 ? nullptr : c->W + (long long)j * N, col + 2 * j, SC,
+                                                            c->W + (long long)(j + 1) * N, fs, c->part, nullptr);
+        count_launch();
+        final(nullptr, sc + I_N2 + j + 1, col + 2 * (j + 1));
       }
-      mdot(w, w, fs, nrhs, c->part, sc + I_N2, SC, st);
-      mscale2_kernel<<<gb, 256, 0, st>>>(w, z, fs, sc + I_N2, SC);
+      mgs_step_kernel<true><<<grid, MB_THREADS, 0, st>>>(w, i > 0 ? c->W + (long long)(i - 1) * N : nullptr,
+                                                         col + 2 * (i - 1), SC, c->r, fs, c->part, part2);
       count_launch();
-      mdot(w, c->r, fs, nrhs, c->part, sc + I_A, SC, st);
-      mfgcr_update_kernel<<<dim3(MB_BLOCKS, nrhs), MB_THREADS, 0, st>>>(x, z, c->r, w, fs, sc + I_A, SC, c->part);
+      final(part2, sc + I_N2 + i, sc + I_A + 2 * i);
+      mfgcr_residual_kernel<<<grid, MB_THREADS, 0, st>>>(c->r, w, fs, sc + I_A + 2 * i, SC, c->part);
       count_launch();
       mdot_final_kernel<<<nrhs, MB_THREADS, 0, st>>>(c->part, MB_BLOCKS, c->rr, 2);
       count_launch();
@@ -467,7 +534,16 @@ static int solve_multi_impl(const hdcr_coarse* co, MultiCache* c, const void* U,
         }
         if (rr[q] > tol2[q]) all = false;
       }
+      if (status == HDCR_OK) done = i + 1;
       if (status != HDCR_OK || all) break;
+    }
+    // x += Z y over the cycle's iterations (one that met a non-finite residual left out)
+    if (done > 0) {
+      mfgcr_coef_kernel<<<nrhs, 1, 0, st>>>(sc, SC, c->restart, done);
+      count_launch();
+      mfgcr_solution_kernel<<<gb, 256, 0, st>>>(x, c->Z, fs, N, sc + I_Y, SC, done);
+      count_launch();
+      HDCR_LAUNCH_CHECK();
     }
     if (status != HDCR_OK) break;
     // true residuals (restart or convergence check)
