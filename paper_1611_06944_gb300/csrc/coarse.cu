@@ -581,7 +581,7 @@ __global__ void prolong_kernel(Geom g, BlockGeom bg, const cpx<R>* __restrict__ 
 // CTAs that share a block's restriction as a cluster: more while there are fewer than four per
 // SM and each still has four rounds of its threads.  With 2^3 x 4 coarse sites (8^3 x 16, 16
 // vectors, FP32) a block per CTA left most of the chip idle: 129 us a launch.
-static int restrict_cluster(long long ctas, long long rounds) {
+int restrict_cluster(long long ctas, long long rounds) {
   int S = 1;
   while (S < 8 && ctas * S < 4 * 152 && rounds >= 8 * S) S *= 2;
   return S;
@@ -627,6 +627,7 @@ int launch_restrict(const hdcr_subspace* sub, const cpx<R>* fine, cpx<R>* coarse
     return two ? restrict_launch<R, 2, RP_NR>(sub, fine, coarse, nrhs, st)
                : restrict_launch<R, 1, RP_NR>(sub, fine, coarse, nrhs, st);
   } else {
+    if (sub->fx && nrhs <= 65535) return launch_restrict_fx(sub, fine, coarse, nrhs, st);
     return restrict_launch<R, 1, 1>(sub, fine, coarse, nrhs, st);  // bound by the FP64 pipe, not by the basis
   }
 }
@@ -653,6 +654,7 @@ int launch_prolong(const hdcr_subspace* sub, const cpx<R>* coarse, const cpx<R>*
     return two ? prolong_launch<R, 2, RP_NR>(sub, coarse, fine_in, fine, nrhs, st)
                : prolong_launch<R, 1, RP_NR>(sub, coarse, fine_in, fine, nrhs, st);
   } else {
+    if (sub->fx && nrhs <= 65535) return launch_prolong_fx(sub, coarse, fine_in, fine, nrhs, st);
     return prolong_launch<R, 1, 1>(sub, coarse, fine_in, fine, nrhs, st);
   }
 }

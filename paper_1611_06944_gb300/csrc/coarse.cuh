@@ -62,6 +62,10 @@ struct hdcr_subspace {
   int dtype;      // storage of the basis vectors (HDCR_C128 / HDCR_C64)
   void* vecs;     // nvec fields, plane layout, block-orthonormal
   int device;
+  // FP64 basis in fixed point for the restriction and prolongation (transfer_fx.cu), made with the
+  // subspace where it takes at most a quarter of the free device memory; else null, and
+  // they run on the FP64 pipe
+  void* fx = nullptr;
   // scratch of hdcr_build_coarse_op, kept for the next build from this basis (a
   // rebuild after a gauge update needs no allocation); builds from one subspace
   // are serialised on build_mu
@@ -102,6 +106,13 @@ int launch_restrict(const hdcr_subspace* sub, const cpx<R>* fine, cpx<R>* coarse
 template <typename R>
 int launch_prolong(const hdcr_subspace* sub, const cpx<R>* coarse, const cpx<R>* fine_in, cpx<R>* fine,
                    int nrhs, cudaStream_t st);
+// the same in FP64 from the fixed-point basis sub->fx; subspace_encode makes it
+int subspace_encode(hdcr_subspace* sub, cudaStream_t st);
+int launch_restrict_fx(const hdcr_subspace* sub, const cpx<double>* fine, cpx<double>* coarse, int nrhs,
+                       cudaStream_t st);
+int launch_prolong_fx(const hdcr_subspace* sub, const cpx<double>* coarse, const cpx<double>* fine_in,
+                      cpx<double>* fine, int nrhs, cudaStream_t st);
+int restrict_cluster(long long ctas, long long rounds);
 template <typename R>
 int launch_coarse_apply(const hdcr_coarse* co, const cpx<R>* in, cpx<R>* out, int nrhs, cudaStream_t st);
 // nbr[a][leg]: the coarse site each leg of site a reaches (device array of Vc * 9 ints)

@@ -463,6 +463,11 @@ static int orthonormalise_and_store(const Geom& g, const BlockGeom& bg, cpx<doub
   const long long n = (long long)nvec * g.V5 * 12;
   if (store_dtype == HDCR_C128) {
     sub->vecs = vecs;  // keep the FP64 buffer
+    const int s = subspace_encode(sub, st);
+    if (s != HDCR_OK) {
+      hdcr_subspace_destroy(sub);
+      return s;
+    }
   } else {
     void* p = nullptr;
     e = cudaMalloc(&p, n * sizeof(cpx<float>));
@@ -696,6 +701,7 @@ extern "C" int hdcr_subspace_get_vectors(const hdcr_subspace* sub, void* out, vo
 extern "C" void hdcr_subspace_destroy(hdcr_subspace* sub) {
   if (!sub) return;
   if (sub->vecs) cudaFree(sub->vecs);
+  if (sub->fx) cudaFree(sub->fx);
   if (sub->build_ws) cudaFree(sub->build_ws);
   delete sub;
 }

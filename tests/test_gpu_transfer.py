@@ -1,6 +1,6 @@
-"""Restriction over clusters of CTAs and several fields a pass, and the prolongation: error
+"""Restriction and prolongation (FP64 in fixed point, FP32 with several fields a pass): error
 against extended precision over block shapes, vector
-counts, numbers of fields, odd and even Ls and field profiles."""
+counts, numbers of fields, odd and even Ls and field profiles, and FP64 values outside the format."""
 import numpy as np
 import pytest
 
@@ -57,9 +57,39 @@ def test_transfer_error(hd, L, Ls, block, nvec, nrhs, wall, dtype):
     def rel(a, b):
         return float(np.sqrt((np.abs(a - b) ** 2).sum() / (np.abs(b) ** 2).sum()))
 
-    # sums of up to 400 products a thread, u sqrt(n) each with u = 1.1e-16 (6e-8), over terms that
-    # partly cancel
-    bound = 4e-15 if dtype == "c128" else 2e-6
+    # FP64: sites summed exactly and rounded to u = 1.1e-16, a few tens of them a thread added in FP64,
+    # over sums that cancel to 1 / sqrt(n) of their terms; FP32: up to 400 products a thread
+    bound = 4e-16 if dtype == "c128" else 2e-6
     assert rel(got, want) <= bound
     wf = np.stack([(phi * x.T[:, :, None]).sum(0) for x in got])
     assert rel(blocks(host(f), L, Ls, block), wf) <= bound
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), 1e250, 1e-250, 0.0])
+def test_values_outside_the_format(hd, value):
+    L, Ls, block = (4, 4, 2, 2), 4, (2, 2, 1, 1)
+    lat = hd.Lattice(L, Ls)
+    vec = dev(planes(synth.gaussian_fermion(L, Ls, 6100, count=6)))
+    sub = hd.subspace_from_vectors(lat, block, vec)
+    phi = host(sub.vectors())
+    pb = blocks(phi, L, Ls, block)
+    v = host(dev(planes(synth.gaussian_fermion(L, Ls, 6101, count=1)))).copy()
+    v[0, 5, 3, 1] = value
+    with np.errstate(all="ignore"):
+        want = (np.conj(pb) * blocks(v, L, Ls, block)[0]).sum(-1).T
+    got = host(hd.restrict(sub, dev(v)))[0]
+    fin = np.isfinite(want.real) & np.isfinite(want.imag)
+    gfin = np.isfinite(got.real) & np.isfinite(got.imag)
+    assert np.array_equal(fin, gfin)
+    scale = np.abs(want[fin]).max()
+    assert np.abs(got[fin] - want[fin]).max() <= 1e-14 * scale
+    c = host(hd.restrict(sub, dev(planes(synth.gaussian_fermion(L, Ls, 6102, count=1))))).copy()
+    c[0, 1, 2] = value
+    with np.errstate(all="ignore"):
+        wf = (pb * c[0].T[:, :, None]).sum(0)
+    gf = blocks(host(hd.prolong(sub, dev(c))), L, Ls, block)[0]
+    fin = np.isfinite(wf.real) & np.isfinite(wf.imag)
+    assert np.array_equal(fin, np.isfinite(gf.real) & np.isfinite(gf.imag))
+    if fin.any():
+        other = np.delete(np.arange(wf.shape[0]), 1)
+        assert np.abs(gf[other] - wf[other]).max() <= 1e-14 * np.abs(wf[other]).max()
