@@ -264,6 +264,11 @@ int cheb_filter(const FineOp<R>& H, cpx<R>* x, int order, double lam_cut, double
   return HDCR_OK;
 }
 
+// Steps between rescalings of the filter's recurrence, which keep it in range: a mode at t = cosh(u) grows
+// by e^u a step, and FP32 holds e^16u up to t = 100, 7 times lam_max.  Every 8 steps the
+// norm and the scaling of both terms took 4% of a filter of order 200 (12 fields at 8^3 x 16 x 8).
+constexpr int FILTER_RESCALE = 16;
+
 template <typename R>
 int cheb_filter_multi(const FineOp<R>& H, cpx<R>* x, int nrhs, int order, double lam_cut, double lam_max,
                       cpx<R>* work, double* n2, RedScratch rs, cudaStream_t st) {
@@ -278,10 +283,35 @@ int cheb_filter_multi(const FineOp<R>& H, cpx<R>* x, int nrhs, int order, double
   bool fused = false;
   if constexpr (sizeof(R) == 4) fused = g5dwf_x2_ok(H.g, x, work) && g5dwf_x2_ok(H.g, work + N, work + 2 * N);
   const void* U = H.U;
+  bool fixed = false;  // FP64 in fixed point: terms pass between the applications encoded
+  if constexpr (sizeof(R) == 8) fixed = H.fixed();
+  auto fx_step = [&](const cpx<R>* cur, cpx<R>* prev, bool first) -> int {
+    if constexpr (sizeof(R) == 8) {
+      const FxCtx& fx = *H.fx;  // cur is encoded in e0, the new term will be
+      FxChebStep step{};
+      step.cur = cur;
+      step.prev = prev;
+      step.a = a;
+      step.b = b;
+      step.first = first;
+      HDCR_TRY(launch_fx_g5dwf(H.g, H.M5, H.mf, fx.u, fx.e0, nullptr, nrhs, st, &fx.e1));
+      return launch_fx_g5dwf_cheb(H.g, H.M5, H.mf, fx.u, fx.e1, step, fx.e0, nrhs, st);
+    }
+    return HDCR_OK;
+  };
+  auto fx_encode = [&](const cpx<R>* v) -> int {
+    if constexpr (sizeof(R) == 8) return launch_fx_encode(H.g, v, nrhs, H.fx->e0, nullptr, H.fx->u, st);
+    return HDCR_OK;
+  };
   // T_0 = x, T_1 = a H^2 x + b x
   rescale_copy(x, t0, N, (R)1, st);
-  HDCR_TRY(launch_g5dwf<R>(H.g, H.M5, H.mf, U, t0, h1, nrhs, st));
-  if (fused) {
+  if (fixed)
+    HDCR_TRY(fx_encode(t0));
+  else
+    HDCR_TRY(launch_g5dwf<R>(H.g, H.M5, H.mf, U, t0, h1, nrhs, st));
+  if (fixed) {
+    HDCR_TRY(fx_step(t0, t1, true));
+  } else if (fused) {
     HDCR_CUDA_TRY(cudaMemsetAsync(t1, 0, sizeof(cpx<R>) * N, st));
     HDCR_TRY(launch_g5dwf_x2_cheb(H.g, H.M5, H.mf, (const cpx<float>*)U, (const cpx<float>*)h1,
                                   (const cpx<float>*)t0, (cpx<float>*)t1, (float)(0.5 * a), (float)(0.5 * b), nrhs,
@@ -295,8 +325,10 @@ int cheb_filter_multi(const FineOp<R>& H, cpx<R>* x, int nrhs, int order, double
   cpx<R>* cur = t1;
   for (int k = 2; k <= order; ++k) {
     // T_k = 2 t(H^2) T_{k-1} - T_{k-2}, written over T_{k-2}
-    HDCR_TRY(launch_g5dwf<R>(H.g, H.M5, H.mf, U, cur, h1, nrhs, st));
-    if (fused) {
+    if (!fixed) HDCR_TRY(launch_g5dwf<R>(H.g, H.M5, H.mf, U, cur, h1, nrhs, st));
+    if (fixed) {
+      HDCR_TRY(fx_step(cur, prev, false));
+    } else if (fused) {
       HDCR_TRY(launch_g5dwf_x2_cheb(H.g, H.M5, H.mf, (const cpx<float>*)U, (const cpx<float>*)h1,
                                     (const cpx<float>*)cur, (cpx<float>*)prev, (float)a, (float)b, nrhs, st));
     } else {
@@ -307,10 +339,11 @@ int cheb_filter_multi(const FineOp<R>& H, cpx<R>* x, int nrhs, int order, double
     cpx<R>* t = prev;
     prev = cur;
     cur = t;
-    if (k % 8 == 0) {  // keep the growing recurrence in range: one common rescale of both terms
+    if (k % FILTER_RESCALE == 0 && k < order) {  // one common rescale of both terms
       HDCR_TRY(launch_norm2<R>(cur, N, rs, n2, st));
       rescale2_kernel<R><<<nb, 256, 0, st>>>(cur, prev, N, n2); count_launch();
       HDCR_LAUNCH_CHECK();
+      if (fixed) HDCR_TRY(fx_encode(cur));
     }
   }
   HDCR_TRY(launch_norm2<R>(cur, N, rs, n2, st));

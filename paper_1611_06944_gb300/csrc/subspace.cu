@@ -530,6 +530,10 @@ static int filter_all_cheb(const Geom& g, const hdcr_dwf_params* p, const void* 
   RedBuffers rb{{nullptr, nullptr}, nullptr, 0, nullptr};
   int s = red_buffers_alloc(&rb, 2);
   FineOp<R> H{g, p->M5, p->mf, Ur};
+  FxCtx fx;
+  if (f64) fx_ctx_alloc(&fx, g, half);
+  H.fx = &fx;
+  if (s == HDCR_OK) s = fx_ctx_links(fx, g, (const cpx<double>*)U, st);
   if (s == HDCR_OK) s = launch_convert(noise, HDCR_C128, x, f64 ? HDCR_C128 : HDCR_C64, fs * half, st);
   if (s == HDCR_OK) s = cheb_filter_multi<R>(H, x, half, sp->order, sp->lam_cut, sp->lam_max, work, rb.scal, rb.rs, st);
   for (int i = 0; i < half && s == HDCR_OK; ++i) {
@@ -544,6 +548,7 @@ static int filter_all_cheb(const Geom& g, const hdcr_dwf_params* p, const void* 
   }
   cudaStreamSynchronize(st);
   red_buffers_free(&rb);
+  fx_ctx_free(&fx);
   cudaFree(mem);
   return s;
 }

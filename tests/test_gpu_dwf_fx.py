@@ -175,3 +175,20 @@ def test_red_black_shapes(hd, L, Ls, bc):
     r = b - dwf.apply_H(U, natural(host(x), L, Ls), 1.8, mf, bc)
     # the Schur residual stops at 1e-10; the reconstruction adds rounding times the condition number
     assert np.linalg.norm(r) <= 2e-10 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("order", [1, 2, 16, 17, 40])
+def test_fp64_filter_matches_the_oracle(hd, order):
+    """The FP64 Chebyshev filter's encoded steps around its rescalings, three fields at once, on a
+    basis that one orthonormalisation of the oracle's filtered vectors must reproduce."""
+    L, Ls, block, mf = (4, 4, 2, 4), 5, (2, 2, 1, 2), 0.05
+    U = synth.gauge_field(L, 0.4, 5500)
+    noise = synth.gaussian_fermion(L, Ls, 5501, count=3)
+    sub = hd.build_subspace(hd.Lattice(L, Ls), dev(links(U)), dev(planes(noise)), 1.8, mf, block, order=order,
+                            lam_cut=0.5)
+    g = mg.Geometry(L, Ls, block)
+    f = np.stack([mg.chebyshev_filter(U, n, 1.8, mf, 1, 0.5, 8.0, order) for n in noise])
+    phi = mg.block_orthonormalise(mg.to_blocks(g, mg.chiral_split(f)))
+    want = np.stack([mg.from_blocks(g, v) for v in phi])
+    # order x 1e-16 of rounding a step times the blocks' condition number
+    assert relerr(natural(host(sub.vectors()), L, Ls), want) <= 1e-10
