@@ -73,12 +73,6 @@ SOLVE = dict(tol=1e-10, restart=24, smoother="chebyshev", smoother_order=10, che
 # fifth-dimension hops P_-psi(s+1), P_+psi(s-1) (12 complex subtractions, 24): 1416.
 # Gamma5 and the R5 reflection are signs and a permutation (free).
 FLOPS_PER_SITE = 1320 + 4 * 24
-# FP64 instructions per 5d site the FP64 kernel issues (each one slot of the FP64
-# pipe whether add, multiply or FMA): per hop 12 projection adds, 72 for the
-# SU(3) x half-spinor (4 per complex multiply(-add)), 24 FMAs accumulating the upper
-# and the Gamma5-signed lower spins with the boundary factor; plus 24 multiplies
-# (diagonal) and 24 FMAs (fifth dimension).
-FP64_INSTR_PER_SITE = 8 * (12 + 72 + 24) + 48
 
 
 # algorithmic bytes per 5d site of one application (read psi, write H psi, links / Ls)
@@ -88,12 +82,13 @@ def bytes_per_site(real_bytes: int, Ls: int) -> float:
 
 # DRAM traffic of one FP64 / FP32 / FP16-storage stencil launch at 16^4 x 16 from ncu, with the hash of
 # the stencil sources it was measured on (reported as null once the sources change)
-NCU_TRAFFIC = {"f64": 449.67e6, "f32": 202.18e6, "h16": 106.18e6, "src_hash": "272691dffa098572"}
+NCU_TRAFFIC = {"f64": 539.33e6, "f32": 202.18e6, "h16": 106.18e6, "src_hash": "28101ddd10c136a5"}
 
 
 def stencil_src_hash() -> str:
     h = hashlib.sha256()
-    for f in ("dwf_stencil.cuh", "dwf.cu", "dwf_x2.cu", "dwf_x2.cuh", "dwf_h16.cu", "hdcr_internal.cuh"):
+    for f in ("dwf_stencil.cuh", "dwf.cu", "dwf_fx.cu", "dwf_fx.cuh", "fx_device.cuh", "dwf_x2.cu", "dwf_x2.cuh", "dwf_h16.cu",
+              "hdcr_internal.cuh"):
         with open(os.path.join(ROOT, "paper_1611_06944_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -350,22 +345,24 @@ def run_ours(args, world, rank, local):
     ms64c = st64c["ms"] / max(st64c["launches"], 1)
     share64c = ms64c * st64c["all_launches"] / (elapsed * 1e3)
     fp64_peak = hd.probe_fma_rate(torch.complex128)            # measured on this GPU, this run
-    pipe = FP64_INSTR_PER_SITE * sites64 / (ms64 * 1e-3) / (fp64_peak * 1e12 / 2)
-    roofline = {"bound": "alu", "kernel": "g5dwf FP64 (H = Gamma5 D_dwf)", "achieved": round(achieved, 4),
-                "peak": round(fp64_peak, 4), "unit": "TFLOP/s", "frac": round(achieved / fp64_peak, 4),
-                "traffic": NCU_TRAFFIC["f64"] if same_src else None,
-                "flops_per_site": FLOPS_PER_SITE, "fp64_instr_per_site": FP64_INSTR_PER_SITE,
-                "fp64_pipe_frac": round(pipe, 4), "avg_launch_ms": round(ms64, 4),
-                "share_of_step": round(share64, 3), "peak_source": "measured",
+    bps64 = bytes_per_site(8, LS)
+    gbs64 = sites64 * bps64 / (ms64 * 1e-3) / 1e9
+    roofline = {"bound": "hbm", "kernel": "g5dwf FP64 in fixed point (H = Gamma5 D_dwf, with the operand's encoding "
+                                          "where the solve has not encoded it already)",
+                "achieved": round(gbs64, 1), "peak": pk["hbm_gbs"], "unit": "GB/s",
+                "frac": round(gbs64 / pk["hbm_gbs"], 4), "traffic": NCU_TRAFFIC["f64"] if same_src else None,
+                "bytes_per_site": bps64, "flops_per_site": FLOPS_PER_SITE, "tflops": round(achieved, 4),
+                "fp64_fma_tflops": round(fp64_peak, 4), "avg_launch_ms": round(ms64, 4),
+                "share_of_step": round(share64, 3), "peak_source": pk["source"],
                 "with_fused_smoother_step": {
-                    "kernel": "g5dwf FP64 with one Chebyshev recurrence step in its epilogue",
+                    "kernel": "the same with one Chebyshev recurrence step in its epilogue",
                     "launches_per_step": round(st64c["all_launches"] / max(args.steps, 1), 1),
                     "avg_launch_ms": round(ms64c, 4), "share_of_step": round(share64c, 3),
-                    "achieved_tflops": round((FLOPS_PER_SITE + 144) * st64c["sites"] / max(st64c["launches"], 1)
-                                             / max(ms64c * 1e-3, 1e-12) / 1e12, 4)},
-                "peak_note": "FP64 FMA rate measured in this run (hdcr_probe_fma_rate: independent DFMA chains "
-                             "on every SM, FMA = 2 flops); achieved counts the 1416 algorithmic flops per site, "
-                             "fp64_pipe_frac the FP64 instructions the kernel issues against the same rate"}
+                    "tflops": round((FLOPS_PER_SITE + 144) * st64c["sites"] / max(st64c["launches"], 1)
+                                    / max(ms64c * 1e-3, 1e-12) / 1e12, 4)},
+                "peak_note": "the kernel does its products on the integer and FP32 pipes and is limited by their "
+                             "instruction issue, not by memory; fp64_fma_tflops is the FP64 pipe's measured rate "
+                             "(hdcr_probe_fma_rate, FMA = 2 flops), which bounded the operator as FP64 FMAs"}
     roofline_fp32 = {"bound": "hbm", "kernel": "g5dwf FP32 (H = Gamma5 D_dwf)", "achieved": round(gbs32, 1),
                      "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": round(gbs32 / pk["hbm_gbs"], 4),
                      "traffic": NCU_TRAFFIC["f32"] if same_src else None, "bytes_per_site": bps32,
