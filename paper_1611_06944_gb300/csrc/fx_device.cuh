@@ -17,6 +17,12 @@ __device__ __forceinline__ int2 fx_limbs(i64 v) {
   return make_int2((int)(t >> 30), __float_as_int(l));
 }
 
+// the same with the second limb an integer: V = 2^30 x + y
+__device__ __forceinline__ int2 fx_int_limbs(i64 v) {
+  const i64 t = v + (1LL << 29);
+  return make_int2((int)(t >> 30), (int)((unsigned)t & 0x3fffffffu) - (1 << 29));
+}
+
 // V of one component of a group whose largest biased exponent is mx (in range), that exponent's
 // numbers scaled to 2^(52 + up) .. 2^(53 + up), rounded to nearest
 __device__ __forceinline__ i64 fx_fixed(double x, int mx, int up) {

@@ -28,13 +28,9 @@ constexpr int FXT_KC = 8;  // basis vectors per restriction CTA
 // biased exponents that a group's sum may start from, so that it stays a normal number
 constexpr int FXT_LOW = 70, FXT_HIGH = 2000;
 
-__device__ __forceinline__ int2 fxt_limbs(i64 v) {
-  const i64 t = v + (1LL << 29);
-  return make_int2((int)(t >> 30), (int)((unsigned)t & 0x3fffffffu) - (1 << 29));
-}
 __device__ __forceinline__ int4 fxt_encode(cpx<double> x, int ex) {
   if (ex == 0 || ex == FX_RAW) return make_int4(0, 0, 0, 0);
-  const int2 a = fxt_limbs(fx_fixed(x.re, ex, FX_UP)), b = fxt_limbs(fx_fixed(x.im, ex, FX_UP));
+  const int2 a = fx_int_limbs(fx_fixed(x.re, ex, FX_UP)), b = fx_int_limbs(fx_fixed(x.im, ex, FX_UP));
   return make_int4(a.x, a.y, b.x, b.y);
 }
 

@@ -93,3 +93,28 @@ def test_values_outside_the_format(hd, value):
     if fin.any():
         other = np.delete(np.arange(wf.shape[0]), 1)
         assert np.abs(gf[other] - wf[other]).max() <= 1e-14 * np.abs(wf[other]).max()
+
+
+# vector counts whose tiles fill one to six sets of threads and one to three rounds of them (46
+# and 64: one set), Ls for which the last chunk of 96 elements ends inside a group of 16, shares of a block
+@pytest.mark.parametrize("L,Ls,block,nvec", [((4, 4, 2, 2), 3, (2, 2, 1, 1), 2), ((4, 4, 4, 4), 5, (2, 2, 2, 2), 8),
+                                             ((4, 4, 4, 4), 8, (2, 2, 2, 2), 24), ((6, 2, 2, 6), 7, (3, 1, 1, 3), 34),
+                                             ((4, 4, 4, 4), 4, (2, 2, 2, 2), 46), ((4, 4, 4, 4), 5, (2, 2, 2, 2), 64)])
+@pytest.mark.parametrize("scale", [None, "spread", "outside"])
+def test_block_orthonormalisation(hd, L, Ls, block, nvec, scale):
+    v = synth.gaussian_fermion(L, Ls, 6100, count=nvec)
+    if scale == "spread":       # the fifth dimension's profile, and vectors of different sizes
+        v = v * np.exp(-3.0 * np.arange(Ls))[:, None, None]
+        v = v * 10.0 ** (np.arange(nvec) % 7 - 3.0).reshape((-1,) + (1,) * 7)
+    elif scale == "outside":    # groups of one vector below the format's smallest exponent
+        v[0][..., :2, :] *= 1e-220
+    got = host(hd.subspace_from_vectors(hd.Lattice(L, Ls), block, dev(planes(v)), store_dtype=torch.complex128).vectors())
+    q = blocks(got, L, Ls, block).astype(np.clongdouble)
+    x = blocks(host(dev(planes(v))), L, Ls, block).astype(np.clongdouble)
+    for a in range(q.shape[1]):
+        # the second round's Gram matrix is the identity to cond(V)^2 u; its factor's inverse and the
+        # product with it add nvec terms each
+        gram = np.conj(q[:, a]) @ q[:, a].T
+        assert np.abs(gram - np.eye(nvec)).max() <= 1.2e-16 * (16 + 2 * nvec)
+        r = np.conj(q[:, a]) @ x[:, a].T
+        assert (np.abs(np.tril(r, -1)).max(0) / np.sqrt((np.abs(x[:, a]) ** 2).sum(-1))).max() <= 1e-13
