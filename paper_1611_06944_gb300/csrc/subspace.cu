@@ -197,13 +197,13 @@ __device__ __forceinline__ void cqr_tile(int t, int nt, int* j, int* k) {
 // part[a][q] = sum over share q of block a of conj(v_j) v_k (upper 2x2 tiles)
 //
 // As FP64 multiply-adds this ran at 0.79 of the FP64 pipe: 42.4 ms a round at 16^4 x 16 with 24
-// vectors, 16.6 ms now (wide integer multiply-adds, and 16 warps an SM to
-// hide the shared memory reads).  The basis it leads to is orthonormal to 4.5e-16 .. 6.6e-16 where the FP64 sums gave
-// 1.6e-15 .. 4.8e-15 (8^4 x 8, 24 vectors; smaller blocks 3e-16 .. 6e-16, before 3e-16 .. 8e-16).
-// The chunk is encoded in fixed point on its way to shared memory:
-// groups of CQR_G elements of a vector share an exponent, x = (2^30 H + L) 2^(ex - 1079),
-// |H| <= 2^27, -2^29 <= L < 2^29, 57 bits below the group's largest component.  A group's sum
-// is exact in 64 bits up to the dropped L L' (H H' below 2^59, the cross products below 2^62),
+// vectors, 16.6 ms now (the wide integer multiply-adds alone would take 5).  The basis it leads to
+// is orthonormal to 4.4e-16 .. 6.6e-16 where the FP64 sums gave 1.6e-15 .. 4.8e-15 (8^4 x 8, 24
+// vectors; smaller blocks 3e-16 .. 6e-16, before 3e-16 .. 8e-16).  The chunk is encoded in fixed
+// point on its way to shared memory: groups of CQR_G elements of a vector share an exponent,
+// x = (2^30 H + L) 2^(ex - 1079), |H| <= 2^27, -2^29 <= L < 2^29, 57 bits below the group's
+// largest component.  A group's sum is exact in 64 bits up to the dropped L L' (H H' below
+// 2^59, the cross products below 2^62),
 // three wide integer multiply-adds a real product, and groups are added in FP64.  A pair of groups
 // outside the format is summed in FP64 from the vectors.  With fewer tiles than threads the
 // groups of a chunk are dealt to P sets of threads, whose sums are added in the sets' order.
