@@ -265,9 +265,10 @@ int cheb_filter(const FineOp<R>& H, cpx<R>* x, int order, double lam_cut, double
 }
 
 // Steps between rescalings of the filter's recurrence, which keep it in range: a mode at t = cosh(u) grows
-// by e^u a step, and FP32 holds e^16u up to t = 100, 7 times lam_max.  Every 8 steps the
-// norm and the scaling of both terms took 4% of a filter of order 200 (12 fields at 8^3 x 16 x 8).
-constexpr int FILTER_RESCALE = 16;
+// by e^u a step.  The rescaling's norm squares the elements in the field's precision, so what
+// counts is that a mode's square stays finite: in FP32 8 steps hold to t of about 130, 16 to 8.5 ..
+// 15 only, which an eigenvalue of 2.2 lam_max reaches, or lam_cut close to lam_max.
+constexpr int FILTER_RESCALE = 8;
 
 template <typename R>
 int cheb_filter_multi(const FineOp<R>& H, cpx<R>* x, int nrhs, int order, double lam_cut, double lam_max,

@@ -192,3 +192,20 @@ def test_fp64_filter_matches_the_oracle(hd, order):
     want = np.stack([mg.from_blocks(g, v) for v in phi])
     # order x 1e-16 of rounding a step times the blocks' condition number
     assert relerr(natural(host(sub.vectors()), L, Ls), want) <= 1e-10
+
+
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
+def test_filter_with_modes_far_above_its_interval(hd, dtype):
+    """lam_max at 0.35 of the spectrum's top: modes at t = 15, which grow by 30 a step, must not
+    take the recurrence or the rescaling's norm out of range."""
+    L, Ls, block, mf = (4, 4, 2, 4), 5, (2, 2, 1, 2), 0.05
+    U = synth.gauge_field(L, 0.4, 5500)
+    noise = synth.gaussian_fermion(L, Ls, 5501, count=2)
+    sub = hd.build_subspace(hd.Lattice(L, Ls), dev(links(U)), dev(planes(noise)), 1.8, mf, block, order=24,
+                            lam_cut=0.5, lam_max=2.5, filter_dtype=torch.complex64 if dtype == "c64" else torch.complex128)
+    g = mg.Geometry(L, Ls, block)
+    f = np.stack([mg.chebyshev_filter(U, n, 1.8, mf, 1, 0.5, 2.5, 24) for n in noise])
+    phi = mg.block_orthonormalise(mg.to_blocks(g, mg.chiral_split(f)))
+    want = np.stack([mg.from_blocks(g, v) for v in phi])
+    # the blocks' vectors have a condition number of 2.2; 24 steps of about 10 roundings each
+    assert relerr(natural(host(sub.vectors()), L, Ls), want) <= (1e-4 if dtype == "c64" else 1e-11)
