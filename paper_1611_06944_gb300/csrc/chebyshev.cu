@@ -117,7 +117,7 @@ int cheb_smoother(const FineOp<R>& H, const cpx<R>* r, cpx<R>* out, const std::v
   if constexpr (sizeof(R) == 8)
     if (H.fixed() && order >= 1) {
       HDCR_TRY(launch_fx_encode(H.g, r, H.nrhs, H.fx->e0, nullptr, H.fx->u, st));
-      return cheb_smoother_fx(H, H.fx->e0, H.fx->e1, out, c, lo, hi, w, st, matvecs);
+      return cheb_smoother_fx(H, fx_of(H.fx->e0, r), H.fx->e1, out, c, lo, hi, w, st, matvecs);
     }
   const R a = (R)(2.0 / (hi - lo)), b = (R)(-(hi + lo) / (hi - lo));
   // v = H r (held in t0 = T_0 v)
@@ -193,12 +193,12 @@ int cheb_smoother_fx(const FineOp<double>& H, const FxField& a, const FxField& b
   FxChebStep step{};
   step.a = 2.0 / (hi - lo);
   step.b = -(hi + lo) / (hi - lo);
-  // T_0 = v = H r, kept and encoded; then T_k from H (H T_{k-1}), the inner one only encoded
+  // T_0 = v = H r, kept and encoded; then T_k from H (H T_{k-1})
   HDCR_TRY(timed(0, [&] { return launch_fx_g5dwf(g, H.M5, H.mf, u, a, w.t0, H.nrhs, st, &b); }));
   cpx<double>* prev = w.t0;
   cpx<double>* cur = w.t0;
   for (int k = 1; k <= order; ++k) {
-    HDCR_TRY(timed(0, [&] { return launch_fx_g5dwf(g, H.M5, H.mf, u, b, nullptr, H.nrhs, st, &a); }));
+    HDCR_TRY(timed(0, [&] { return launch_fx_g5dwf(g, H.M5, H.mf, u, fx_of(b, cur), w.h1, H.nrhs, st, &a); }));
     step.first = k == 1;
     step.last = k == order && k > 1;
     step.cur = cur;
@@ -206,7 +206,7 @@ int cheb_smoother_fx(const FineOp<double>& H, const FxField& a, const FxField& b
     step.acc = out;
     step.ck = c[k];
     step.c0 = 0.5 * c[0];
-    HDCR_TRY(timed(3, [&] { return launch_fx_g5dwf_cheb(g, H.M5, H.mf, u, a, step, b, H.nrhs, st); }));
+    HDCR_TRY(timed(3, [&] { return launch_fx_g5dwf_cheb(g, H.M5, H.mf, u, fx_of(a, w.h1), step, b, H.nrhs, st); }));
     prev = cur;
     cur = step.prev;
   }
@@ -295,8 +295,8 @@ int cheb_filter_multi(const FineOp<R>& H, cpx<R>* x, int nrhs, int order, double
       step.a = a;
       step.b = b;
       step.first = first;
-      HDCR_TRY(launch_fx_g5dwf(H.g, H.M5, H.mf, fx.u, fx.e0, nullptr, nrhs, st, &fx.e1));
-      return launch_fx_g5dwf_cheb(H.g, H.M5, H.mf, fx.u, fx.e1, step, fx.e0, nrhs, st);
+      HDCR_TRY(launch_fx_g5dwf(H.g, H.M5, H.mf, fx.u, fx_of(fx.e0, cur), h1, nrhs, st, &fx.e1));
+      return launch_fx_g5dwf_cheb(H.g, H.M5, H.mf, fx.u, fx_of(fx.e1, h1), step, fx.e0, nrhs, st);
     }
     return HDCR_OK;
   };

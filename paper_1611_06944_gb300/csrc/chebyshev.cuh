@@ -30,8 +30,8 @@ int cheb_smoother(const FineOp<R>& H, const cpx<R>* r, cpx<R>* out, const std::v
                   double hi, ChebWork<R>& w, cudaStream_t st, int* matvecs);
 
 // The same in FP64 through the encoded fields of H.fx (H.fixed() must hold, order >= 1): r is
-// given encoded in ``a``, and out is left encoded in ``b`` as well (a and b the two fields of
-// H.fx).  Terms pass between the applications encoded.
+// given encoded in ``a`` (with r at a.f64), and out is left encoded in ``b`` as well (a and b the
+// two fields of H.fx).  Terms pass between the applications encoded.
 int cheb_smoother_fx(const FineOp<double>& H, const FxField& a, const FxField& b, cpx<double>* out,
                      const std::vector<double>& c, double lo, double hi, ChebWork<double>& w, cudaStream_t st,
                      int* matvecs);

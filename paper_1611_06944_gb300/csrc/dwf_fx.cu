@@ -36,10 +36,9 @@ __global__ void __launch_bounds__(128) fx_encode_kernel(int ls, i64 nsites, cons
 }
 
 // ------------------------------------------------------------------- stencil
-// a real coefficient of the operator, encoded on the host
+// a real coefficient of the operator, encoded on the host: (h + l / 2^30) 2^(ex - 1052)
 struct FxCoef {
-  int h, ex;
-  float l;
+  int h, l, ex;
   double d;
 };
 
@@ -48,6 +47,15 @@ struct FxParams {
 };
 
 __device__ __forceinline__ int4 ldi(const int4* p) { return __ldg(p); }
+
+// field r of a launch over several
+__device__ __forceinline__ FxField fx_field_r(const Geom& g, const FxField& f, int r) {
+  FxField q;
+  q.v = f.v + (i64)r * 12 * g.V5;
+  q.ex = f.ex + (i64)r * g.V5;
+  q.f64 = f.f64 + (i64)r * 12 * g.V5;
+  return q;
+}
 
 // (row, lower component) tables of i sigma_k: component a of i sigma_k w is
 // sign * i^rot * w[1 - a or a]
@@ -61,75 +69,76 @@ struct ISigma {
 
 // u + S i^rot d
 __device__ __forceinline__ int4 fx_add(int4 u, int4 d, int S, int rot) {
-  const float ul = __int_as_float(u.y), um = __int_as_float(u.w), dl = __int_as_float(d.y), dm = __int_as_float(d.w);
   if (rot == 0)
-    return S > 0 ? make_int4(u.x + d.x, __float_as_int(ul + dl), u.z + d.z, __float_as_int(um + dm))
-                 : make_int4(u.x - d.x, __float_as_int(ul - dl), u.z - d.z, __float_as_int(um - dm));
-  return S > 0 ? make_int4(u.x - d.z, __float_as_int(ul - dm), u.z + d.x, __float_as_int(um + dl))
-               : make_int4(u.x + d.z, __float_as_int(ul + dm), u.z - d.x, __float_as_int(um - dl));
+    return S > 0 ? make_int4(u.x + d.x, u.y + d.y, u.z + d.z, u.w + d.w)
+                 : make_int4(u.x - d.x, u.y - d.y, u.z - d.z, u.w - d.w);
+  return S > 0 ? make_int4(u.x - d.z, u.y - d.w, u.z + d.x, u.w + d.y)
+               : make_int4(u.x + d.z, u.y + d.w, u.z - d.x, u.w - d.y);
 }
 
+// A real of a site is certain once one of its terms is at least 2^52 (high word FX_CERTAIN).  The integers
+// err by about 0.9 of their unit (8 hops' rounded cross products and dropped L L', operands
+// held to 1/2 of the last bit); FP64 multiply-adds round each of some 12 sums to 2^-53 of it, 0.29 of a
+// unit each once it is at 2^52, so from there on they err by as much.  At 2^51 components of 0.1 of a
+// site's largest came out at 1.7e-16 of themselves instead of FP64's 1.5e-16; at 2^53 the error is no
+// smaller where it matters, and a solver's fields send a site or two of 8^4 x 8 to FP64 in most
+// iterations: 94 instead of 68 us an iteration of CR.
+// A term of 2^59 or more (high word FX_HUGE) could take the sum out of range; a term of
+// numbers in the format may reach 2^60.6, with links far from unitary.
+constexpr int FX_CERTAIN = 1 << 20, FX_HUGE = 1 << 27;
+constexpr unsigned FX_ALL = 0xffffff;  // bit 2 (3 spin + colour) + (0 re, 1 im) for each real
+
 // acc -= one hop without its factor 1/2, each colour component of its two spins rounded to
-// nearest after a right shift by sh.  acc[spin][colour][re, im].
+// nearest after a right shift by sh.  acc[spin][colour][re, im].  A complex product takes three
+// real ones, a (c + d), d (a + b) and c (a - b) for (a + i b) (c + i d).
 template <int MU, int SIGN>
 __device__ __forceinline__ void fx_hop(const int4* __restrict__ Ul, const int4* __restrict__ nb, int ls, int sh,
-                                       bool flip, i64 (&acc)[4][3][2]) {
+                                       bool flip, i64 (&acc)[4][3][2], unsigned& ok, int& top) {
   typedef ISigma<MU> T;
-  // the two spins of h = u -+ ..., their high limbs as integers and as floats, and their low limbs
-  int h[2][3][2];
-  float f[2][3][2], l[2][3][2];
+  int4 h[2][3];  // the two spins of u -+ ...
 #pragma unroll
   for (int j = 0; j < 2; ++j)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const int4 u = ldi(nb + (3 * j + c) * ls), d = ldi(nb + (6 + 3 * T::idx(j) + c) * ls);
-      int4 w = fx_add(u, d, SIGN * T::sign(j), T::rot());
-      if (MU == 3 && flip)  // the antiperiodic boundary's factor -1
-        w = make_int4(-w.x, w.y ^ 0x80000000, -w.z, w.w ^ 0x80000000);
-      h[j][c][0] = w.x;
-      h[j][c][1] = w.z;
-      f[j][c][0] = (float)w.x;
-      f[j][c][1] = (float)w.z;
-      l[j][c][0] = __int_as_float(w.y);
-      l[j][c][1] = __int_as_float(w.w);
+      h[j][c] = fx_add(u, d, SIGN * T::sign(j), T::rot());
     }
-  const i64 half = 1LL << (sh - 1);
-  const float down = __int_as_float((127 - sh) << 23);  // 2^-sh
+  const i64 half = (1LL << sh) >> 1;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    int mr[3], mi[3];
-    float fr[3], fi[3], lr[3], li[3];
+    int4 m[3];
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-      const int4 m = ldi(Ul + (SIGN > 0 ? 3 * c + b : 3 * b + c));
-      mr[b] = m.x;
-      mi[b] = m.z;
-      fr[b] = (float)m.x;
-      fi[b] = (float)m.z;
-      lr[b] = __int_as_float(m.y);
-      li[b] = __int_as_float(m.w);
+      m[b] = ldi(Ul + (SIGN > 0 ? 3 * c + b : 3 * b + c));
+      if (MU == 3 && flip) m[b] = make_int4(-m[b].x, -m[b].y, -m[b].z, -m[b].w);  // the antiperiodic boundary
     }
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      // re: m.re v.re -+ m.im v.im;  im: m.re v.im +- m.im v.re
-      i64 hr = half, hi = half;
-      float cr = 0.f, ci = 0.f;
+      i64 k1 = half, k2 = 0, k3 = 0, x1 = 1LL << 29, x2 = 0, x3 = 0;
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
-        const int n = -mi[b];
-        hr = mw(SIGN > 0 ? n : mi[b], h[j][b][1], mw(mr[b], h[j][b][0], hr));
-        hi = mw(SIGN > 0 ? mi[b] : n, h[j][b][0], mw(mr[b], h[j][b][1], hi));
-        cr = fmaf(fr[b], l[j][b][0], fmaf(lr[b], f[j][b][0], cr));
-        ci = fmaf(fr[b], l[j][b][1], fmaf(lr[b], f[j][b][1], ci));
-        const float s = SIGN > 0 ? 1.f : -1.f;
-        cr = fmaf(-s * fi[b], l[j][b][1], fmaf(-s * li[b], f[j][b][1], cr));
-        ci = fmaf(s * fi[b], l[j][b][0], fmaf(s * li[b], f[j][b][0], ci));
+        const int4 v = h[j][b];
+        const int sH = v.x + v.z, sL = v.y + v.w;
+        // a + b and a - b, b the link's imaginary part or, in its adjoint, minus that
+        const int pH = SIGN > 0 ? m[b].x + m[b].z : m[b].x - m[b].z, pL = SIGN > 0 ? m[b].y + m[b].w : m[b].y - m[b].w;
+        const int qH = SIGN > 0 ? m[b].x - m[b].z : m[b].x + m[b].z, qL = SIGN > 0 ? m[b].y - m[b].w : m[b].y + m[b].w;
+        k1 = mw(m[b].x, sH, k1);
+        k2 = mw(pH, v.z, k2);
+        k3 = mw(qH, v.x, k3);
+        x1 = mw(m[b].x, sL, mw(m[b].y, sH, x1));
+        x2 = mw(pH, v.w, mw(pL, v.z, x2));
+        x3 = mw(qH, v.y, mw(qL, v.x, x3));
       }
-      const i64 pr = (hr >> sh) + __float2int_rn(cr * down), pi = (hi >> sh) + __float2int_rn(ci * down);
+      const i64 pr = (k1 - k2 + ((x1 - x2) >> 30)) >> sh, pi = (k1 - k3 + ((x1 - x3) >> 30)) >> sh;
       acc[j][c][0] -= pr;
       acc[j][c][1] -= pi;
       // lower = -+ i sigma h, subtracted: component a takes S i^rot of spin j = idx(a)
       const int a = T::idx(j), S = MU == 3 ? SIGN : SIGN * T::sign(a);
+      const int up = 2 * (3 * j + c), lo = 2 * (3 * (2 + a) + c);
+      const int ar = abs((int)(pr >> 32)), ai = abs((int)(pi >> 32));
+      if (ar >= FX_CERTAIN) ok |= 1u << up | 1u << (lo + T::rot());
+      if (ai >= FX_CERTAIN) ok |= 2u << up | 1u << (lo + 1 - T::rot());
+      top |= ar | ai;
       if (T::rot() == 0) {
         acc[2 + a][c][0] += S > 0 ? pr : -pr;
         acc[2 + a][c][1] += S > 0 ? pi : -pi;
@@ -141,82 +150,80 @@ __device__ __forceinline__ void fx_hop(const int4* __restrict__ Ul, const int4* 
   }
 }
 
-// k v rounded to nearest after a right shift by sh >= 0
+// k v rounded to nearest after a right shift by sh >= 0, in a quarter of the unit of the integers' product
 __device__ __forceinline__ i64 fx_mul(const FxCoef& k, int h, int l, int sh) {
-  const float c = fmaf((float)k.h, __int_as_float(l), k.l * (float)h);
-  return (mw(k.h, h, (1LL << sh) >> 1) >> sh) + __float2int_rn(c * __int_as_float((127 - sh) << 23));
+  const i64 x = mw(k.h, l, mw(k.l, h, 1LL << 27)) >> 28;
+  return ((mw(k.h, h, 0) << 2) + x + ((1LL << sh) >> 1)) >> sh;
 }
 
 // ------------------------------------------------ sites that need FP64 itself
-template <int MU, int SIGN>
-__device__ void fx_slow_hop(const Geom& g, const FxLinks& u, const FxField& in, int ls, int x4, int s, const int co[4],
-                            cpx<double> (&acc)[4][3]) {
-  int ph;
-  const int y4 = neighbour<MU, SIGN>(g, co, &ph);
-  const int l4 = MU * g.V4 + (SIGN > 0 ? x4 : y4);
-  const int le = u.ex[l4], fe = in.ex[y4 * ls + s];
-  cpx<double> m[9], v[12];
-  for (int i = 0; i < 9; ++i) m[i] = fx_value(u.v[(unsigned)(l4 * 9) + i], le, 1052);
-  for (int c = 0; c < 12; ++c) v[c] = fx_value(in.v[(unsigned)(y4 * 12 * ls + s) + c * ls], fe, 1051);
-  const double coef = -0.5 * ph;
-  for (int c = 0; c < 3; ++c) {
-    cpx<double> p[2];
-    for (int a = 0; a < 2; ++a) {
-      cpx<double> t(0.0, 0.0);
-      for (int b = 0; b < 3; ++b) {
-        const cpx<double> d = v[6 + 3 * ISigma<MU>::idx(a) + b];
-        const cpx<double> w = ISigma<MU>::rot() ? times_i(d) : d;
-        const double sg = SIGN * ISigma<MU>::sign(a);
-        const cpx<double> h(v[3 * a + b].re + sg * w.re, v[3 * a + b].im + sg * w.im);
-        t = SIGN > 0 ? cmadd(t, m[3 * c + b], h) : cjmadd(t, m[3 * b + c], h);
-      }
-      p[a] = t;
-      acc[a][c].re = fma(coef, t.re, acc[a][c].re);
-      acc[a][c].im = fma(coef, t.im, acc[a][c].im);
-    }
-    for (int a = 0; a < 2; ++a) {
-      const cpx<double> q = p[ISigma<MU>::idx(a)];
-      const cpx<double> w = ISigma<MU>::rot() ? times_i(q) : q;
-      const double cl = coef * (MU == 3 ? -SIGN : -SIGN * ISigma<MU>::sign(a));
-      acc[2 + a][c].re = fma(cl, w.re, acc[2 + a][c].re);
-      acc[2 + a][c].im = fma(cl, w.im, acc[2 + a][c].im);
-    }
-  }
-}
-
-// (D_dwf in)(x4, s) in FP64 arithmetic from the encoded operands
-__device__ void fx_slow_site(const Geom& g, const FxParams& p, const FxLinks& u, const FxField& in, int x4, int s,
-                             bool local, cpx<double> (&acc)[4][3]) {
-  const int ls = g.Ls;
-  int co[4];
-  x4_coords(g, x4, co);
-  const int sn = s + 1 == ls ? 0 : s + 1, sp = s == 0 ? ls - 1 : s - 1;
-  const double wn = s + 1 == ls ? p.mmf.d : 1.0, wp = s == 0 ? p.mmf.d : 1.0;
-  const int4* b = in.v + (unsigned)(x4 * 12 * ls);
-  const int* e = in.ex + (unsigned)(x4 * ls);
+// (D_dwf in)(x4, s), or its 4d hops alone, from the FP64 operands: the FP64 kernel's arithmetic in
+// its order, with one body for the eight hops.  tab: the site's hop table.
+template <bool LOCAL>
+__device__ __forceinline__ void fx_fp64_site(const FxParams& p, const cpx<double>* U, const cpx<double>* in,
+                                             const int4* tab, int ls, int x4, int s, cpx<double> (&acc)[12]) {
+#pragma unroll
   for (int c = 0; c < 12; ++c) {
-    acc[c / 3][c % 3] = cpx<double>(0.0, 0.0);
-    if (!local) continue;
-    const cpx<double> v = fx_value(b[c * ls + s], e[s], 1051);
-    const int so = c < 6 ? sp : sn;
-    const double w = c < 6 ? wp : wn;
-    const cpx<double> o = fx_value(b[c * ls + so], e[so], 1051);
-    acc[c / 3][c % 3] = cpx<double>(fma(-w, o.re, p.diag.d * v.re), fma(-w, o.im, p.diag.d * v.im));
+    acc[c] = cpx<double>(0.0, 0.0);
+    if (!LOCAL) continue;
+    const cpx<double>* row = in + (unsigned)((x4 * 12 + c) * ls);
+    const bool wall = c < 6 ? s == 0 : s + 1 == ls;
+    const cpx<double> v = ld(row + s), o = ld(row + (c < 6 ? (wall ? ls - 1 : s - 1) : (wall ? 0 : s + 1)));
+    const double w = wall ? p.mmf.d : 1.0;
+    acc[c] = cpx<double>(fma(-w, o.re, p.diag.d * v.re), fma(-w, o.im, p.diag.d * v.im));
   }
-  fx_slow_hop<0, 1>(g, u, in, ls, x4, s, co, acc);
-  fx_slow_hop<0, -1>(g, u, in, ls, x4, s, co, acc);
-  fx_slow_hop<1, 1>(g, u, in, ls, x4, s, co, acc);
-  fx_slow_hop<1, -1>(g, u, in, ls, x4, s, co, acc);
-  fx_slow_hop<2, 1>(g, u, in, ls, x4, s, co, acc);
-  fx_slow_hop<2, -1>(g, u, in, ls, x4, s, co, acc);
-  fx_slow_hop<3, 1>(g, u, in, ls, x4, s, co, acc);
-  fx_slow_hop<3, -1>(g, u, in, ls, x4, s, co, acc);
+#pragma unroll 1
+  for (int d = 0; d < 8; ++d) {
+    const int4 t = tab[d];
+    const int mu = d >> 1;
+    const bool back = d & 1, swap = mu < 2, rot = mu == 0 || mu == 2;  // (ISigma's tables)
+    const double coef = t.w ? 0.5 : -0.5, S = back ? -1.0 : 1.0;
+    const double s0 = mu == 3 ? -S : S, s1 = mu == 0 ? S : -S;  // the signs of i sigma's two components
+    const cpx<double>* nb = in + (unsigned)(t.x * 12 + s);
+    const cpx<double>* Ul = U + (unsigned)t.y;
+    cpx<double> h[2][3], q[2][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const cpx<double> u0 = ld(nb + c * ls), u1 = ld(nb + (3 + c) * ls);
+      cpx<double> d0 = ld(nb + (swap ? 9 + c : 6 + c) * ls), d1 = ld(nb + (swap ? 6 + c : 9 + c) * ls);
+      if (rot) {
+        d0 = times_i(d0);
+        d1 = times_i(d1);
+      }
+      h[0][c] = cpx<double>(fma(s0, d0.re, u0.re), fma(s0, d0.im, u0.im));
+      h[1][c] = cpx<double>(fma(s1, d1.re, u1.re), fma(s1, d1.im, u1.im));
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      q[0][c] = q[1][c] = cpx<double>(0.0, 0.0);
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        cpx<double> m = ld(Ul + (back ? 3 * b + c : 3 * c + b));
+        if (back) m.im = -m.im;
+        q[0][c] = cmadd(q[0][c], m, h[0][b]);
+        q[1][c] = cmadd(q[1][c], m, h[1][b]);
+      }
+    }
+    // lower = -+ i sigma of the upper
+    const double c0 = mu == 3 ? -coef * S : -coef * s0, c1 = mu == 3 ? -coef * S : -coef * s1;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      cpx<double> l0 = swap ? q[1][c] : q[0][c], l1 = swap ? q[0][c] : q[1][c];
+      if (rot) {
+        l0 = times_i(l0);
+        l1 = times_i(l1);
+      }
+      acc[c] = cpx<double>(fma(coef, q[0][c].re, acc[c].re), fma(coef, q[0][c].im, acc[c].im));
+      acc[3 + c] = cpx<double>(fma(coef, q[1][c].re, acc[3 + c].re), fma(coef, q[1][c].im, acc[3 + c].im));
+      acc[6 + c] = cpx<double>(fma(c0, l0.re, acc[6 + c].re), fma(c0, l0.im, acc[6 + c].im));
+      acc[9 + c] = cpx<double>(fma(c1, l1.re, acc[9 + c].re), fma(c1, l1.im, acc[9 + c].im));
+    }
+  }
 }
 
 // ------------------------------------------------------------------ the kernel
 // What a launch does with h = H in at each site
 constexpr int FX_OUT = 0;    // out = h
-constexpr int FX_ENC = 1;    // h encoded into enc
 constexpr int FX_BOTH = 2;   // out = h, h encoded into enc
 constexpr int FX_DOT = 3;    // out = h and Re <src, h> into *result
 constexpr int FX_RES = 4;    // out = src - h, also encoded into enc
@@ -225,7 +232,7 @@ constexpr int FX_CHEB1 = 6;  // prev <- nx = a h + b cur, acc = c0 cur + ck nx, 
 constexpr int FX_CHEBL = 7;  // acc += ck (2 (a h + b cur) - prev), acc encoded into enc
 // the red-black launches: the 4d hops alone, h = D_hop in on the sites of one parity
 constexpr int FX_RB = 8;      // out = h
-// w = M5 v - h, v = src: out = w, |w|^2 into *result and Gamma5 w encoded into enc; with dag
+// w = M5 v - h, v = src: out = w, |w|^2 into *result and Gamma5 w into prev and encoded into enc; with dag
 // v = Gamma5 src and out = Gamma5 w
 constexpr int FX_RBS = 9;
 constexpr bool fx_reduces(int mode) { return mode == FX_DOT || mode == FX_RBS; }
@@ -243,8 +250,8 @@ struct FxEpilogue {
 };
 
 // one complex number of the epilogue: h in, the value to encode out.  The Chebyshev steps
-// are three FP64 multiply-adds a real, each a quarter of the clock that the whole stencil
-// takes per real on the integer and FP32 pipes.
+// are three FP64 multiply-adds a real, 1.5 clocks of an SM beside the 3.4 of the stencil's integer
+// products.
 template <int MODE>
 __device__ __forceinline__ cpx<double> fx_epilogue(const FxEpilogue& ep, i64 o, cpx<double> h, double& dot) {
   if (MODE == FX_OUT || MODE == FX_BOTH || MODE == FX_DOT) st(ep.out + o, h);
@@ -315,7 +322,10 @@ __device__ __forceinline__ void fx_rb_output(const Geom& g, const FxEpilogue& ep
   if (!ep.dag) {
     const int ex = fx_mark(fx_top(h), FX_SITE_MIN, FX_SITE_MAX);
 #pragma unroll
-    for (int c = 0; c < 12; ++c) ep.enc.v[site + c * ls + sr] = fx_encode(h[c], ex, FX_UP);
+    for (int c = 0; c < 12; ++c) {
+      ep.enc.v[site + c * ls + sr] = fx_encode(h[c], ex, FX_UP);
+      st(ep.prev + site + c * ls + sr, h[c]);
+    }
     ep.enc.ex[x4 * ls + sr] = ex;
   }
 }
@@ -334,37 +344,35 @@ constexpr int FX_THREADS = 256;  // (4d site, s) of a tile
 constexpr int FX_BLOCKS = 2;     // full tiles per SM
 constexpr int FX_MAX_SITES = FX_THREADS / 2;  // Ls >= 2
 constexpr int FX_SPLIT_SITES = 32;  // (4d site, s) of a tile whose sites are split over four warps
-// Launches of at most this many 5d sites split them: encoding and operator, whole sites
-// and split, took 17.3 and 9.3 us at 4^4 x 8 (2048 sites), 24.7 and 20.4 at 18,900, the same at
-// 32,768, and 59.9 and 70.8 at 131,072
+// Launches of at most this many 5d sites split them: a call (encoding and operator), whole sites
+// and split, took 25 and 18 us at 4^4 x 8 (2048 sites), 34 and 28 at 18,900, 32 and 31 at
+// 32,768, 43 and 51 at 65,536 and 78 and 91 at 131,072
 constexpr long long FX_SPLIT_MAX = 24576;
 
-// A site that reads an operand outside the format: the whole of its output.  Returns
-// its share of the dot product.
+// A site that reads an operand outside the format, or has a real that is not certain: the whole
+// of its output in FP64
 template <int MODE>
-__device__ __noinline__ double fx_slow_output(Geom g, FxParams p, FxLinks u, FxField in, FxEpilogue ep, int r, int x4,
-                                              int s) {
-  cpx<double> a[4][3], w[12];
-  fx_slow_site(g, p, u, in, x4, s, MODE < FX_RB, a);
+__device__ __forceinline__ void fx_slow_output(const Geom& g, const FxParams& p, const FxLinks& u, const FxField& in,
+                                               const FxEpilogue& ep, const int4* tab, int r, int x4, int s,
+                                               double& dot) {
+  cpx<double> w[12];
+  fx_fp64_site<MODE < FX_RB>(p, u.f64, in.f64, tab, g.Ls, x4, s, w);
   if (MODE >= FX_RB) {
-    double dot = 0.0;
-    for (int c = 0; c < 12; ++c) w[c] = a[c / 3][c % 3];
     fx_rb_output<MODE>(g, ep, g.Ls, x4, s, w, dot);
-    return dot;
+    return;
   }
-  const int so = g.Ls - 1 - s;
-  const i64 o0 = ((i64)r * g.V4 + x4) * 12 * g.Ls + so;
-  double d = 0.0;
+  const i64 site = (i64)r * g.V4 + x4, o0 = site * 12 * g.Ls + (g.Ls - 1 - s);
+#pragma unroll
   for (int c = 0; c < 12; ++c) {
     const double sg = c < 6 ? 1.0 : -1.0;
-    w[c] = fx_epilogue<MODE>(ep, o0 + c * g.Ls, cpx<double>(sg * a[c / 3][c % 3].re, sg * a[c / 3][c % 3].im), d);
+    w[c] = fx_epilogue<MODE>(ep, o0 + c * g.Ls, cpx<double>(sg * w[c].re, sg * w[c].im), dot);
   }
   if (MODE != FX_OUT && MODE != FX_DOT && ep.enc.v) {
     const int ex = fx_mark(fx_top(w), FX_SITE_MIN, FX_SITE_MAX);
+#pragma unroll
     for (int c = 0; c < 12; ++c) ep.enc.v[o0 + c * g.Ls] = fx_encode(w[c], ex, FX_UP);
-    ep.enc.ex[((i64)r * g.V4 + x4) * g.Ls + so] = ex;
+    ep.enc.ex[site * g.Ls + (g.Ls - 1 - s)] = ex;
   }
-  return d;
 }
 
 __device__ __forceinline__ int fx_tile_site(const Geom& g, const FxTile& t, int tile, int i) {
@@ -416,36 +424,39 @@ __device__ __forceinline__ int4 fx_hop_entry(const Geom& g, const FxLinks& u, in
   return make_int4(y4 * g.Ls, l4 * 9, u.ex[l4], mu == 3 && wrap && g.bc_t < 0);
 }
 
-// the encoded form of r 2^(C - 2101) in a site whose numbers have at least lz leading sign-equal bits
+// the encoded form of r 2^(C - 2102) in a site whose numbers have at least lz leading sign-equal bits
 __device__ __forceinline__ int2 fx_renorm(i64 r, int lz) {
-  return fx_limbs(lz >= 5 ? r << (lz - 5) : (r + ((1LL << (5 - lz)) >> 1)) >> (5 - lz));
+  return fx_limbs(lz >= 6 ? r << (lz - 6) : (r + ((1LL << (6 - lz)) >> 1)) >> (6 - lz));
 }
 
 // part < 0: the whole site; else direction part's two hops, and with parts 0 and 1 one chirality
 // of the fifth-dimension part
 template <int LS, int MODE>
 __device__ __forceinline__ void fx_site(const Geom& g, const FxParams& p, const FxLinks& u, const FxField& in,
-                                        const int4* tab, int x4, int s, int C, i64 (&acc)[4][3][2], int part = -1) {
+                                        const int4* tab, int x4, int s, int C, i64 (&acc)[4][3][2], unsigned& ok,
+                                        int part = -1) {
   const int ls = ls_of<LS>(g);
 #pragma unroll
   for (int c = 0; c < 12; ++c) acc[c / 3][c % 3][0] = acc[c / 3][c % 3][1] = 0;
+  int top = 0;
 #pragma unroll 1
   for (int d = part < 0 ? 0 : 2 * part; d < (part < 0 ? 8 : 2 * part + 2); ++d) {
     const int4 t = tab[d];
-    const int sh = min(C - (t.z + __ldg(in.ex + t.x + s)) + 3, 61);
+    const int sh = min(C - (t.z + __ldg(in.ex + t.x + s)), 61);
     const int4* nb = in.v + (unsigned)(t.x * 12 + s);
     const int4* Ul = u.v + (unsigned)t.y;
     switch (d) {
-      case 0: fx_hop<0, 1>(Ul, nb, ls, sh, false, acc); break;
-      case 1: fx_hop<0, -1>(Ul, nb, ls, sh, false, acc); break;
-      case 2: fx_hop<1, 1>(Ul, nb, ls, sh, false, acc); break;
-      case 3: fx_hop<1, -1>(Ul, nb, ls, sh, false, acc); break;
-      case 4: fx_hop<2, 1>(Ul, nb, ls, sh, false, acc); break;
-      case 5: fx_hop<2, -1>(Ul, nb, ls, sh, false, acc); break;
-      case 6: fx_hop<3, 1>(Ul, nb, ls, sh, t.w != 0, acc); break;
-      default: fx_hop<3, -1>(Ul, nb, ls, sh, t.w != 0, acc); break;
+      case 0: fx_hop<0, 1>(Ul, nb, ls, sh, false, acc, ok, top); break;
+      case 1: fx_hop<0, -1>(Ul, nb, ls, sh, false, acc, ok, top); break;
+      case 2: fx_hop<1, 1>(Ul, nb, ls, sh, false, acc, ok, top); break;
+      case 3: fx_hop<1, -1>(Ul, nb, ls, sh, false, acc, ok, top); break;
+      case 4: fx_hop<2, 1>(Ul, nb, ls, sh, false, acc, ok, top); break;
+      case 5: fx_hop<2, -1>(Ul, nb, ls, sh, false, acc, ok, top); break;
+      case 6: fx_hop<3, 1>(Ul, nb, ls, sh, t.w != 0, acc, ok, top); break;
+      default: fx_hop<3, -1>(Ul, nb, ls, sh, t.w != 0, acc, ok, top); break;
     }
   }
+  if (top >= FX_HUGE) ok |= FX_ALL + 1;  // (never FX_ALL then)
   if (MODE >= FX_RB) return;
   // diagonal and fifth dimension: the upper spins couple to s - 1, the lower to s + 1
   const int* e = in.ex + x4 * ls;
@@ -461,25 +472,37 @@ __device__ __forceinline__ void fx_site(const Geom& g, const FxParams& p, const 
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
       const int4 v = ldi(self + c * ls + s), w = ldi(self + c * ls + so);
-      acc[2 * h + c / 3][c % 3][0] += fx_mul(p.diag, v.x, v.y, s0) - fx_mul(k, w.x, w.y, s1);
-      acc[2 * h + c / 3][c % 3][1] += fx_mul(p.diag, v.z, v.w, s0) - fx_mul(k, w.z, w.w, s1);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const i64 a = fx_mul(p.diag, i ? v.z : v.x, i ? v.w : v.y, s0), b = fx_mul(k, i ? w.z : w.x, i ? w.w : w.y, s1);
+        if (max(abs((int)(a >> 32)), abs((int)(b >> 32))) >= FX_CERTAIN) ok |= 1u << (2 * (6 * h + c) + i);
+        acc[2 * h + c / 3][c % 3][i] += a - b;
+      }
     }
   }
 }
 
-// the exponent C of a site's terms: (D_dwf in)(x4, s) = sum 2^(C - 2101); FX_RAW / 2 or more
-// where an operand is not in the format
+// the exponent C of a site's terms: (D_dwf in)(x4, s) = sum 2^(C - 2102); FX_RAW / 2 or more
+// where an operand is not in the format.  ok: every real is certain where all operands are zero
 template <int LS, int MODE>
 __device__ __forceinline__ int fx_scale(const Geom& g, const FxParams& p, const FxField& in, const int4* tab, int x4,
-                                        int s) {
+                                        int s, unsigned& ok) {
   const int ls = ls_of<LS>(g);
   const int* e = in.ex + x4 * ls;
   const int wn = s + 1 == ls, wp = s == 0;
-  int C = 0;
-  if (MODE < FX_RB) C = max(p.diag.ex + __ldg(e + s), max((wn ? p.mmf.ex : p.one.ex) + __ldg(e + (wn ? 0 : s + 1)),
-                                            (wp ? p.mmf.ex : p.one.ex) + __ldg(e + (wp ? ls - 1 : s - 1)))) - 2;
+  int C = 0, any = 0;
+  if (MODE < FX_RB) {
+    const int e0 = __ldg(e + s), en = __ldg(e + (wn ? 0 : s + 1)), ep = __ldg(e + (wp ? ls - 1 : s - 1));
+    any = e0 | en | ep;
+    C = max(p.diag.ex + e0, max((wn ? p.mmf.ex : p.one.ex) + en, (wp ? p.mmf.ex : p.one.ex) + ep)) - 2;
+  }
 #pragma unroll
-  for (int d = 0; d < 8; ++d) C = max(C, tab[d].z + __ldg(in.ex + tab[d].x + s));
+  for (int d = 0; d < 8; ++d) {
+    const int ed = __ldg(in.ex + tab[d].x + s);
+    any |= ed;
+    C = max(C, tab[d].z + ed);
+  }
+  ok = any == 0 ? FX_ALL : 0;
   return C;
 }
 
@@ -510,18 +533,19 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) g5dwf_fx_kernel(Geom g,
     const bool on = site < t.ns && sx4[b][min(site, t.ns - 1)] < g.V4;
     if (on) {
       const int x4 = sx4[b][site];
-      FxField f{in.v + (i64)r * 12 * g.V5, in.ex + (i64)r * g.V5};
+      const FxField f = fx_field_r(g, in, r);
       const int4* tab = tabs[b] + site * 8;
-      const int C = fx_scale<LS, MODE>(g, p, f, tab, x4, s);
-      if (C < FX_RAW / 2) {
-        i64 v[4][3][2];
-        fx_site<LS, MODE>(g, p, u, f, tab, x4, s, C, v);
+      unsigned ok;
+      const int C = fx_scale<LS, MODE>(g, p, f, tab, x4, s, ok);
+      i64 v[4][3][2];
+      if (C < FX_RAW / 2) fx_site<LS, MODE>(g, p, u, f, tab, x4, s, C, v, ok);
+      if (C < FX_RAW / 2 && ok == FX_ALL) {
         const i64 o0 = (i64)r * 12 * g.V5 + (unsigned)(x4 * 12 * ls + (ls - 1 - s));  // the R5 reflection
 #pragma unroll
         for (int c = MODE < FX_RB ? 6 : 12; c < 12; ++c)
 #pragma unroll
           for (int k = 0; k < 2; ++k) v[c / 3][c % 3][k] = -v[c / 3][c % 3][k];  // gamma5
-        if (MODE == FX_ENC || MODE == FX_BOTH) {  // encoded from the integers
+        if (MODE == FX_BOTH) {  // encoded from the integers
           u64 any = 0;
 #pragma unroll
           for (int i = 0; i < 24; ++i) {
@@ -529,15 +553,13 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) g5dwf_fx_kernel(Geom g,
             any |= (u64)(q ^ (q >> 63));
           }
           const int lz = any ? __clzll((i64)any) : 64;
-          int ex = lz == 64 ? 0 : C - lz - 1015;
+          int ex = lz == 64 ? 0 : C - lz - 1016;
           if (lz < 64 && (ex < FX_SITE_MIN || ex > FX_SITE_MAX)) ex = FX_RAW;
 #pragma unroll
           for (int c = 0; c < 12; ++c) {
             const i64 re = v[c / 3][c % 3][0], im = v[c / 3][c % 3][1];
             int4 q = make_int4(0, 0, 0, 0);
-            if (ex == FX_RAW) {
-              q = fx_encode(cpx<double>(fx_to_double(re, C - 1015), fx_to_double(im, C - 1015)), FX_RAW, FX_UP);
-            } else if (ex != 0) {
+            if (ex != 0 && ex != FX_RAW) {
               const int2 a = fx_renorm(re, lz), d = fx_renorm(im, lz);
               q = make_int4(a.x, a.y, d.x, d.y);
             }
@@ -549,14 +571,14 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) g5dwf_fx_kernel(Geom g,
           cpx<double> w[12];
 #pragma unroll
           for (int c = 0; c < 12; ++c)
-            w[c] = cpx<double>(fx_to_double(v[c / 3][c % 3][0], C - 1015), fx_to_double(v[c / 3][c % 3][1], C - 1015));
+            w[c] = cpx<double>(fx_to_double(v[c / 3][c % 3][0], C - 1016), fx_to_double(v[c / 3][c % 3][1], C - 1016));
           fx_rb_output<MODE>(g, ep, ls, x4, s, w, acc_d[0]);
-        } else if (MODE != FX_ENC) {
+        } else {
           cpx<double> w[12];
 #pragma unroll
           for (int c = 0; c < 12; ++c)
-            w[c] = fx_epilogue<MODE>(ep, o0 + c * ls, cpx<double>(fx_to_double(v[c / 3][c % 3][0], C - 1015),
-                                                                  fx_to_double(v[c / 3][c % 3][1], C - 1015)),
+            w[c] = fx_epilogue<MODE>(ep, o0 + c * ls, cpx<double>(fx_to_double(v[c / 3][c % 3][0], C - 1016),
+                                                                  fx_to_double(v[c / 3][c % 3][1], C - 1016)),
                                      acc_d[0]);
           if ((MODE == FX_RES || MODE == FX_CHEB || MODE == FX_CHEB1 || MODE == FX_CHEBL) && ep.enc.v) {
             const int ex = fx_mark(fx_top(w), FX_SITE_MIN, FX_SITE_MAX);
@@ -566,7 +588,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) g5dwf_fx_kernel(Geom g,
           }
         }
       } else {
-        acc_d[0] += fx_slow_output<MODE>(g, p, u, f, ep, r, x4, s);
+        fx_slow_output<MODE>(g, p, u, f, ep, tab, r, x4, s, acc_d[0]);
       }
     }
     fill(tile + gridDim.x, b ^ 1);
@@ -587,6 +609,7 @@ __global__ void __launch_bounds__(4 * FX_SPLIT_SITES, 4) g5dwf_fx_split_kernel(G
   __shared__ int4 tabs[FX_SPLIT_SITES / 2 * 8];
   __shared__ int sx4[FX_SPLIT_SITES / 2];
   __shared__ i64 sum[24][4][FX_SPLIT_SITES];
+  __shared__ unsigned oks[4][FX_SPLIT_SITES];
   const int ls = ls_of<LS>(g);
   const int part = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int site = lane / ls, s = lane - site * ls;
@@ -601,17 +624,20 @@ __global__ void __launch_bounds__(4 * FX_SPLIT_SITES, 4) g5dwf_fx_split_kernel(G
     __syncthreads();
     const int x4 = site < t.ns ? sx4[site] : g.V4;
     const bool on = x4 < g.V4;
-    FxField f{in.v + (i64)r * 12 * g.V5, in.ex + (i64)r * g.V5};
+    const FxField f = fx_field_r(g, in, r);
     int C = FX_RAW;
-    if (on) C = fx_scale<LS, MODE>(g, p, f, tabs + site * 8, x4, s);
-    const bool fx = C < FX_RAW / 2;
+    unsigned ok = 0;
+    if (on) C = fx_scale<LS, MODE>(g, p, f, tabs + site * 8, x4, s, ok);
+    bool fx = C < FX_RAW / 2;
     if (fx) {
       i64 v[4][3][2];
-      fx_site<LS, MODE>(g, p, u, f, tabs + site * 8, x4, s, C, v, part);
+      fx_site<LS, MODE>(g, p, u, f, tabs + site * 8, x4, s, C, v, ok, part);
 #pragma unroll
       for (int i = 0; i < 24; ++i) sum[i][part][lane] = v[i / 6][i / 2 % 3][i % 2];
     }
+    oks[part][lane] = ok;
     __syncthreads();
+    fx = fx && (oks[0][lane] | oks[1][lane] | oks[2][lane] | oks[3][lane]) == FX_ALL;
     if (fx) {
       const i64 o0 = (i64)r * 12 * g.V5 + (unsigned)(x4 * 12 * ls + (ls - 1 - s));  // the R5 reflection
 #pragma unroll
@@ -624,11 +650,11 @@ __global__ void __launch_bounds__(4 * FX_SPLIT_SITES, 4) g5dwf_fx_split_kernel(G
           for (int q = 0; q < 4; ++q) v[k] += sum[2 * c + k][q][lane];
           if (part >= 2) v[k] = -v[k];  // gamma5
         }
-        fx_epilogue<MODE>(ep, o0 + c * ls, cpx<double>(fx_to_double(v[0], C - 1015), fx_to_double(v[1], C - 1015)),
+        fx_epilogue<MODE>(ep, o0 + c * ls, cpx<double>(fx_to_double(v[0], C - 1016), fx_to_double(v[1], C - 1016)),
                           acc_d[0]);
       }
     } else if (on && part == 0) {
-      acc_d[0] += fx_slow_output<MODE>(g, p, u, f, ep, r, x4, s);
+      fx_slow_output<MODE>(g, p, u, f, ep, tabs + site * 8, r, x4, s, acc_d[0]);
     }
     __syncthreads();
   }
@@ -659,7 +685,7 @@ FxField fx_field_at(const Geom& g, int nrhs, void* mem) {
 }
 
 static FxCoef fx_coef(double x) {
-  FxCoef k{0, 0, 0.f, x};
+  FxCoef k{0, 0, 0, x};
   if (x == 0.0) return k;
   int e = 0;
   const double m = frexp(x, &e);  // 0.5 <= |m| < 1, x = m 2^e: biased exponent e + 1022
@@ -669,7 +695,7 @@ static FxCoef fx_coef(double x) {
   }
   const double y = ldexp(m, 30);
   k.h = (int)rint(y);
-  k.l = (float)(y - k.h);
+  k.l = (int)ldexp(y - k.h, 30);  // (53 bits of m below 2^30: exact)
   k.ex = e + 1022;
   return k;
 }
@@ -768,7 +794,6 @@ int launch_fx_g5dwf(const Geom& g, double M5, double mf, const FxLinks& u, const
   FxEpilogue ep{};
   ep.out = out;
   if (enc) ep.enc = *enc;
-  if (!out) return fx_launch<FX_ENC>(g, M5, mf, u, in, ep, nrhs, st);
   if (enc) return fx_launch<FX_BOTH>(g, M5, mf, u, in, ep, nrhs, st);
   return fx_launch<FX_OUT>(g, M5, mf, u, in, ep, nrhs, st);
 }
@@ -780,12 +805,13 @@ int launch_fx_rb_hop(const Geom& g, const FxLinks& u, const FxField& in, cpx<dou
 }
 
 int launch_fx_rb_schur(const Geom& g, double diag, double mf, const FxLinks& u, const FxField& in,
-                       const cpx<double>* src, cpx<double>* out, bool dag, const FxField& enc, RedScratch rs,
-                       double* norm2, int par, cudaStream_t st) {
+                       const cpx<double>* src, cpx<double>* out, bool dag, const FxField& enc, cpx<double>* g5,
+                       RedScratch rs, double* norm2, int par, cudaStream_t st) {
   FxEpilogue ep{};
   ep.src = src;
   ep.out = out;
   ep.enc = enc;
+  ep.prev = g5;
   ep.a = diag;
   ep.c0 = mf;
   ep.dag = dag;
@@ -797,8 +823,9 @@ int launch_fx_rb_schur(const Geom& g, double diag, double mf, const FxLinks& u, 
 // M5^{-1} on the sites of one parity (rbcg.cu describes it), the result encoded: a CTA's rows
 // over s are brought into shared memory in runs, each is substituted by one thread, and a site's
 // 12 rows are encoded together.  FP64 substitution, 3 FP64 instructions a real.
-__global__ void __launch_bounds__(128) fx_rb_m5inv_kernel(Geom g, int ns, const cpx<double>* __restrict__ in, FxField out,
-                                                          int par, double a, double mf) {
+__global__ void __launch_bounds__(128) fx_rb_m5inv_kernel(Geom g, int ns, const cpx<double>* __restrict__ in,
+                                                          cpx<double>* __restrict__ out64, FxField out, int par,
+                                                          double a, double mf) {
   extern __shared__ cpx<double> rows[];  // [ns * 12][Ls + 1]
   __shared__ int sx4[64];
   const int ls = g.Ls, pitch = ls + 1, half = g.V4 / 2;
@@ -839,18 +866,22 @@ __global__ void __launch_bounds__(128) fx_rb_m5inv_kernel(Geom g, int ns, const 
     for (int c = 0; c < 12; ++c) x[c] = rows[(site * 12 + c) * pitch + s];
     const int ex = fx_mark(fx_top(x), FX_SITE_MIN, FX_SITE_MAX);
 #pragma unroll
-    for (int c = 0; c < 12; ++c) out.v[(unsigned)((sx4[site] * 12 + c) * ls + s)] = fx_encode(x[c], ex, FX_UP);
+    for (int c = 0; c < 12; ++c) {
+      const unsigned o = (unsigned)((sx4[site] * 12 + c) * ls + s);
+      out.v[o] = fx_encode(x[c], ex, FX_UP);
+      st(out64 + o, x[c]);
+    }
     out.ex[sx4[site] * ls + s] = ex;
   }
 }
 
-int launch_fx_rb_m5inv(const Geom& g, const cpx<double>* in, const FxField& out, int par, double a, double mf,
-                       cudaStream_t st) {
+int launch_fx_rb_m5inv(const Geom& g, const cpx<double>* in, cpx<double>* out64, const FxField& out, int par,
+                       double a, double mf, cudaStream_t st) {
   int ns = 128 / g.Ls;
   ns = ns < 1 ? 1 : ns > 32 ? 32 : ns;
   const size_t smem = sizeof(cpx<double>) * (size_t)ns * 12 * (g.Ls + 1);
   HDCR_CUDA_TRY(cudaFuncSetAttribute(fx_rb_m5inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  fx_rb_m5inv_kernel<<<(g.V4 / 2 + ns - 1) / ns, 128, smem, st>>>(g, ns, in, out, par, a, mf);
+  fx_rb_m5inv_kernel<<<(g.V4 / 2 + ns - 1) / ns, 128, smem, st>>>(g, ns, in, out64, out, par, a, mf);
   count_launch();
   HDCR_LAUNCH_CHECK();
   return HDCR_OK;
@@ -917,11 +948,11 @@ int launch_fx_g5dwf_cheb(const Geom& g, double M5, double mf, const FxLinks& u, 
   return fx_launch<FX_CHEB>(g, M5, mf, u, in, ep, nrhs, st);
 }
 
-int launch_fx_g5dwf_dot(const Geom& g, double M5, double mf, const FxLinks& u, const FxField& in,
-                        const cpx<double>* in64, cpx<double>* out, RedScratch rs, double* result, cudaStream_t st) {
+int launch_fx_g5dwf_dot(const Geom& g, double M5, double mf, const FxLinks& u, const FxField& in, cpx<double>* out,
+                        RedScratch rs, double* result, cudaStream_t st) {
   FxEpilogue ep{};
   ep.out = out;
-  ep.src = in64;
+  ep.src = in.f64;
   ep.rs = rs;
   ep.result = result;
   return fx_launch<FX_DOT>(g, M5, mf, u, in, ep, 1, st);
@@ -937,11 +968,12 @@ int launch_fx_apply(const Geom& g, double M5, double mf, const cpx<double>* U, c
                     cpx<double>* out, int nrhs, void* scratch, size_t bytes, cudaStream_t st) {
   int fit = nrhs;
   while (fit > 1 && fx_scratch_bytes(g, fit) > bytes) --fit;
-  const FxLinks u = fx_links_at(g, scratch);
+  FxLinks u = fx_links_at(g, scratch);
+  u.f64 = U;
   for (int r = 0; r < nrhs; r += fit) {
     const int m = nrhs - r < fit ? nrhs - r : fit;
-    const FxField f = fx_field_at(g, m, (char*)scratch + fx_links_bytes(g));
     const i64 o = (i64)r * 12 * g.V5;
+    const FxField f = fx_of(fx_field_at(g, m, (char*)scratch + fx_links_bytes(g)), in + o);
     HDCR_TRY(launch_fx_encode(g, in + o, m, f, r == 0 ? U : nullptr, u, st));
     HDCR_TRY(launch_fx_g5dwf(g, M5, mf, u, f, out + o, m, st));
   }
@@ -967,7 +999,8 @@ void fx_ctx_free(FxCtx* c) {
   *c = FxCtx();
 }
 
-int fx_ctx_links(const FxCtx& c, const Geom& g, const cpx<double>* U, cudaStream_t st) {
+int fx_ctx_links(FxCtx& c, const Geom& g, const cpx<double>* U, cudaStream_t st) {
+  c.u.f64 = U;
   return c.mem ? launch_fx_encode(g, nullptr, 0, c.e0, U, c.u, st) : HDCR_OK;
 }
 
@@ -976,7 +1009,7 @@ int fx_ctx_apply(const FxCtx& c, const Geom& g, double M5, double mf, const cpx<
   int slot;
   stencil_timer_begin(0, g.V5 * nrhs, st, &slot);
   int s = launch_fx_encode(g, in, nrhs, c.e0, nullptr, c.u, st);
-  if (s == HDCR_OK) s = launch_fx_g5dwf(g, M5, mf, c.u, c.e0, out, nrhs, st);
+  if (s == HDCR_OK) s = launch_fx_g5dwf(g, M5, mf, c.u, fx_of(c.e0, in), out, nrhs, st);
   stencil_timer_end(slot, st);
   return s;
 }
@@ -986,7 +1019,7 @@ int fx_ctx_apply_dot(const FxCtx& c, const Geom& g, double M5, double mf, const 
   int slot;
   stencil_timer_begin(0, g.V5, st, &slot);
   int s = launch_fx_encode(g, in, 1, c.e0, nullptr, c.u, st);
-  if (s == HDCR_OK) s = launch_fx_g5dwf_dot(g, M5, mf, c.u, c.e0, in, out, rs, result, st);
+  if (s == HDCR_OK) s = launch_fx_g5dwf_dot(g, M5, mf, c.u, fx_of(c.e0, in), out, rs, result, st);
   stencil_timer_end(slot, st);
   return s;
 }

@@ -8,17 +8,10 @@ namespace hdcr {
 typedef long long i64;
 typedef unsigned long long u64;
 
-constexpr int FX_UP = 6;  // a field's largest components: 2^58 <= |V| < 2^59; a link's one more
+constexpr int FX_UP = 5;  // a field's largest components: 2^57 <= |V| < 2^58; a link's one more
 
-// (H, L) of V: H the nearest multiple of 2^30, L the rest as a float in units of it
+// V = 2^30 H + L, H the nearest integer
 __device__ __forceinline__ int2 fx_limbs(i64 v) {
-  const i64 t = v + (1LL << 29);
-  const float l = (float)((int)((unsigned)t & 0x3fffffffu) - (1 << 29)) * 0x1p-30f;
-  return make_int2((int)(t >> 30), __float_as_int(l));
-}
-
-// the same with the second limb an integer: V = 2^30 x + y
-__device__ __forceinline__ int2 fx_int_limbs(i64 v) {
   const i64 t = v + (1LL << 29);
   return make_int2((int)(t >> 30), (int)((unsigned)t & 0x3fffffffu) - (1 << 29));
 }
@@ -54,17 +47,9 @@ __device__ __forceinline__ int fx_mark(unsigned top, int emin, int emax) {
   return !(top >> 31) ? 0 : mx < emin || mx > emax ? FX_RAW : mx;
 }
 
-// one number of a group with exponent mark ex
+// one number of a group with exponent mark ex (whose words are zero outside the format)
 __device__ __forceinline__ int4 fx_encode(cpx<double> x, int ex, int up) {
-  if (ex == FX_RAW)
-    return make_int4(__double2hiint(x.re), __double2loint(x.re), __double2hiint(x.im), __double2loint(x.im));
-  if (ex == 0) return make_int4(0, 0, 0, 0);
-  const int2 a = fx_limbs(fx_fixed(x.re, ex, up)), b = fx_limbs(fx_fixed(x.im, ex, up));
-  return make_int4(a.x, a.y, b.x, b.y);
-}
-
-// the same where ex is known to be in range
-__device__ __forceinline__ int4 fx_encode_in(cpx<double> x, int ex, int up) {
+  if (ex == 0 || ex == FX_RAW) return make_int4(0, 0, 0, 0);
   const int2 a = fx_limbs(fx_fixed(x.re, ex, up)), b = fx_limbs(fx_fixed(x.im, ex, up));
   return make_int4(a.x, a.y, b.x, b.y);
 }
@@ -77,15 +62,6 @@ __device__ __forceinline__ double fx_to_double(i64 r, int be) {
   const u64 n = (m << lz) >> 1;  // leading bit 62
   const u64 q = ((n + 0x1ff + ((n >> 10) & 1)) >> 10) + ((u64)(be - lz - 1) << 52);
   return __longlong_as_double((i64)(q | ((u64)r & 0x8000000000000000ull)));
-}
-
-// the FP64 value of an encoded number of a field (scale 1051) or a link (1052)
-__device__ __forceinline__ double fx_value(int h, int l, int ex, int scale) {
-  if (ex == FX_RAW) return __hiloint2double(h, l);
-  return ldexp((double)h + (double)__int_as_float(l), ex - scale);
-}
-__device__ __forceinline__ cpx<double> fx_value(int4 w, int ex, int scale) {
-  return cpx<double>(fx_value(w.x, w.y, ex, scale), fx_value(w.z, w.w, ex, scale));
 }
 
 __device__ __forceinline__ i64 mw(int a, int b, i64 c) { return c + (i64)a * b; }

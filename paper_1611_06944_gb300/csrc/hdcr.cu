@@ -330,7 +330,7 @@ static int residual(const FineOp<R>& H, SolveCache* c, const cpx<R>* r, const cp
                     cpx<R>* out, cudaStream_t st) {
   if constexpr (sizeof(R) == 8) {
     if (H.fixed()) {
-      const FxField& in = zin ? *zin : H.fx->e0;
+      const FxField in = fx_of(zin ? *zin : H.fx->e0, z);
       if (!zin) HDCR_TRY(launch_fx_encode(H.g, z, H.nrhs, in, nullptr, H.fx->u, st));
       int slot;
       stencil_timer_begin(0, H.g.V5 * H.nrhs, st, &slot);
@@ -352,7 +352,7 @@ static int smooth_residual(const FineOp<R>& H, SolveCache* c, const hdcr_solve_p
                            VStats* vs, cudaStream_t st) {
   if constexpr (sizeof(R) == 8)
     if (H.fixed() && prm->smoother_kind == HDCR_SMOOTHER_CHEBYSHEV)
-      return cheb_smoother_fx(H, H.fx->e1, H.fx->e0, e, c->cheb_c, prm->cheb_lo, prm->cheb_hi,
+      return cheb_smoother_fx(H, fx_of(H.fx->e1, t2), H.fx->e0, e, c->cheb_c, prm->cheb_lo, prm->cheb_hi,
                               *(ChebWork<double>*)c->chw, st, &vs->fine);
   return smooth<R>(H, c, prm, t2, e, vs, st);
 }

@@ -329,13 +329,14 @@ static int rb_solve_impl(const Geom& g, const hdcr_dwf_params* prm, const cpx<do
     for (int k = 0; !converged && k < max_iter; ++k) {
       const int par = k & 1;
       if (fx.mem) {
-        // q = S p from p encoded in e0, with |q|^2 and Gamma5 q encoded there in its place; Ap = S^dag q
-        HDCR_TRY(launch_fx_rb_hop(g, fx.u, fx.e0, w.a, 0, st));
-        HDCR_TRY(launch_fx_rb_m5inv(g, w.a, fx.e1, 0, S.a, S.mf, st));
-        HDCR_TRY(launch_fx_rb_schur(g, S.a, S.mf, fx.u, fx.e1, w.p, w.q, false, fx.e0, rs, &d->qq, 1, st));
-        HDCR_TRY(launch_fx_rb_hop(g, fx.u, fx.e0, w.a, 0, st));
-        HDCR_TRY(launch_fx_rb_m5inv(g, w.a, fx.e1, 0, S.a, S.mf, st));
-        HDCR_TRY(launch_fx_rb_schur(g, S.a, S.mf, fx.u, fx.e1, w.q, w.Ap, true, fx.e0, rs, nullptr, 1, st));
+        // q = S p from p encoded in e0, with |q|^2 and Gamma5 q (g1) encoded there in its place; Ap = S^dag q
+        const FxField y = fx_of(fx.e1, w.b2);
+        HDCR_TRY(launch_fx_rb_hop(g, fx.u, fx_of(fx.e0, w.p), w.a, 0, st));
+        HDCR_TRY(launch_fx_rb_m5inv(g, w.a, w.b2, y, 0, S.a, S.mf, st));
+        HDCR_TRY(launch_fx_rb_schur(g, S.a, S.mf, fx.u, y, w.p, w.q, false, fx.e0, w.g1, rs, &d->qq, 1, st));
+        HDCR_TRY(launch_fx_rb_hop(g, fx.u, fx_of(fx.e0, w.g1), w.a, 0, st));
+        HDCR_TRY(launch_fx_rb_m5inv(g, w.a, w.b2, y, 0, S.a, S.mf, st));
+        HDCR_TRY(launch_fx_rb_schur(g, S.a, S.mf, fx.u, y, w.q, w.Ap, true, fx.e0, nullptr, rs, nullptr, 1, st));
       } else {
         HDCR_TRY(S.schur(w.p, w.q, st));
         HDCR_TRY(launch_norm2<double>(w.q, n, rs, &d->qq, st));

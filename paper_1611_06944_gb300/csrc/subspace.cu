@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(GS_THREADS, 2) cqr_gram_kernel(Geom g, BlockGe
       const int m = fx_mark(top | any, CQR_EX_MIN, CQR_EX_MAX);
       int4 w = make_int4(0, 0, 0, 0);
       if (m != 0 && m != FX_RAW) {
-        const int2 u = fx_int_limbs(fx_fixed(x[0].re, m, CQR_UP)), v = fx_int_limbs(fx_fixed(x[0].im, m, CQR_UP));
+        const int2 u = fx_limbs(fx_fixed(x[0].re, m, CQR_UP)), v = fx_limbs(fx_fixed(x[0].im, m, CQR_UP));
         w = make_int4(u.x, u.y, v.x, v.y);
       }
       xe[k * (CQR_E + 1) + e] = w;

@@ -24,15 +24,12 @@ namespace hdcr {
 namespace cg = cooperative_groups;
 
 constexpr int FXT_THREADS = 128;
+constexpr int FXT_UP = 6;  // the largest components: 2^58 <= |V| < 2^59
 constexpr int FXT_KC = 8;  // basis vectors per restriction CTA
 // biased exponents that a group's sum may start from, so that it stays a normal number
 constexpr int FXT_LOW = 70, FXT_HIGH = 2000;
 
-__device__ __forceinline__ int4 fxt_encode(cpx<double> x, int ex) {
-  if (ex == 0 || ex == FX_RAW) return make_int4(0, 0, 0, 0);
-  const int2 a = fx_int_limbs(fx_fixed(x.re, ex, FX_UP)), b = fx_int_limbs(fx_fixed(x.im, ex, FX_UP));
-  return make_int4(a.x, a.y, b.x, b.y);
-}
+__device__ __forceinline__ int4 fxt_encode(cpx<double> x, int ex) { return fx_encode(x, ex, FXT_UP); }
 
 __global__ void __launch_bounds__(128) fxt_encode_kernel(int ls, i64 sites, const cpx<double>* __restrict__ in, FxField f) {
   const i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x;

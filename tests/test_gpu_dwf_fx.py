@@ -87,7 +87,7 @@ def test_error_is_not_above_the_fp64_kernels(hd, L, Ls, bc, wall):
 
     fp64 = err(apply_with(hd, lat, Ud, pd, 0))
     full = hd.apply_g5dwf(lat, Ud, pd, 1.8, 0.01)
-    # 1.1e-16 measured on every shape, 1.5e-16 for the FP64 kernel
+    # 5e-17 measured on every shape, 1.5e-16 for the FP64 kernel
     assert err(full) <= fp64 <= 2.5e-16
     for k in (3, 2, 1):
         assert torch.equal(apply_with(hd, lat, Ud, pd, k), full)
@@ -209,3 +209,130 @@ def test_filter_with_modes_far_above_its_interval(hd, dtype):
     want = np.stack([mg.from_blocks(g, v) for v in phi])
     # the blocks' vectors have a condition number of 2.2; 24 steps of about 10 roundings each
     assert relerr(natural(host(sub.vectors()), L, Ls), want) <= (1e-4 if dtype == "c64" else 1e-11)
+
+
+def links_of(kind, L):
+    U = synth.gauge_field(L, 0.5, 5600)
+    if kind == "random":
+        return U
+    one = np.zeros_like(U)
+    phase = np.random.default_rng(5601).uniform(-np.pi, np.pi, U.shape[:-2] + (2,))
+    for c, t in enumerate((phase[..., 0], phase[..., 1], -phase[..., 0] - phase[..., 1])):
+        one[..., c, c] = np.exp(1j * t) if kind == "diagonal" else 1.0
+    return one
+
+
+@pytest.mark.parametrize("link", ["unit", "diagonal", "random"])
+@pytest.mark.parametrize("grade", ["colour", "colour_near", "spin", "imaginary", "spread", "zeros"])
+def test_components_of_different_size(hd, link, grade):
+    """Components of a site of very different sizes, with links that mix them and that do not: the error of
+    each component, relative to that component, is not above the FP64 kernel's."""
+    L, Ls, bc = (4, 6, 4, 4), 6, -1
+    U = links_of(link, L)
+    psi = synth.gaussian_fermion(L, Ls, 5602)
+    rng = np.random.default_rng(5603)
+    if grade == "colour":
+        psi = psi * np.array([1.0, 1e-5, 1e-10])
+    elif grade == "colour_near":
+        psi = psi * np.array([1.0, 0.1, 0.02])
+    elif grade == "spin":
+        psi = psi * np.array([1.0, 1e-3, 1e-6, 1e-9])[:, None]
+    elif grade == "imaginary":
+        psi = psi.real + 1e-9j * psi.imag
+    elif grade == "spread":
+        psi = psi * 2.0 ** rng.uniform(-45.0, 0.0, psi.shape)
+    else:
+        psi = psi * rng.integers(0, 2, psi.shape)
+    lat = hd.Lattice(L, Ls, bc)
+    Ud, pd = dev(links(U)), dev(planes(psi))
+    want = apply_extended(U, psi, 0.01, bc)
+    fx = natural(host(hd.apply_g5dwf(lat, Ud, pd, 1.8, 0.01)), L, Ls)
+    fp64 = natural(host(apply_with(hd, lat, Ud, pd, 0)), L, Ls)
+    for part in (np.real, np.imag):
+        # per (spin, colour), and per site over all of them against the site's own terms
+        e, f, w = (np.sqrt((part(a).reshape(-1, 12).astype(np.longdouble) ** 2).sum(0)) for a in (fx - want, fp64 - want, want))
+        # FP64: about 2e-16 of a component (a few of its roundings); both are sums of 2304 random roundings each
+        assert (e <= 1.15 * f + 1e-17 * w).all(), (part.__name__, e / w, f / w)
+
+
+def one_colour(a):
+    a = a.copy()
+    a[..., 1:] = 0.0
+    return a
+
+
+@pytest.mark.parametrize("cycle", ["symmetric", "post"])
+@pytest.mark.parametrize("order", [1, 2, 3])
+def test_short_smoothers_where_every_site_is_computed_in_fp64(hd, order, cycle):
+    """As above with links that do not mix the colours and fields of one colour, whose zero components
+    no sum can make certain: each epilogue behind the FP64 arithmetic, from the FP64 operands that
+    the solver keeps beside the encoded ones."""
+    L, Ls, block, M5, mf = (4, 4, 4, 4), 6, (2, 2, 2, 2), 1.8, 0.05
+    U = links_of("diagonal", L)
+    b = one_colour(synth.gaussian_fermion(L, Ls, 5701))
+    vec = one_colour(synth.gaussian_fermion(L, Ls, 5702, count=8))
+    lat = hd.Lattice(L, Ls)
+    Ud, bd = dev(links(U)), dev(planes(b))
+    sub = hd.subspace_from_vectors(lat, block, dev(planes(vec)))
+    co = hd.build_coarse_op(sub, Ud, M5, mf)
+    x = torch.zeros_like(bd)
+    hd.hdcr_solve_into(co, Ud, bd, x, tol=1e-14, max_outer=1, restart=1, smoother_order=order, coarse_solver="cr",
+                       coarse_tol=1e-13, coarse_max=20000, cycle=cycle)
+    p = mg.HDCRParams(M5=M5, mf=mf, bc_t=1)
+    osub = mg.basis_from_vectors(mg.Geometry(L, Ls, block), vec)
+    A = mg.coarse_op(U, osub, M5, mf, 1)
+    D = mg.coarse_dense(A, osub.geom)
+
+    def S(r):
+        return mg.chebyshev_smoother(U, r, p, 1.0, 64.0, order)
+
+    def Q(c):
+        return np.linalg.solve(D, c.reshape(-1)).reshape(c.shape)
+
+    z = mg.vcycle(U, osub, A, b, p, S=S, Qc=Q, cycle=cycle)
+    w = dwf.apply_H(U, z, M5, mf, 1)
+    want = np.vdot(w, b) / np.vdot(w, w).real * z
+    assert relerr(natural(host(x), L, Ls), want) <= 1e-9
+
+
+@pytest.mark.parametrize("solver", ["cr", "cgne", "hdcr", "multi"])
+def test_solvers_where_every_site_is_computed_in_fp64(hd, solver):
+    L, Ls, block, M5, mf, bc = (4, 4, 4, 4), 6, (2, 2, 2, 2), 1.8, 0.1, -1
+    U = links_of("diagonal", L)
+    b = one_colour(synth.gaussian_fermion(L, Ls, 5801, count=3))
+    lat = hd.Lattice(L, Ls, bc)
+    Ud, bd = dev(links(U)), dev(planes(b))
+    if solver in ("hdcr", "multi"):
+        vec = one_colour(synth.gaussian_fermion(L, Ls, 5802, count=8))
+        co = hd.build_coarse_op(hd.subspace_from_vectors(lat, block, dev(planes(vec))), Ud, M5, mf)
+        hd.coarse_invert(co)
+    if solver == "multi":
+        x = hd.hdcr_solve_multi(co, Ud, bd, tol=1e-10, max_outer=300, restart=8, inner_dtype=torch.complex128)[0]
+    else:
+        solve = {"cr": lambda v: hd.cr_solve(lat, Ud, v, M5, mf, tol=1e-10), "cgne": lambda v: hd.cgne_rb_solve(
+            lat, Ud, v, M5, mf, tol=1e-10), "hdcr": lambda v: hd.hdcr_solve(co, Ud, v, tol=1e-10, max_outer=300, restart=8,
+                                                                           inner_dtype=torch.complex128)}[solver]
+        x = torch.stack([solve(v.contiguous())[0] for v in bd.reshape(3, -1, *bd.shape[-2:])])
+    for f, s in zip(natural(host(x), L, Ls).reshape((3,) + b.shape[1:]), b):
+        r = s - dwf.apply_H(U, f, M5, mf, bc)
+        # the recursive (Schur) residual stops at 1e-10; rounding times the condition number beside it
+        assert np.linalg.norm(r) <= 2e-10 * np.linalg.norm(s)
+        assert not f[..., 1:].any()
+
+
+def test_filter_where_every_site_is_computed_in_fp64(hd):
+    """The FP64 filter on fields whose colours are graded by 1e-5 and 1e-10 with links that do not mix them:
+    one noise field, whose two chiral halves are only normalised in each block."""
+    L, Ls, block, mf, order = (4, 4, 2, 4), 5, (4, 4, 2, 4), 0.05, 20
+    U = links_of("diagonal", L)
+    noise = synth.gaussian_fermion(L, Ls, 5901, count=1) * np.array([1.0, 1e-5, 1e-10])
+    block = (2, 2, 1, 2)
+    sub = hd.build_subspace(hd.Lattice(L, Ls), dev(links(U)), dev(planes(noise)), 1.8, mf, block, order=order,
+                            lam_cut=0.5)
+    g = mg.Geometry(L, Ls, block)
+    f = np.stack([mg.chebyshev_filter(U, n, 1.8, mf, 1, 0.5, 8.0, order) for n in noise])
+    phi = mg.block_orthonormalise(mg.to_blocks(g, mg.chiral_split(f)))
+    want = np.stack([mg.from_blocks(g, v) for v in phi])
+    got = natural(host(sub.vectors()), L, Ls)
+    for c in range(3):  # each colour on its own scale; 20 steps of rounding
+        assert relerr(got[..., c], want[..., c]) <= 1e-12
