@@ -118,3 +118,52 @@ def test_block_orthonormalisation(hd, L, Ls, block, nvec, scale):
         assert np.abs(gram - np.eye(nvec)).max() <= 1.2e-16 * (16 + 2 * nvec)
         r = np.conj(q[:, a]) @ x[:, a].T
         assert (np.abs(np.tril(r, -1)).max(0) / np.sqrt((np.abs(x[:, a]) ** 2).sum(-1))).max() <= 1e-13
+
+
+GRADES = {"colour": (np.array([1.0, 1e-5, 1e-10]), np.array([1e-10, 1e-5, 1.0])),
+          "colour_near": (np.array([1.0, 0.1, 0.01]), np.array([0.01, 0.1, 1.0])),
+          "spin": (np.array([1.0, 1.0, 1e-7, 1e-7])[:, None], np.array([1e-7, 1e-7, 1.0, 1.0])[:, None])}
+
+
+@pytest.mark.parametrize("L,Ls,block,nvec", [((4, 4, 2, 4), 6, (2, 2, 1, 2), 2), ((8, 4, 4, 4), 16, (4, 2, 2, 2), 12),
+                                             ((4, 4, 4, 4), 3, (2, 2, 2, 2), 18)])
+@pytest.mark.parametrize("grade", ["colour", "colour_near", "spin", "imaginary", "one_site"])
+def test_components_of_different_size(hd, L, Ls, block, nvec, grade):
+    """Fields that are large where the basis is small: each real of the coefficients and of the
+    prolonged field is as accurate as FP64 sums of its own terms."""
+    vec = synth.gaussian_fermion(L, Ls, 6200, count=nvec)
+    v = synth.gaussian_fermion(L, Ls, 6201, count=2)
+    if grade in GRADES:
+        vec, v = vec * GRADES[grade][0], v * GRADES[grade][1]
+    elif grade == "imaginary":
+        vec, v = vec.real + 1e-9j * vec.imag, v.real + 1e-9j * v.imag
+    else:  # one 4d site of each block far larger in the field, and far smaller in the basis
+        s = np.ones(tuple(L[::-1]) + (1, 1, 1))
+        s[tuple(slice(None, None, b) for b in block[::-1])] = 1e9
+        vec, v = vec / s, v * s
+    lat = hd.Lattice(L, Ls)
+    sub = hd.subspace_from_vectors(lat, block, dev(planes(vec)))
+    vd = dev(planes(v))
+    c = hd.restrict(sub, vd)
+    f = hd.prolong(sub, c)
+    phi = blocks(host(sub.vectors()), L, Ls, block).astype(np.clongdouble)
+    vb = blocks(host(vd), L, Ls, block).astype(np.clongdouble)
+    got = host(c).astype(np.clongdouble)
+
+    def terms(a, b, conj):
+        """exact a b (a conjugated or not) and the sum of the magnitudes of each real's terms, over the last axis."""
+        s = 1 if conj else -1
+        re, im = a.real * b.real + s * a.imag * b.imag, a.real * b.imag - s * a.imag * b.real
+        tr, ti = np.abs(a.real * b.real) + np.abs(a.imag * b.imag), np.abs(a.real * b.imag) + np.abs(a.imag * b.real)
+        return re.sum(-1), im.sum(-1), tr.sum(-1), ti.sum(-1)
+
+    # FP64 multiply-adds: at most 2 nvec = 36 roundings (prolongation) or the few dozen of a thread (restriction) of
+    # partial sums below the sum of magnitudes, 2^-53 sqrt(36) with a factor of 1.5 over the largest of many
+    bound = 1e-15
+    for r in range(2):
+        re, im, tr, ti = terms(phi, vb[r][None], True)  # (nvec, Vc)
+        assert (np.abs(got[r].real.T - re) <= bound * tr).all() and (np.abs(got[r].imag.T - im) <= bound * ti).all()
+        a, b = phi.transpose(1, 2, 0), got[r][:, None, :]
+        re, im, tr, ti = terms(a, b, False)
+        fb = blocks(host(f), L, Ls, block)[r].astype(np.clongdouble)
+        assert (np.abs(fb.real - re) <= bound * tr).all() and (np.abs(fb.imag - im) <= bound * ti).all()
