@@ -5,13 +5,11 @@
 //   P_S = sum |phi_k^b><phi_k^b| (Eq. 4.3) is a projector (Cholesky QR twice,
 //   Gram-Schmidt for ill-conditioned blocks).
 // All of it runs in FP64; the basis is then stored in the requested dtype.
-#include <algorithm>
 #include <vector>
 
 #include "host_io.cuh"
 #include "chebyshev.cuh"
 #include "coarse.cuh"
-#include "fx_device.cuh"
 
 namespace hdcr {
 
@@ -168,11 +166,6 @@ constexpr int CQR_E = 96;         // elements (site x component) of a block per 
 constexpr int CQR_MAXV = 64;      // largest nvec handled (else Gram-Schmidt throughout)
 constexpr int CQR_TILES = 3;      // 2 x 2 Gram tiles per thread: (nvec/2)(nvec/2+1)/2 <= 3 * 256
 constexpr double CQR_TOL = 1e-8;
-constexpr int CQR_G = 16;         // elements that share an exponent in the Gram kernel's chunk
-constexpr int CQR_GROUPS = CQR_E / CQR_G;
-constexpr int CQR_UP = 4;         // their numbers have at most 57 bits
-constexpr int CQR_EX_MIN = 400, CQR_EX_MAX = 1600;
-constexpr int CQR_BE_MIN = 70, CQR_BE_MAX = 2000;  // a sum's leading exponent, so that it stays a normal number
 
 // offset of element le of block a: elements ordered by the block's 4d sites, then
 // component and s, so one 4d site's 12 Ls elements are contiguous in the field
@@ -195,38 +188,21 @@ __device__ __forceinline__ void cqr_tile(int t, int nt, int* j, int* k) {
 }
 
 // part[a][q] = sum over share q of block a of conj(v_j) v_k (upper 2x2 tiles)
-//
-// As FP64 multiply-adds this ran at 0.79 of the FP64 pipe: 42.4 ms a round at 16^4 x 16 with 24
-// vectors, 16.6 ms now (the wide integer multiply-adds alone would take 5).  The basis it leads to
-// is orthonormal to 4.4e-16 .. 6.6e-16 where the FP64 sums gave 1.6e-15 .. 4.8e-15 (8^4 x 8, 24
-// vectors; smaller blocks 3e-16 .. 6e-16, before 3e-16 .. 8e-16).  The chunk is encoded in fixed
-// point on its way to shared memory: groups of CQR_G elements of a vector share an exponent,
-// x = (2^30 H + L) 2^(ex - 1079), |H| <= 2^27, -2^29 <= L < 2^29, 57 bits below the group's
-// largest component.  A group's sum is exact in 64 bits up to the dropped L L' (H H' below
-// 2^59, the cross products below 2^62),
-// three wide integer multiply-adds a real product, and groups are added in FP64.  A pair of groups
-// outside the format is summed in FP64 from the vectors.  With fewer tiles than threads the
-// groups of a chunk are dealt to P sets of threads, whose sums are added in the sets' order.
-// Rows are CQR_E + 1 elements apart: the vectors of a warp's tiles then lie in different banks.
-__global__ void __launch_bounds__(GS_THREADS, 2) cqr_gram_kernel(Geom g, BlockGeom bg,
-                                                                 const cpx<double>* __restrict__ vecs, int nvec,
-                                                                 int S, const int* __restrict__ skip,
-                                                                 cpx<double>* __restrict__ part) {
-  extern __shared__ int4 xe[];  // [nvec][CQR_E + 1], then the groups' exponents [nvec][CQR_GROUPS]
-  int* ex = reinterpret_cast<int*>(xe + nvec * (CQR_E + 1));
+__global__ void __launch_bounds__(GS_THREADS) cqr_gram_kernel(Geom g, BlockGeom bg, const cpx<double>* __restrict__ vecs,
+                                                              int nvec, int S, const int* __restrict__ skip,
+                                                              cpx<double>* __restrict__ part) {
+  extern __shared__ cpx<double> xs[];  // [nvec][CQR_E]
   const int a = blockIdx.x, q = blockIdx.y;
   if (skip[a]) return;
   const long long fs = g.V5 * 12;
   const long long ne = bg.K5 * 12;
   const long long e0 = ne * q / S, e1 = ne * (q + 1) / S;
   const int nt = nvec / 2, ntiles = nt * (nt + 1) / 2;
-  const int P = max(1, min(CQR_GROUPS, GS_THREADS / ntiles));
-  const int set = P > 1 ? threadIdx.x / ntiles : 0;  // set P and above: threads without a tile
   double acc[CQR_TILES][8];
   int tj[CQR_TILES], tk[CQR_TILES];
 #pragma unroll
   for (int i = 0; i < CQR_TILES; ++i) {
-    const int t = P > 1 ? (i == 0 && set < P ? (int)threadIdx.x - set * ntiles : ntiles) : (int)threadIdx.x + i * GS_THREADS;
+    const int t = threadIdx.x + i * GS_THREADS;
     tj[i] = tk[i] = -1;
     if (t < ntiles) cqr_tile(t, nt, &tj[i], &tk[i]);
 #pragma unroll
@@ -235,99 +211,40 @@ __global__ void __launch_bounds__(GS_THREADS, 2) cqr_gram_kernel(Geom g, BlockGe
   for (long long c0 = e0; c0 < e1; c0 += CQR_E) {
     const int n = (int)(e1 - c0 < CQR_E ? e1 - c0 : CQR_E);
     __syncthreads();
-    // nvec is even and CQR_E a multiple of 16: a half warp holds one group, and whole half
-    // warps leave the loop together
     for (int i = threadIdx.x; i < nvec * CQR_E; i += GS_THREADS) {
       const int k = i / CQR_E, e = i - k * CQR_E;
-      const cpx<double> x[1] = {e < n ? vecs[(long long)k * fs + cqr_off(g, bg, a, c0 + e)] : cpx<double>(0.0, 0.0)};
-      const unsigned half = 0xffffu << (threadIdx.x & 16);
-      unsigned top = fx_top(x), any = top & 0x80000000u;
-      top &= 0x7fffffffu;
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) {
-        top = max(top, __shfl_xor_sync(half, top, o));
-        any |= __shfl_xor_sync(half, any, o);
-      }
-      const int m = fx_mark(top | any, CQR_EX_MIN, CQR_EX_MAX);
-      int4 w = make_int4(0, 0, 0, 0);
-      if (m != 0 && m != FX_RAW) {
-        const int2 u = fx_limbs(fx_fixed(x[0].re, m, CQR_UP)), v = fx_limbs(fx_fixed(x[0].im, m, CQR_UP));
-        w = make_int4(u.x, u.y, v.x, v.y);
-      }
-      xe[k * (CQR_E + 1) + e] = w;
-      if (e % CQR_G == 0) ex[k * CQR_GROUPS + e / CQR_G] = m;
+      xs[i] = e < n ? vecs[(long long)k * fs + cqr_off(g, bg, a, c0 + e)] : cpx<double>(0.0, 0.0);
     }
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < CQR_TILES; ++i) {
       if (tj[i] < 0) continue;
+      const cpx<double>* x0 = xs + tj[i] * CQR_E;
+      const cpx<double>* x1 = x0 + CQR_E;
+      const cpx<double>* y0 = xs + tk[i] * CQR_E;
+      const cpx<double>* y1 = y0 + CQR_E;
       double* A = acc[i];
-      for (int b = set; b * CQR_G < n; b += P) {
-        const int ej[2] = {ex[tj[i] * CQR_GROUPS + b], ex[(tj[i] + 1) * CQR_GROUPS + b]};
-        const int ek[2] = {ex[tk[i] * CQR_GROUPS + b], ex[(tk[i] + 1) * CQR_GROUPS + b]};
-        const int4* x0 = xe + tj[i] * (CQR_E + 1) + b * CQR_G;
-        const int4* y0 = xe + tk[i] * (CQR_E + 1) + b * CQR_G;
-        i64 h[8], l[8];
-#pragma unroll
-        for (int m = 0; m < 8; ++m) h[m] = 0, l[m] = 1LL << 29;
-#pragma unroll 2
-        for (int e = 0; e < CQR_G; ++e) {
-          const int4 u[2] = {x0[e], x0[e + CQR_E + 1]}, w[2] = {y0[e], y0[e + CQR_E + 1]};
-#pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            const int4 p = u[m >> 1], r = w[m & 1];  // conj(p) r
-            const int nz = -p.z, nw = -p.w;
-            h[2 * m] = mw(p.z, r.z, mw(p.x, r.x, h[2 * m]));
-            h[2 * m + 1] = mw(nz, r.x, mw(p.x, r.z, h[2 * m + 1]));
-            l[2 * m] = mw(p.w, r.z, mw(p.z, r.w, mw(p.y, r.x, mw(p.x, r.y, l[2 * m]))));
-            l[2 * m + 1] = mw(nw, r.x, mw(nz, r.y, mw(p.y, r.z, mw(p.x, r.w, l[2 * m + 1]))));
-          }
-        }
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          const int p = ej[m >> 1], r = ek[m & 1];
-          const int be = p + r - 1012;  // both scaled by 2^-1049 (H), a leading bit 63
-          if (p == 0 || r == 0) {
-            if (p != FX_RAW && r != FX_RAW) continue;
-          } else if (p != FX_RAW && r != FX_RAW && be >= CQR_BE_MIN && be <= CQR_BE_MAX) {
-            A[2 * m] += fx_to_double(h[2 * m] + (l[2 * m] >> 30), be);
-            A[2 * m + 1] += fx_to_double(h[2 * m + 1] + (l[2 * m + 1] >> 30), be);
-            continue;
-          }
-          const cpx<double>* f = vecs + (long long)(tj[i] + (m >> 1)) * fs;
-          const cpx<double>* s = vecs + (long long)(tk[i] + (m & 1)) * fs;
-          for (int e = b * CQR_G; e < min(n, (b + 1) * CQR_G); ++e) {
-            const unsigned o = cqr_off(g, bg, a, c0 + e);
-            const cpx<double> u = f[o], w = s[o];
-            A[2 * m] = fma(u.re, w.re, fma(u.im, w.im, A[2 * m]));
-            A[2 * m + 1] = fma(u.re, w.im, fma(-u.im, w.re, A[2 * m + 1]));
-          }
-        }
+      for (int e = 0; e < n; ++e) {
+        const cpx<double> u0 = x0[e], u1 = x1[e], w0 = y0[e], w1 = y1[e];
+        A[0] = fma(u0.re, w0.re, fma(u0.im, w0.im, A[0]));
+        A[1] = fma(u0.re, w0.im, fma(-u0.im, w0.re, A[1]));
+        A[2] = fma(u0.re, w1.re, fma(u0.im, w1.im, A[2]));
+        A[3] = fma(u0.re, w1.im, fma(-u0.im, w1.re, A[3]));
+        A[4] = fma(u1.re, w0.re, fma(u1.im, w0.im, A[4]));
+        A[5] = fma(u1.re, w0.im, fma(-u1.im, w0.re, A[5]));
+        A[6] = fma(u1.re, w1.re, fma(u1.im, w1.im, A[6]));
+        A[7] = fma(u1.re, w1.im, fma(-u1.im, w1.re, A[7]));
       }
     }
   }
-  if (P > 1) {  // one sum of a tile a thread
-    double* sums = reinterpret_cast<double*>(xe);
-    __syncthreads();
-    if (tj[0] >= 0) {
-#pragma unroll
-      for (int m = 0; m < 8; ++m) sums[m * GS_THREADS + threadIdx.x] = acc[0][m];
-    }
-    __syncthreads();
-    if (set > 0) return;
-    for (int p = 1; p < P; ++p) {
-#pragma unroll
-      for (int m = 0; m < 8; ++m) acc[0][m] += sums[m * GS_THREADS + p * ntiles + threadIdx.x];
-    }
-  }
-  cpx<double>* R = part + ((long long)a * S + q) * nvec * nvec;
+  cpx<double>* P = part + ((long long)a * S + q) * nvec * nvec;
 #pragma unroll
   for (int i = 0; i < CQR_TILES; ++i) {
     if (tj[i] < 0) continue;
-    R[tj[i] * nvec + tk[i]] = cpx<double>(acc[i][0], acc[i][1]);
-    R[tj[i] * nvec + tk[i] + 1] = cpx<double>(acc[i][2], acc[i][3]);
-    R[(tj[i] + 1) * nvec + tk[i]] = cpx<double>(acc[i][4], acc[i][5]);
-    R[(tj[i] + 1) * nvec + tk[i] + 1] = cpx<double>(acc[i][6], acc[i][7]);
+    P[tj[i] * nvec + tk[i]] = cpx<double>(acc[i][0], acc[i][1]);
+    P[tj[i] * nvec + tk[i] + 1] = cpx<double>(acc[i][2], acc[i][3]);
+    P[(tj[i] + 1) * nvec + tk[i]] = cpx<double>(acc[i][4], acc[i][5]);
+    P[(tj[i] + 1) * nvec + tk[i] + 1] = cpx<double>(acc[i][6], acc[i][7]);
   }
 }
 
@@ -457,8 +374,7 @@ static int cholesky_qr2(const Geom& g, const BlockGeom& bg, cpx<double>* vecs, i
   // skip flags [0, Vc), then the list of flagged blocks handed to the caller
   if (e == cudaSuccess) e = cudaMallocAsync(&skip, sizeof(int) * (2 * (size_t)Vc + 1), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(skip, 0, sizeof(int) * (2 * (size_t)Vc + 1), st);
-  const size_t smem_gram = std::max((sizeof(int4) * (CQR_E + 1) + sizeof(int) * CQR_GROUPS) * (size_t)nvec,
-                                    sizeof(double) * 8 * GS_THREADS);
+  const size_t smem_gram = sizeof(cpx<double>) * (size_t)nvec * CQR_E;
   const size_t smem_chol = sizeof(cpx<double>) * nn + sizeof(double) * nvec;
   const size_t smem_apply = sizeof(cpx<double>) * (nn + (size_t)nvec * CQR_E);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(cqr_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_gram);

@@ -95,8 +95,8 @@ def test_values_outside_the_format(hd, value):
         assert np.abs(gf[other] - wf[other]).max() <= 1e-14 * np.abs(wf[other]).max()
 
 
-# vector counts whose tiles fill one to six sets of threads and one to three rounds of them (46
-# and 64: one set), Ls for which the last chunk of 96 elements ends inside a group of 16, shares of a block
+# vector counts whose tiles fill one to three rounds of the threads, Ls for which the last chunk of 96
+# elements is short, shares of a block
 @pytest.mark.parametrize("L,Ls,block,nvec", [((4, 4, 2, 2), 3, (2, 2, 1, 1), 2), ((4, 4, 4, 4), 5, (2, 2, 2, 2), 8),
                                              ((4, 4, 4, 4), 8, (2, 2, 2, 2), 24), ((6, 2, 2, 6), 7, (3, 1, 1, 3), 34),
                                              ((4, 4, 4, 4), 4, (2, 2, 2, 2), 46), ((4, 4, 4, 4), 5, (2, 2, 2, 2), 64)])
@@ -106,7 +106,7 @@ def test_block_orthonormalisation(hd, L, Ls, block, nvec, scale):
     if scale == "spread":       # the fifth dimension's profile, and vectors of different sizes
         v = v * np.exp(-3.0 * np.arange(Ls))[:, None, None]
         v = v * 10.0 ** (np.arange(nvec) % 7 - 3.0).reshape((-1,) + (1,) * 7)
-    elif scale == "outside":    # groups of one vector below the format's smallest exponent
+    elif scale == "outside":    # parts of one vector whose squares underflow
         v[0][..., :2, :] *= 1e-220
     got = host(hd.subspace_from_vectors(hd.Lattice(L, Ls), block, dev(planes(v)), store_dtype=torch.complex128).vectors())
     q = blocks(got, L, Ls, block).astype(np.clongdouble)
@@ -167,3 +167,26 @@ def test_components_of_different_size(hd, L, Ls, block, nvec, grade):
         re, im, tr, ti = terms(a, b, False)
         fb = blocks(host(f), L, Ls, block)[r].astype(np.clongdouble)
         assert (np.abs(fb.real - re) <= bound * tr).all() and (np.abs(fb.imag - im) <= bound * ti).all()
+
+
+@pytest.mark.parametrize("nvec", [2, 6])
+def test_block_orthonormalisation_of_vectors_at_opposite_walls(hd, nvec):
+    """Half of the vectors decay from one wall and half from the other, by e^-2 a site: where an orthonormal
+    vector is smallest (1e-13) it comes from Gram entries of 1e-12, which must be as accurate as their own
+    terms allow."""
+    L, Ls, block = (4, 4, 2, 4), 16, (2, 2, 1, 2)
+    s = np.arange(Ls)
+    v = synth.gaussian_fermion(L, Ls, 6300, count=nvec)
+    for k in range(nvec):
+        v[k] *= np.exp(-2.0 * (s if k < nvec // 2 else s[::-1]))[:, None, None]
+    got = blocks(host(hd.subspace_from_vectors(hd.Lattice(L, Ls), block, dev(planes(v))).vectors()), L, Ls, block)
+    q = blocks(host(dev(planes(v))), L, Ls, block).astype(np.clongdouble)
+    for k in range(nvec):  # modified Gram-Schmidt, twice, in extended precision
+        for _ in range(2):
+            for j in range(k):
+                q[k] -= q[j] * (np.conj(q[j]) * q[k]).sum(-1, keepdims=True)
+        q[k] /= np.sqrt((np.abs(q[k]) ** 2).sum(-1, keepdims=True))
+    shape = (nvec, q.shape[1], -1, 12, Ls)
+    e = np.sqrt((np.abs((got - q).reshape(shape)) ** 2).sum((1, 2, 3)))
+    w = np.sqrt((np.abs(q.reshape(shape)) ** 2).sum((1, 2, 3)))
+    assert (e <= 1e-13 * w).all(), e / w
