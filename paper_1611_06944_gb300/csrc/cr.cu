@@ -268,6 +268,7 @@ HDCR_INST_CR(float)
 
 void cr_graph_free(CRGraph* g) {
   if (g->exec) cudaGraphExecDestroy(g->exec);
+  if (g->far) cudaGraphExecDestroy(g->far);
   *g = CRGraph();
 }
 
@@ -299,7 +300,8 @@ static int cr_solve_impl(const Geom& g, const hdcr_dwf_params* p, const void* U,
   CRConfig cfg;
   cfg.tol = tol;
   cfg.max_iter = max_iter;
-  cfg.check_every = 8;
+  cfg.check_every = sizeof(R) == 8 ? 2 : 8;
+  cfg.ahead = sizeof(R) == 8 ? 4 : 1;
   CRGraph graph;  // the iterations between host checks replay from one CUDA graph
   cfg.graph = &graph;
   CRResult res;

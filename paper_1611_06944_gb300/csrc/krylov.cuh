@@ -3,6 +3,8 @@
 // no host synchronisation.
 #pragma once
 
+#include <math.h>
+
 #include "dwf_fx.cuh"
 
 namespace hdcr {
@@ -88,6 +90,8 @@ struct CRGraph {
   long long n = 0;
   int ck = 0;
   unsigned long long kernels = 0;  // kernels one replay launches
+  cudaGraphExec_t far = nullptr;   // CRConfig::ahead times as many iterations
+  unsigned long long far_kernels = 0;
 };
 void cr_graph_free(CRGraph* g);
 // the current device's stream for captures (created once, non-blocking)
@@ -99,6 +103,7 @@ struct CRConfig {
   int fixed_iters = -1; // >= 0: run exactly this many iterations, no test, no host sync
   bool x_zero = false;  // x is zero on entry: skip the initial H x
   int check_every = 4;  // host convergence test every k iterations
+  int ahead = 1;  // above 1: k * ahead iterations a graph replay while the residual is far from the tolerance
   CRGraph* graph = nullptr;  // convergence mode: replay the iterations from this graph
 };
 
@@ -194,37 +199,46 @@ int cr_run(const Op& A, const cpx<R>* b, cpx<R>* x, CRWork<R>& w, const CRConfig
       cr_graph_free(gr);
       cudaStream_t cs;
       HDCR_TRY(capture_stream(&cs));
-      const unsigned long long before = launches_so_far();
-      HDCR_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-      int cap = HDCR_OK;
-      for (int i = 0; i < ck && cap == HDCR_OK; ++i) {
-        cap = launch_cr_update_xr<R>(x, w.r, w.p, w.Ap, n, rs, s, cs);
-        if (cap == HDCR_OK && cudaMemcpyAsync(ring + i, &s->rr, sizeof(double), cudaMemcpyDeviceToHost, cs) !=
-                                  cudaSuccess)
-          cap = HDCR_ERR_CUDA;
-        if (cap == HDCR_OK) cap = A.apply_dot(w.r, w.Ar, rs, &s->gamma_new, cs);
-        if (cap == HDCR_OK) cap = launch_cr_update_p<R>(w.r, w.p, w.Ar, w.Ap, n, rs, s, cs);
-      }
-      cudaGraph_t graph = nullptr;
-      const cudaError_t ee = cudaStreamEndCapture(cs, &graph);
-      if (cap == HDCR_OK && ee == cudaSuccess) {
-        if (cudaGraphInstantiate(&gr->exec, graph, 0) != cudaSuccess) gr->exec = nullptr;
-      }
-      if (graph) cudaGraphDestroy(graph);
-      cudaGetLastError();
-      gr->kernels = launches_so_far() - before;
-      uncount_launches(gr->kernels);  // captured, not launched
+      auto capture = [&](int iters, cudaGraphExec_t* exec, unsigned long long* kernels) -> int {
+        const unsigned long long before = launches_so_far();
+        HDCR_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+        int cap = HDCR_OK;
+        for (int i = 0; i < iters && cap == HDCR_OK; ++i) {
+          cap = launch_cr_update_xr<R>(x, w.r, w.p, w.Ap, n, rs, s, cs);
+          if (cap == HDCR_OK && cudaMemcpyAsync(ring + i % ck, &s->rr, sizeof(double), cudaMemcpyDeviceToHost, cs) !=
+                                    cudaSuccess)
+            cap = HDCR_ERR_CUDA;
+          if (cap == HDCR_OK) cap = A.apply_dot(w.r, w.Ar, rs, &s->gamma_new, cs);
+          if (cap == HDCR_OK) cap = launch_cr_update_p<R>(w.r, w.p, w.Ar, w.Ap, n, rs, s, cs);
+        }
+        cudaGraph_t graph = nullptr;
+        const cudaError_t ee = cudaStreamEndCapture(cs, &graph);
+        if (cap == HDCR_OK && ee == cudaSuccess) {
+          if (cudaGraphInstantiate(exec, graph, 0) != cudaSuccess) *exec = nullptr;
+        }
+        if (graph) cudaGraphDestroy(graph);
+        cudaGetLastError();
+        *kernels = launches_so_far() - before;
+        uncount_launches(*kernels);  // captured, not launched
+        return HDCR_OK;
+      };
+      HDCR_TRY(capture(ck, &gr->exec, &gr->kernels));
+      if (gr->exec && cfg.ahead > 1) HDCR_TRY(capture(ck * cfg.ahead, &gr->far, &gr->far_kernels));
       gr->n = n;
       gr->ck = ck;
       for (int i = 0; i < 6; ++i) gr->key[i] = key[i];
     }
     // whole chunks from the graph while they fit under niter; the rest runs eagerly below
+    bool far = false;
+    double before = ring[0];  // |r|^2 before the chunk
     while (gr->exec && k0 + ck <= niter) {
-      HDCR_CUDA_TRY(cudaGraphLaunch(gr->exec, st));
-      count_launches(gr->kernels);
-      k0 += ck;
+      if (k0 + ck * cfg.ahead > niter) far = false;
+      const int run = far ? cfg.ahead : 1;
+      HDCR_CUDA_TRY(cudaGraphLaunch(far ? gr->far : gr->exec, st));
+      count_launches(far ? gr->far_kernels : gr->kernels);
+      k0 += run * ck;
       out.iters = k0;
-      out.matvecs += ck;
+      out.matvecs += run * ck;
       HDCR_CUDA_TRY(cudaStreamSynchronize(st));
       for (int i = 0; i < ck; ++i) {
         const double rr = ring[i];
@@ -243,6 +257,12 @@ int cr_run(const Op& A, const cpx<R>* b, cpx<R>* x, CRWork<R>& w, const CRConfig
         if (res) *res = out;
         return HDCR_OK;
       }
+      // the longer chunk where one that shrinks the residual as the last did would leave |r|^2 at 16
+      // times its goal: near the tolerance every short chunk is tested
+      const double rr = ring[ck - 1];
+      const double shrink = before > rr ? pow(rr / before, (double)cfg.ahead / run) : 1.0;
+      far = gr->far && rr * shrink > 16.0 * cfg.tol * cfg.tol * scale2;
+      before = rr;
     }
   }
   int pending = 0;

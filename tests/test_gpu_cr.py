@@ -128,3 +128,17 @@ def test_cr_fp32_on_many_site_groups(hd):
     true = np.sqrt(dwf.norm2(br - dwf.apply_H(Ur, xg, 1.8, 0.01)) / dwf.norm2(br))
     assert true < 1e-2          # FP32 recursion: the true residual stalls above the recursive one
     assert abs(st["true_resid"] - true) <= 0.05 * true
+
+
+@pytest.mark.parametrize("mf", [0.05, 0.8])
+def test_cr_fp64_stops_within_two_iterations_of_its_tolerance(hd, mf):
+    """FP64 CR tests every second iteration: three fewer must not reach the tolerance."""
+    L, Ls = (4, 4, 2, 4), 6
+    U, b = dev(links(synth.gauge_field(L, 0.3, 1300))), dev(planes(synth.gaussian_fermion(L, Ls, 1301)))
+    lat = hd.Lattice(L, Ls)
+    for tol in (3e-1, 1e-1, 1e-2, 1e-3, 1e-4, 3e-6, 1e-8, 1e-10):
+        n = hd.cr_solve(lat, U, b, 1.8, mf, tol=tol)[1]["iters"]
+        if n > 3:
+            with pytest.raises(hd.HDCRError) as e:
+                hd.cr_solve(lat, U, b, 1.8, mf, tol=tol, max_iter=n - 3)
+            assert e.value.status == -3
