@@ -161,10 +161,10 @@ int hdcr_apply_g5dwf(const hdcr_geom* g, const hdcr_dwf_params* p, const void* U
  * encodes its operands as fixed-point integers in device memory first, in
  * hdcr_apply_scratch_bytes bytes for all nrhs fields; with less, a multiple of fields at a time
  * that fits (at least hdcr_apply_scratch_bytes for one field), and with less than that
- * on the FP64 pipe from the operands themselves, several times slower.  The integers hold
+ * on the FP64 pipe from the operands themselves, about three times slower, as hdcr_apply_g5dwf does,
+ * which allocates nothing.  The integers hold
  * 58 bits below the largest component of a 5d site; a site with a component for which that would
- * be less accurate than FP64 arithmetic is computed in FP64 from the operands.  hdcr_apply_g5dwf
- * allocates the scratch on ``stream`` from the device's memory pool.  ``scratch`` is 16-byte
+ * be less accurate than FP64 arithmetic is computed in FP64 from the operands.  ``scratch`` is 16-byte
  * aligned and used on ``stream`` only until the call's work there is done; it may be null.
  * hdcr_apply_scratch_bytes is 0 for other dtypes and for a geometry that is not admissible. */
 size_t hdcr_apply_scratch_bytes(const hdcr_geom* g, int dtype, int nrhs);

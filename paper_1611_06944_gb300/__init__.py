@@ -229,8 +229,8 @@ _SCRATCH_MAX = 1 << 30  # most scratch bytes an application over many fields ask
 
 def _apply_scratch(lat, psi, n, stream):
     """Scratch of an FP64 application from torch's allocator, allocated on the stream that
-    uses it; None where the library allocates what it can itself: under stream capture, and
-    when torch is out of memory."""
+    uses it; None under stream capture, where a graph would keep naming it, and when torch is out of
+    memory: the application then runs on the FP64 pipe without scratch."""
     one, field = lat._scratch
     if one == 0 or torch._C._cuda_isCurrentStreamCapturing():
         return None

@@ -310,19 +310,8 @@ extern "C" int hdcr_apply_g5dwf(const hdcr_geom* gp, const hdcr_dwf_params* p, c
     stencil_timer_end(slot, as_stream(stream));
     return s;
   }
-  if (dtype == HDCR_C128) {
-    cudaStream_t st = as_stream(stream);
-    const size_t one = fx_scratch_bytes(g, 1), all = fx_scratch_bytes(g, nrhs), most = (size_t)1 << 30;
-    const size_t bytes = all <= most ? all : one > most ? one : most;
-    void* scratch = nullptr;
-    if (!fx_ok(g) || cudaMallocAsync(&scratch, bytes, st) != cudaSuccess) {
-      cudaGetLastError();
-      scratch = nullptr;
-    }
-    const int s = apply_c128(g, p, U, in, out, nrhs, scratch, bytes, st);
-    if (scratch) cudaFreeAsync(scratch, st);
-    return s;
-  }
+  // without scratch, which only the caller can keep: the FP64 pipe
+  if (dtype == HDCR_C128) return launch_g5dwf<double>(g, p->M5, p->mf, U, in, out, nrhs, as_stream(stream));
   if (dtype == HDCR_C64) return launch_g5dwf<float>(g, p->M5, p->mf, U, in, out, nrhs, as_stream(stream));
   set_error("hdcr_apply_g5dwf: unknown dtype %d", dtype);
   return HDCR_ERR_BAD_ARG;

@@ -336,3 +336,41 @@ def test_filter_where_every_site_is_computed_in_fp64(hd):
     got = natural(host(sub.vectors()), L, Ls)
     for c in range(3):  # each colour on its own scale; 20 steps of rounding
         assert relerr(got[..., c], want[..., c]) <= 1e-12
+
+
+def test_c_entry_allocates_nothing(hd):
+    """hdcr_apply_g5dwf in FP64 takes no memory from the device's pool, eagerly and captured (an
+    allocation node would keep a graph from running twice at once), and is the FP64 kernel."""
+    L, Ls = (4, 4, 2, 4), 6
+    lat = hd.Lattice(L, Ls)
+    U = dev(links(synth.gauge_field(L, 0.5, 6000)))
+    psi = dev(planes(synth.gaussian_fermion(L, Ls, 6001, count=2)))
+    g, p = lat.c_geom(), hd._params(1.8, 0.01)
+    hd._L.hdcr_apply_scratch_bytes
+    with open("/proc/self/maps") as f:
+        path = next(line.split()[-1] for line in f if "libcudart" in line)
+    rt = ctypes.CDLL(path)
+    pool, used, zero = ctypes.c_void_p(), ctypes.c_uint64(), ctypes.c_uint64(0)
+    assert rt.cudaDeviceGetDefaultMemPool(ctypes.byref(pool), torch.cuda.current_device()) == 0
+    used_high = 8  # cudaMemPoolAttrUsedMemHigh
+
+    def call(out):
+        assert hd._L.hdcr_apply_g5dwf(hd.C_ref(g), hd.C_ref(p), U.data_ptr(), psi.data_ptr(), out.data_ptr(), 0, 2,
+                                      ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+
+    want = apply_with(hd, lat, U, psi, 0)
+    eager, captured, binding = torch.empty_like(psi), torch.zeros_like(psi), torch.zeros_like(psi)
+    torch.cuda.synchronize()
+    assert rt.cudaMemPoolSetAttribute(pool, used_high, ctypes.byref(zero)) == 0
+    call(eager)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call(captured)
+        hd.apply_g5dwf(lat, U, psi, 1.8, 0.01, out=binding)
+    for _ in range(2):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert rt.cudaMemPoolGetAttribute(pool, used_high, ctypes.byref(used)) == 0
+    assert used.value == 0
+    assert torch.equal(eager, want) and torch.equal(captured, want) and torch.equal(binding, want)
