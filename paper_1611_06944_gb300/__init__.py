@@ -148,12 +148,15 @@ class Lattice:
         return self.V4 * self.Ls
 
     @functools.cached_property
-    def _scratch(self) -> tuple:
-        """(bytes of links, bytes a field) of an FP64 application's scratch, (0, 0) for none."""
-        g = self.c_geom()
-        one = _L.hdcr_apply_scratch_bytes(C_ref(g), _lib.HDCR_C128, 1)
-        two = _L.hdcr_apply_scratch_bytes(C_ref(g), _lib.HDCR_C128, 2)
-        return one, two - one
+    def _scratch(self) -> dict:
+        """{number of fields: bytes of an FP64 application's scratch}, filled as numbers are met."""
+        return {}
+
+    def _scratch_bytes(self, n: int) -> int:
+        size = self._scratch.get(n)
+        if size is None:
+            size = self._scratch[n] = _L.hdcr_apply_scratch_bytes(C_ref(self.c_geom()), _lib.HDCR_C128, n)
+        return size
 
     def c_geom(self) -> _lib.hdcr_geom:
         g = _lib.hdcr_geom()
@@ -231,10 +234,11 @@ def _apply_scratch(lat, psi, n, stream):
     """Scratch of an FP64 application from torch's allocator, allocated on the stream that
     uses it; None under stream capture, where a graph would keep naming it, and when torch is out of
     memory: the application then runs on the FP64 pipe without scratch."""
-    one, field = lat._scratch
-    if one == 0 or torch._C._cuda_isCurrentStreamCapturing():
+    size = lat._scratch_bytes(n)
+    if size == 0 or torch._C._cuda_isCurrentStreamCapturing():
         return None
-    size = max(one, min(one + (n - 1) * field, _SCRATCH_MAX))
+    if size > _SCRATCH_MAX:
+        size = max(lat._scratch_bytes(1), _SCRATCH_MAX)
     try:
         if stream is None:
             return torch.empty(size, dtype=torch.uint8, device=psi.device)

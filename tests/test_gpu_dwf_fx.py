@@ -374,3 +374,16 @@ def test_c_entry_allocates_nothing(hd):
     assert rt.cudaMemPoolGetAttribute(pool, used_high, ctypes.byref(used)) == 0
     assert used.value == 0
     assert torch.equal(eager, want) and torch.equal(captured, want) and torch.equal(binding, want)
+
+
+@pytest.mark.parametrize("L,Ls,n", [((3, 3, 3, 2), 7, 3), ((3, 5, 3, 3), 7, 6), ((5, 3, 1, 3), 2, 12), ((4, 4, 2, 2), 4, 5)])
+def test_binding_asks_for_scratch_of_all_fields(hd, L, Ls, n):
+    """V5 = 2, 1, 2 and 0 mod 4: the exponents of n fields are rounded up once, not n times.  One encoding
+    and one operator launch."""
+    lat = hd.Lattice(L, Ls)
+    U = dev(links(synth.gauge_field(L, 0.5, 6100)))
+    psi = dev(planes(synth.gaussian_fermion(L, Ls, 6101, count=n)))
+    before = hd._L.hdcr_launch_count()
+    out = hd.apply_g5dwf(lat, U, psi, 1.8, 0.01)
+    assert hd._L.hdcr_launch_count() - before == 2
+    assert torch.equal(out, apply_with(hd, lat, U, psi, n))
