@@ -295,7 +295,7 @@ static int cr_solve_impl(const Geom& g, const hdcr_dwf_params* p, const void* U,
   CRWork<R> w;
   HDCR_TRY(crwork_alloc<R>(&w, H.n()));
   FxCtx fx;
-  if (sizeof(R) == 8) fx_ctx_alloc(&fx, g, 1);
+  if (sizeof(R) == 8) fx_ctx_alloc(&fx, g, 1, 1);
   H.fx = &fx;
   CRConfig cfg;
   cfg.tol = tol;

@@ -980,18 +980,18 @@ int launch_fx_apply(const Geom& g, double M5, double mf, const cpx<double>* U, c
   return HDCR_OK;
 }
 
-void fx_ctx_alloc(FxCtx* c, const Geom& g, int nrhs) {
+void fx_ctx_alloc(FxCtx* c, const Geom& g, int nrhs, int vectors) {
   *c = FxCtx();
   if (!fx_ok(g)) return;
   const size_t lb = fx_links_bytes(g), fb = fx_field_bytes(g, nrhs);
-  if (cudaMalloc(&c->mem, lb + 2 * fb) != cudaSuccess) {
+  if (cudaMalloc(&c->mem, lb + vectors * fb) != cudaSuccess) {
     cudaGetLastError();
     c->mem = nullptr;
     return;
   }
   c->u = fx_links_at(g, c->mem);
   c->e0 = fx_field_at(g, nrhs, (char*)c->mem + lb);
-  c->e1 = fx_field_at(g, nrhs, (char*)c->mem + lb + fb);
+  if (vectors > 1) c->e1 = fx_field_at(g, nrhs, (char*)c->mem + lb + fb);
 }
 
 void fx_ctx_free(FxCtx* c) {

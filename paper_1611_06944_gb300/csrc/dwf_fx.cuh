@@ -113,15 +113,17 @@ int launch_fx_rb_m5inv(const Geom& g, const cpx<double>* in, cpx<double>* out64,
 int launch_fx_rb_p(const Geom& g, const cpx<double>* r, cpx<double>* p, const FxField& out, int par, const double* rr,
                    int k, cudaStream_t st);
 
-// What a solver keeps for FP64 applications of H on nrhs fields: the encoded links and two
-// encoded field vectors.  Without memory for it mem stays null and H runs on the FP64 pipe.
+// What a solver keeps for FP64 applications of H on nrhs fields: the encoded links, an encoded field
+// vector and, where encoded fields pass from one application to the next, a second one.  Without
+// memory for it mem stays null and H runs on the FP64 pipe.
 struct FxCtx {
   void* mem = nullptr;
   FxLinks u;
   FxField e0, e1;
 };
-// allocates (leaving mem null when the device is out of memory or fx_ok is false)
-void fx_ctx_alloc(FxCtx* c, const Geom& g, int nrhs);
+// allocates ``vectors`` (1: e0, 2: e0 and e1), leaving mem null when the device is out of memory or
+// fx_ok is false
+void fx_ctx_alloc(FxCtx* c, const Geom& g, int nrhs, int vectors);
 void fx_ctx_free(FxCtx* c);
 // encodes U, which must stay: before the first application of a solve
 int fx_ctx_links(FxCtx& c, const Geom& g, const cpx<double>* U, cudaStream_t st);

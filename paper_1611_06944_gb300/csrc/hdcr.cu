@@ -263,7 +263,7 @@ static int alloc_cache(const hdcr_coarse* co, int restart, SolveCache** out) {
     solve_cache_free(c);  // frees whatever part was allocated
     return s;
   }
-  if (!co->cf) fx_ctx_alloc(&c->fx, co->g, 1);
+  if (!co->cf) fx_ctx_alloc(&c->fx, co->g, 1, sizeof(R) == 8 ? 2 : 1);  // (FP32 V-cycle: the outer H alone)
   *out = c;
   return HDCR_OK;
 }

@@ -320,7 +320,7 @@ static int multi_alloc(const hdcr_coarse* co, int nrhs, int restart, MultiCache*
     multi_cache_free(c);
     return s;
   }
-  fx_ctx_alloc(&c->fx, co->g, nrhs);
+  fx_ctx_alloc(&c->fx, co->g, nrhs, sizeof(R) == 8 ? 2 : 1);  // (FP32 V-cycle: the outer H alone)
   *out = c;
   return HDCR_OK;
 }

@@ -291,7 +291,7 @@ static int rb_solve_impl(const Geom& g, const hdcr_dwf_params* prm, const cpx<do
     return s;
   }
   FxCtx fx;  // the iterations' hops in fixed point; without memory for it they run on the FP64 pipe
-  fx_ctx_alloc(&fx, g, 1);
+  fx_ctx_alloc(&fx, g, 1, 2);
   RBOp S{g, 5.0 - prm->M5, prm->mf, U, &w};
   RBDev* d = w.dev();
   RedScratch rs = w.rb.rs;

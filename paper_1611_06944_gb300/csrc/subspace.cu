@@ -531,7 +531,7 @@ static int filter_all_cheb(const Geom& g, const hdcr_dwf_params* p, const void* 
   int s = red_buffers_alloc(&rb, 2);
   FineOp<R> H{g, p->M5, p->mf, Ur};
   FxCtx fx;
-  if (f64) fx_ctx_alloc(&fx, g, half);
+  if (f64) fx_ctx_alloc(&fx, g, half, 2);
   H.fx = &fx;
   if (s == HDCR_OK) s = fx_ctx_links(fx, g, (const cpx<double>*)U, st);
   if (s == HDCR_OK) s = launch_convert(noise, HDCR_C128, x, f64 ? HDCR_C128 : HDCR_C64, fs * half, st);

@@ -123,3 +123,30 @@ def test_multi_rejects_unsupported(hd):
     s = hd._L.hdcr_solve_multi(co.handle, U.data_ptr(), B.data_ptr(), X.data_ptr(), 65, hd.C_ref(prm), 1, st,
                                torch.cuda.current_stream().cuda_stream)
     assert s == -1
+
+
+@pytest.mark.parametrize("tdt", ["c64", "c128"])
+def test_multi_workspace_holds_no_unused_field(hd, tdt):
+    """What a batched solve keeps with the coarse operator: beside its own fields the encoded operand of the
+    outer FP64 application, and a second encoded field only where the V-cycle is FP64 too."""
+    L, Ls, block, nvec, nrhs, restart = (8, 8, 8, 8), 8, (4, 4, 4, 4), 8, 12, 2
+    tdt = torch.complex64 if tdt == "c64" else torch.complex128
+    lat, Uh, U, sub, co = _setup(hd, L, Ls, block, nvec, 0.1, tdt, seed=1040, order=8, lam_cut=0.5)
+    hd.coarse_invert(co)
+    B = dev(planes(synth.gaussian_fermion(L, Ls, 2040, count=nrhs)))
+    kw = dict(tol=1e-1, inner_dtype=tdt, restart=restart, max_outer=200)
+    hd.hdcr_solve_multi(co, U, B, **kw)  # library handles and the like
+    co = hd.build_coarse_op(sub, U, M5, 0.1, op_dtype=tdt)
+    hd.coarse_invert(co)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    X = torch.zeros_like(B)
+    free = torch.cuda.mem_get_info()[0]
+    hd.hdcr_solve_multi(co, U, B, x0=X, **kw)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    used = free - torch.cuda.mem_get_info()[0]
+    f64, inner = 12 * lat.V5 * nrhs * 16, 12 * lat.V5 * nrhs * (8 if tdt == torch.complex64 else 16)
+    encoded = f64 * 196 // 192 * (1 if tdt == torch.complex64 else 2)
+    # 2 restart + 2 outer fields, 9 of the V-cycle; a quarter of a field for what is smaller than that
+    assert used <= (2 * restart + 2) * f64 + 9 * inner + encoded + f64 // 4
