@@ -219,33 +219,37 @@ static int alloc_cache(const hdcr_coarse* co, int restart, SolveCache** out) {
   c->fs = co->g.V5 * 12;
   c->cs = (long long)co->bg.Vc * co->nvec;
   const size_t f64 = sizeof(cpx<double>) * c->fs, fin = sizeof(cpx<R>) * c->fs, cin = sizeof(cpx<R>) * c->cs;
-  const size_t bytes = f64 * (2 * restart + 2) + fin * 5 + cin * 2 + sizeof(cpx<R>) * (size_t)co->g.V4 * 36 +
-                       sizeof(double) * restart * (2 * restart + 5) + 2048;
+  // the fields' places, laid out twice: for their total size (base null), then in the memory
+  auto lay_out = [&](char* base) {
+    size_t at = 0;
+    auto take = [&](size_t b) {
+      void* q = base + at;
+      at += (b + 255) & ~(size_t)255;
+      return q;
+    };
+    c->Z = (cpx<double>*)take(f64 * restart);
+    c->W = (cpx<double>*)take(f64 * restart);
+    c->r = (cpx<double>*)take(f64);
+    c->tmp = (cpx<double>*)take(f64);
+    c->r_in = take(fin);
+    c->z_in = take(fin);
+    c->t1 = take(fin);
+    c->t2 = take(fin);
+    c->e = take(fin);
+    c->c_rhs = take(cin);
+    c->c_sol = take(cin);
+    c->U_in = take(sizeof(cpx<R>) * (size_t)co->g.V4 * 36);
+    c->B = (double*)take(sizeof(double) * restart * (2 * restart + 5));
+    return at;
+  };
+  const size_t bytes = lay_out(nullptr);
   cudaError_t e = cudaMalloc(&c->mem, bytes);
   if (e != cudaSuccess) {
     delete c;
     set_error("HDCR workspace: cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
     return HDCR_ERR_NO_MEMORY;
   }
-  char* p = (char*)c->mem;
-  auto take = [&](size_t b) {
-    void* q = p;
-    p += (b + 255) & ~(size_t)255;
-    return q;
-  };
-  c->Z = (cpx<double>*)take(f64 * restart);
-  c->W = (cpx<double>*)take(f64 * restart);
-  c->r = (cpx<double>*)take(f64);
-  c->tmp = (cpx<double>*)take(f64);
-  c->r_in = take(fin);
-  c->z_in = take(fin);
-  c->t1 = take(fin);
-  c->t2 = take(fin);
-  c->e = take(fin);
-  c->c_rhs = take(cin);
-  c->c_sol = take(cin);
-  c->U_in = take(sizeof(cpx<R>) * (size_t)co->g.V4 * 36);
-  c->B = (double*)take(sizeof(double) * restart * (2 * restart + 5));
+  lay_out((char*)c->mem);
   int s = red_buffers_alloc(&c->rb, 192);
   CRWork<R>* sw = new CRWork<R>();
   CRWork<R>* cw = new CRWork<R>();

@@ -329,3 +329,23 @@ def test_hdcr_needs_fewer_fine_matvecs_than_cr(hd, L, Ls, block, nvec, lam_cut, 
     print(f"{L} x {Ls}: HDCR {st['iters']} outer iterations, {mv} applications of H; plain CR {st_cr['fine_matvecs']}")
     assert st["status"] == 0 and st["true_resid"] <= 1e-10
     assert mv < st_cr["fine_matvecs"]
+
+
+@pytest.mark.parametrize("inner", ["c128", "c64"])
+def test_hdcr_solve_on_odd_extents(hd, inner):
+    """9^4 x 3 with blocks of 3: fields whose sizes are no multiple of 256 bytes (V5 = 3 mod 8), which the
+    solve's workspace pads one by one."""
+    L, Ls, block, mf = (9, 9, 9, 9), 3, (3, 3, 3, 3), 0.3
+    tdt = torch.complex128 if inner == "c128" else torch.complex64
+    lat = hd.Lattice(L, Ls)
+    U = synth.gauge_field(L, 0.3, 3900)
+    Ud = dev(links(U))
+    sub = hd.build_subspace(lat, Ud, dev(planes(synth.gaussian_fermion(L, Ls, 3901, count=2))), M5, mf, block, order=30,
+                            lam_cut=0.5, store_dtype=tdt)
+    co = hd.build_coarse_op(sub, Ud, M5, mf, op_dtype=tdt)
+    hd.coarse_invert(co)
+    b = synth.gaussian_fermion(L, Ls, 3902)
+    for restart in (1, 3):
+        x, st = hd.hdcr_solve(co, Ud, dev(planes(b)), tol=1e-8, max_outer=500, restart=restart, inner_dtype=tdt)
+        r = b - dwf.apply_H(U, natural(host(x), L, Ls), M5, mf)
+        assert np.sqrt(dwf.norm2(r) / dwf.norm2(b)) <= 1.01e-8
