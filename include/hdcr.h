@@ -306,7 +306,8 @@ int hdcr_cgne_rb_solve(const hdcr_geom* g, const hdcr_dwf_params* p, const void*
  *      k = 0..nvec-1 (FP64), so that P_S of Eq. 4.3 is a projector.
  * The basis is stored in ``store_dtype`` (with C128 a fixed-point copy of the same size is kept
  * beside it for hdcr_restrict and hdcr_prolong where it takes at most a quarter of the
- * free device memory).  U is C128.  Every L[mu] must be a
+ * free device memory; an allocation of the library's that fails takes it back, unless a captured
+ * graph reads it, and both run on the FP64 pipe from then on).  U is C128.  Every L[mu] must be a
  * multiple of block[mu] with L[mu]/block[mu] >= 2; nvec even, 2..256.
  * Errors: BAD_ARG, BAD_GEOMETRY, RANK_DEFICIENT (a vector has nothing left
  * after orthogonalisation: |v| < 1e-12 |v0|), CUDA, NO_MEMORY.

@@ -10,7 +10,7 @@ namespace hdcr {
 int red_buffers_alloc(RedBuffers* rb, int nscal) {
   const size_t bytes = sizeof(double) * (RED_MAX_BLOCKS * RED_MAX_NV + nscal) + 256;
   void* p = nullptr;
-  cudaError_t e = cudaMalloc(&p, bytes);
+  cudaError_t e = dev_malloc(&p, bytes);
   if (e != cudaSuccess) {
     set_error("reduction scratch: cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
     return HDCR_ERR_NO_MEMORY;

@@ -92,7 +92,7 @@ __global__ void rescale2_kernel(cpx<R>* __restrict__ u, cpx<R>* __restrict__ v, 
 template <typename R>
 int cheb_work_alloc(ChebWork<R>* w, long long n) {
   void* p = nullptr;
-  cudaError_t e = cudaMalloc(&p, sizeof(cpx<R>) * n * 4 + 256);
+  cudaError_t e = dev_malloc(&p, sizeof(cpx<R>) * n * 4 + 256);
   if (e != cudaSuccess) return cuda_status(e, "Chebyshev workspace");
   w->t0 = (cpx<R>*)p;
   w->t1 = w->t0 + n;

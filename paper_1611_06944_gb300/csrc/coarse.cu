@@ -627,7 +627,8 @@ int launch_restrict(const hdcr_subspace* sub, const cpx<R>* fine, cpx<R>* coarse
     return two ? restrict_launch<R, 2, RP_NR>(sub, fine, coarse, nrhs, st)
                : restrict_launch<R, 1, RP_NR>(sub, fine, coarse, nrhs, st);
   } else {
-    if (sub->fx && nrhs <= 65535) return launch_restrict_fx(sub, fine, coarse, nrhs, st);
+    std::shared_lock<std::shared_mutex> lock;
+    if (nrhs <= 65535 && subspace_fx_lock(sub, st, &lock)) return launch_restrict_fx(sub, fine, coarse, nrhs, st);
     return restrict_launch<R, 1, 1>(sub, fine, coarse, nrhs, st);  // bound by the FP64 pipe, not by the basis
   }
 }
@@ -654,7 +655,9 @@ int launch_prolong(const hdcr_subspace* sub, const cpx<R>* coarse, const cpx<R>*
     return two ? prolong_launch<R, 2, RP_NR>(sub, coarse, fine_in, fine, nrhs, st)
                : prolong_launch<R, 1, RP_NR>(sub, coarse, fine_in, fine, nrhs, st);
   } else {
-    if (sub->fx && nrhs <= 65535) return launch_prolong_fx(sub, coarse, fine_in, fine, nrhs, st);
+    std::shared_lock<std::shared_mutex> lock;
+    if (nrhs <= 65535 && subspace_fx_lock(sub, st, &lock))
+      return launch_prolong_fx(sub, coarse, fine_in, fine, nrhs, st);
     return prolong_launch<R, 1, 1>(sub, coarse, fine_in, fine, nrhs, st);
   }
 }
@@ -869,7 +872,7 @@ static int build_coarse_op_entry(const hdcr_subspace* sub, const hdcr_dwf_params
     if (sub->build_ws) cudaFree(sub->build_ws);
     sub->build_ws = nullptr;
     sub->build_ws_bytes = 0;
-    HDCR_CUDA_TRY(cudaMalloc(&sub->build_ws, bytes));
+    HDCR_CUDA_TRY(dev_malloc(&sub->build_ws, bytes));
     sub->build_ws_bytes = bytes;
   }
   char* wp = (char*)sub->build_ws;
@@ -908,9 +911,9 @@ static int build_coarse_op_entry(const hdcr_subspace* sub, const hdcr_dwf_params
   co->mf = p->mf;
   cudaGetDevice(&co->device);
   int s = HDCR_OK;
-  cudaError_t e = cudaMalloc(&co->A, dtype_complex_bytes(co->dtype) * (size_t)bg.Vc * NLEGS * nvec * nvec);
+  cudaError_t e = dev_malloc(&co->A, dtype_complex_bytes(co->dtype) * (size_t)bg.Vc * NLEGS * nvec * nvec);
   if (!store_c128) A_build = co->A;
-  if (e == cudaSuccess) e = cudaMalloc(&co->nbr, sizeof(int) * bg.Vc * NLEGS);
+  if (e == cudaSuccess) e = dev_malloc(&co->nbr, sizeof(int) * bg.Vc * NLEGS);
   if (e != cudaSuccess) s = cuda_status(e, "coarse operator storage");
   if (s == HDCR_OK) s = fill_neighbour_table(bg, co->nbr, st);
   if (s == HDCR_OK) {

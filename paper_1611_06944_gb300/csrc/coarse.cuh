@@ -6,7 +6,9 @@
 // fine sites is contiguous in every plane).
 #pragma once
 
+#include <atomic>
 #include <mutex>
+#include <shared_mutex>
 
 #include "krylov.cuh"
 
@@ -63,9 +65,12 @@ struct hdcr_subspace {
   void* vecs;     // nvec fields, plane layout, block-orthonormal
   int device;
   // FP64 basis in fixed point for the restriction and prolongation (transfer_fx.cu), made with the
-  // subspace where it takes at most a quarter of the free device memory; else null, and
-  // they run on the FP64 pipe
+  // subspace where it takes at most a quarter of the free device memory; else, or once dev_malloc
+  // has given it back, null, and they run on the FP64 pipe.  Launches that read it hold fx_mu shared;
+  // one in a captured graph keeps it for good.
   void* fx = nullptr;
+  mutable std::shared_mutex fx_mu;
+  mutable std::atomic<bool> fx_captured{false};
   // scratch of hdcr_build_coarse_op, kept for the next build from this basis (a
   // rebuild after a gauge update needs no allocation); builds from one subspace
   // are serialised on build_mu
@@ -106,8 +111,11 @@ int launch_restrict(const hdcr_subspace* sub, const cpx<R>* fine, cpx<R>* coarse
 template <typename R>
 int launch_prolong(const hdcr_subspace* sub, const cpx<R>* coarse, const cpx<R>* fine_in, cpx<R>* fine,
                    int nrhs, cudaStream_t st);
-// the same in FP64 from the fixed-point basis sub->fx; subspace_encode makes it
+// the same in FP64 from the fixed-point basis sub->fx; subspace_encode makes it, subspace_fx_free ends it
 int subspace_encode(hdcr_subspace* sub, cudaStream_t st);
+void subspace_fx_free(hdcr_subspace* sub);
+// whether there is one for a launch on st, which is then locked until the lock ends
+bool subspace_fx_lock(const hdcr_subspace* sub, cudaStream_t st, std::shared_lock<std::shared_mutex>* lock);
 int launch_restrict_fx(const hdcr_subspace* sub, const cpx<double>* fine, cpx<double>* coarse, int nrhs,
                        cudaStream_t st);
 int launch_prolong_fx(const hdcr_subspace* sub, const cpx<double>* coarse, const cpx<double>* fine_in,

@@ -374,7 +374,7 @@ int dense_solve_prepare(hdcr_coarse* co, int nrhs) {
   if (co->dws) cudaFree(co->dws);
   co->dws = nullptr;
   co->dws_bytes = 0;
-  HDCR_CUDA_TRY(cudaMalloc(&co->dws, need));
+  HDCR_CUDA_TRY(dev_malloc(&co->dws, need));
   co->dws_bytes = need;
   return HDCR_OK;
 }
@@ -425,11 +425,11 @@ int coarse_invert(hdcr_coarse* co, cudaStream_t st) {
   const size_t mbytes = sizeof(cpx<float>) * (size_t)n * n;
   void* M = nullptr;
   void* aux = nullptr;
-  HDCR_CUDA_TRY(cudaMalloc(&M, mbytes + sizeof(int) * (size_t)n));
+  HDCR_CUDA_TRY(dev_malloc(&M, mbytes + sizeof(int) * (size_t)n));
   const long long na = (long long)Vc * NLEGS * nvec * nvec;
   const size_t abytes = sizeof(cpx<float>) * (size_t)(11 * n * GJ_P + na) +
                         sizeof(float) * GJ_MAX_CTAS + sizeof(int) * (size_t)(GJ_MAX_CTAS + n + 5) + 256;
-  cudaError_t e = cudaMalloc(&aux, abytes);
+  cudaError_t e = dev_malloc(&aux, abytes);
   if (e != cudaSuccess) {
     cudaFree(M);
     return cuda_status(e, "dense coarse inverse workspace");

@@ -38,7 +38,7 @@ int handle_of(cublasHandle_t* h) {
     cublasStatus_t s = cublasCreate(&hh);
     if (s != CUBLAS_STATUS_SUCCESS) return blas_status(s, "cublasCreate");
     void* ws = nullptr;
-    cudaError_t e = cudaMalloc(&ws, WS_BYTES);
+    cudaError_t e = dev_malloc(&ws, WS_BYTES);
     if (e != cudaSuccess) {
       cublasDestroy(hh);
       return cuda_status(e, "cuBLAS workspace");

@@ -171,7 +171,7 @@ template <typename R>
 int crwork_alloc(CRWork<R>* w, long long n) {
   void* p = nullptr;
   const size_t bytes = sizeof(cpx<R>) * (size_t)n * 4;
-  cudaError_t e = cudaMalloc(&p, bytes);
+  cudaError_t e = dev_malloc(&p, bytes);
   if (e != cudaSuccess) {
     set_error("CR workspace: cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
     return HDCR_ERR_NO_MEMORY;

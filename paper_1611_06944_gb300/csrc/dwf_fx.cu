@@ -984,7 +984,7 @@ void fx_ctx_alloc(FxCtx* c, const Geom& g, int nrhs, int vectors) {
   *c = FxCtx();
   if (!fx_ok(g)) return;
   const size_t lb = fx_links_bytes(g), fb = fx_field_bytes(g, nrhs);
-  if (cudaMalloc(&c->mem, lb + vectors * fb) != cudaSuccess) {
+  if (dev_malloc(&c->mem, lb + vectors * fb) != cudaSuccess) {
     cudaGetLastError();
     c->mem = nullptr;
     return;

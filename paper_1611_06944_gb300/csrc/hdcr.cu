@@ -243,7 +243,7 @@ static int alloc_cache(const hdcr_coarse* co, int restart, SolveCache** out) {
     return at;
   };
   const size_t bytes = lay_out(nullptr);
-  cudaError_t e = cudaMalloc(&c->mem, bytes);
+  cudaError_t e = dev_malloc(&c->mem, bytes);
   if (e != cudaSuccess) {
     delete c;
     set_error("HDCR workspace: cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));

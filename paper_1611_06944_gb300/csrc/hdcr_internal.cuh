@@ -142,4 +142,15 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 
 size_t dtype_complex_bytes(int dtype);
 
+// cudaMalloc for everything that the library allocates: when the device is out of memory, fixed-point copies of
+// bases (transfer_fx.cu), which are not needed, are given back one by one
+cudaError_t dev_malloc_bytes(void** p, size_t bytes);
+template <typename T>
+cudaError_t dev_malloc(T** p, size_t bytes) {
+  void* q = nullptr;
+  const cudaError_t e = dev_malloc_bytes(&q, bytes);
+  if (e == cudaSuccess) *p = (T*)q;
+  return e;
+}
+
 }  // namespace hdcr

@@ -281,7 +281,7 @@ static int multi_alloc(const hdcr_coarse* co, int nrhs, int restart, MultiCache*
   const size_t bytes = f64 * (2 * (size_t)restart + 2) + fin * 5 + cin * 2 + sizeof(cpx<R>) * (size_t)co->g.V4 * 36 +
                        sizeof(double) * (size_t)(nrhs * c->SC + 4 * nrhs) + 2 * sizeof(double2) * nrhs * MB_BLOCKS +
                        16 * 256;
-  cudaError_t e = cudaMalloc(&c->mem, bytes);
+  cudaError_t e = dev_malloc(&c->mem, bytes);
   if (e != cudaSuccess) {
     delete c;
     set_error("multi-RHS HDCR workspace: cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));

@@ -389,13 +389,13 @@ int build_impl(hdcr_coarse* co, const hdcr_level2_params* p, const void* noise, 
   cpx<R>* s = nullptr;
   cpx<R>* zero = nullptr;
   cpx<double>* phi = nullptr;
-  HDCR_CUDA_TRY(cudaMalloc(&s, sizeof(cpx<R>) * (size_t)(h * cs + cs)));
+  HDCR_CUDA_TRY(dev_malloc(&s, sizeof(cpx<R>) * (size_t)(h * cs + cs)));
   zero = s + h * cs;
   int status = HDCR_OK;
   auto fail = [&](int st_) {
     if (status == HDCR_OK) status = st_;
   };
-  if (cudaMalloc(&phi, sizeof(cpx<double>) * (size_t)(n2 * cs)) != cudaSuccess) fail(HDCR_ERR_NO_MEMORY);
+  if (dev_malloc(&phi, sizeof(cpx<double>) * (size_t)(n2 * cs)) != cudaSuccess) fail(HDCR_ERR_NO_MEMORY);
   if (status == HDCR_OK && cudaMemsetAsync(zero, 0, sizeof(cpx<R>) * cs, st) != cudaSuccess) fail(HDCR_ERR_CUDA);
   CRWork<R>* cw = (CRWork<R>*)l->crw;
   if (status == HDCR_OK) {
@@ -503,10 +503,10 @@ int level2_build(hdcr_coarse* co, const hdcr_level2_params* p, const void* noise
   c2->M5 = co->M5;
   c2->mf = co->mf;
   c2->device = co->device;
-  if (cudaMalloc(&c2->A, cb * (size_t)q.Vc2 * NLEGS * n2 * n2) != cudaSuccess ||
-      cudaMalloc(&c2->nbr, sizeof(int) * (size_t)q.Vc2 * NLEGS) != cudaSuccess ||
-      cudaMalloc(&l->phi2, cb * (size_t)n2 * cs) != cudaSuccess ||
-      cudaMalloc(&l->ws, cb * (size_t)((2 * L2_RESTART + 4) * cs + 2 * (long long)q.Vc2 * n2)) != cudaSuccess) {
+  if (dev_malloc(&c2->A, cb * (size_t)q.Vc2 * NLEGS * n2 * n2) != cudaSuccess ||
+      dev_malloc(&c2->nbr, sizeof(int) * (size_t)q.Vc2 * NLEGS) != cudaSuccess ||
+      dev_malloc(&l->phi2, cb * (size_t)n2 * cs) != cudaSuccess ||
+      dev_malloc(&l->ws, cb * (size_t)((2 * L2_RESTART + 4) * cs + 2 * (long long)q.Vc2 * n2)) != cudaSuccess) {
     cudaGetLastError();
     s = HDCR_ERR_NO_MEMORY;
     set_error("hdcr_coarse_build_level2: out of device memory");

@@ -340,9 +340,9 @@ static int cf_build_impl(const hdcr_subspace* sub, double M5, const CFCoef& cf, 
   cpx<double>* Y = nullptr;
   int s = HDCR_OK;
   const size_t abytes = sizeof(cpx<double>) * (size_t)bg.Vc * NLEGS * nvec * nvec;
-  cudaError_t e = cudaMalloc(&co->A, abytes);
-  if (e == cudaSuccess) e = cudaMalloc(&co->nbr, sizeof(int) * bg.Vc * NLEGS);
-  if (e == cudaSuccess) e = cudaMalloc(&Y, sizeof(cpx<double>) * fs);
+  cudaError_t e = dev_malloc(&co->A, abytes);
+  if (e == cudaSuccess) e = dev_malloc(&co->nbr, sizeof(int) * bg.Vc * NLEGS);
+  if (e == cudaSuccess) e = dev_malloc(&Y, sizeof(cpx<double>) * fs);
   if (e == cudaSuccess) e = cudaMemsetAsync(co->A, 0, abytes, st);
   if (e != cudaSuccess) s = cuda_status(e, "continued-fraction coarse operator storage");
   if (s == HDCR_OK) s = fill_neighbour_table(bg, co->nbr, st);
@@ -384,7 +384,7 @@ static int cf_filter_impl(const Geom& g, double M5, const CFCoef& cf, const void
     CRWork<R> w;
     HDCR_TRY(crwork_alloc<R>(&w, n));
     cpx<R>* zero = nullptr;
-    cudaError_t e = cudaMalloc(&zero, sizeof(cpx<R>) * n);
+    cudaError_t e = dev_malloc(&zero, sizeof(cpx<R>) * n);
     if (e == cudaSuccess) e = cudaMemsetAsync(zero, 0, sizeof(cpx<R>) * n, st);
     if (e != cudaSuccess) s = cuda_status(e, "continued-fraction filter workspace");
     CRConfig cfg;

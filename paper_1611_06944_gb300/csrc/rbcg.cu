@@ -281,7 +281,7 @@ static int rb_solve_impl(const Geom& g, const hdcr_dwf_params* prm, const cpx<do
   }
   RBWork w;
   const size_t fb = sizeof(cpx<double>) * (size_t)n;
-  HDCR_CUDA_TRY(cudaMalloc(&w.mem, fb * 11));
+  HDCR_CUDA_TRY(dev_malloc(&w.mem, fb * 11));
   cpx<double>* base = (cpx<double>*)w.mem;
   cpx<double>** slots[11] = {&w.eta, &w.a, &w.b2, &w.xo, &w.t, &w.r, &w.p, &w.q, &w.Ap, &w.g1, &w.g2};
   for (int i = 0; i < 11; ++i) *slots[i] = base + (size_t)i * n;

@@ -417,7 +417,7 @@ static int cholesky_qr2(const Geom& g, const BlockGeom& bg, cpx<double>* vecs, i
 static int orthonormalise_and_store(const Geom& g, const BlockGeom& bg, cpx<double>* vecs, int nvec,
                                     int store_dtype, cudaStream_t st, hdcr_subspace** out) {
   int* dstatus = nullptr;
-  cudaError_t e0 = cudaMalloc(&dstatus, sizeof(int));
+  cudaError_t e0 = dev_malloc(&dstatus, sizeof(int));
   if (e0 != cudaSuccess) {
     cudaFree(vecs);
     return cuda_status(e0, "subspace status flag");
@@ -470,7 +470,7 @@ static int orthonormalise_and_store(const Geom& g, const BlockGeom& bg, cpx<doub
     }
   } else {
     void* p = nullptr;
-    e = cudaMalloc(&p, n * sizeof(cpx<float>));
+    e = dev_malloc(&p, n * sizeof(cpx<float>));
     if (e != cudaSuccess) {
       cudaFree(vecs);
       delete sub;
@@ -517,7 +517,7 @@ static int filter_all_cheb(const Geom& g, const hdcr_dwf_params* p, const void* 
   const size_t bytes = sizeof(cpx<R>) * fs * half * 5 + sizeof(cpx<double>) * fs +
                        (f64 ? 0 : sizeof(cpx<R>) * g.V4 * 36) + 1024;
   void* mem = nullptr;
-  HDCR_CUDA_TRY(cudaMalloc(&mem, bytes));
+  HDCR_CUDA_TRY(dev_malloc(&mem, bytes));
   cpx<R>* x = (cpx<R>*)mem;
   cpx<R>* work = x + fs * half;
   cpx<double>* x64 = (cpx<double>*)(work + 4 * fs * half);
@@ -562,7 +562,7 @@ static int filter_all(const Geom& g, const hdcr_dwf_params* p, const void* U, co
   // x (R), zero (R), x64 scratch, U in R
   const size_t bytes = sizeof(cpx<R>) * fs * 2 + sizeof(cpx<double>) * fs + (f64 ? 0 : sizeof(cpx<R>) * g.V4 * 36) + 512;
   void* mem = nullptr;
-  HDCR_CUDA_TRY(cudaMalloc(&mem, bytes));
+  HDCR_CUDA_TRY(dev_malloc(&mem, bytes));
   cpx<R>* x = (cpx<R>*)mem;
   cpx<R>* zero = x + fs;
   cpx<double>* x64 = (cpx<double>*)(zero + fs);
@@ -603,7 +603,7 @@ static int build_subspace_impl(const Geom& g, const BlockGeom& bg, const hdcr_dw
                                hdcr_subspace** out) {
   const long long fs = g.V5 * 12;
   cpx<double>* vecs = nullptr;
-  HDCR_CUDA_TRY(cudaMalloc(&vecs, sizeof(cpx<double>) * fs * sp->nvec));
+  HDCR_CUDA_TRY(dev_malloc(&vecs, sizeof(cpx<double>) * fs * sp->nvec));
   int s;
   if (sp->kind == HDCR_SUBSPACE_CHEBYSHEV)
     s = sp->filter_dtype == HDCR_C128 ? filter_all_cheb<double>(g, p, U, noise, sp, vecs, st)
@@ -679,7 +679,7 @@ extern "C" int hdcr_subspace_from_vectors(const hdcr_geom* gp, const int block[4
   cudaStream_t st = as_stream(stream);
   const long long n = (long long)nvec * g.V5 * 12;
   cpx<double>* vecs = nullptr;
-  HDCR_CUDA_TRY(cudaMalloc(&vecs, sizeof(cpx<double>) * n));
+  HDCR_CUDA_TRY(dev_malloc(&vecs, sizeof(cpx<double>) * n));
   cudaMemcpyAsync(vecs, vectors, sizeof(cpx<double>) * n, cudaMemcpyDeviceToDevice, st);
   return orthonormalise_and_store(g, bg, vecs, nvec, store_dtype, st, out);
 }
@@ -706,7 +706,7 @@ extern "C" int hdcr_subspace_get_vectors(const hdcr_subspace* sub, void* out, vo
 extern "C" void hdcr_subspace_destroy(hdcr_subspace* sub) {
   if (!sub) return;
   if (sub->vecs) cudaFree(sub->vecs);
-  if (sub->fx) cudaFree(sub->fx);
+  subspace_fx_free(sub);
   if (sub->build_ws) cudaFree(sub->build_ws);
   delete sub;
 }

@@ -18,6 +18,9 @@
 #include <cooperative_groups.h>
 #include <math.h>
 
+#include <algorithm>
+#include <vector>
+
 #include "coarse.cuh"
 #include "fx_device.cuh"
 
@@ -333,6 +336,10 @@ static FxField basis_field(const hdcr_subspace* sub) {
   return f;
 }
 
+// the subspaces that have one
+static std::mutex g_fx_mu;
+static std::vector<hdcr_subspace*> g_fx_subs;
+
 int subspace_encode(hdcr_subspace* sub, cudaStream_t st) {
   const size_t n = (size_t)sub->nvec * sub->g.V5, bytes = n * 12 * sizeof(int4) + n * sizeof(int);
   size_t free_bytes = 0, total = 0;
@@ -347,7 +354,58 @@ int subspace_encode(hdcr_subspace* sub, cudaStream_t st) {
   count_launch();
   HDCR_LAUNCH_CHECK();
   HDCR_CUDA_TRY(cudaStreamSynchronize(st));
+  std::lock_guard<std::mutex> lock(g_fx_mu);
+  g_fx_subs.push_back(sub);
   return HDCR_OK;
+}
+
+void subspace_fx_free(hdcr_subspace* sub) {
+  std::lock_guard<std::mutex> lock(g_fx_mu);
+  g_fx_subs.erase(std::remove(g_fx_subs.begin(), g_fx_subs.end(), sub), g_fx_subs.end());
+  if (sub->fx) cudaFree(sub->fx);
+  sub->fx = nullptr;
+}
+
+bool subspace_fx_lock(const hdcr_subspace* sub, cudaStream_t st, std::shared_lock<std::shared_mutex>* lock) {
+  *lock = std::shared_lock<std::shared_mutex>(sub->fx_mu);
+  if (!sub->fx) {
+    lock->unlock();
+    return false;
+  }
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {
+    cudaGetLastError();
+    sub->fx_captured = true;
+  } else if (status != cudaStreamCaptureStatusNone) {
+    sub->fx_captured = true;
+  }
+  return true;
+}
+
+// gives back one copy on the current device that no captured graph reads, its launches done
+static bool give_back_one() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::lock_guard<std::mutex> lock(g_fx_mu);
+  for (size_t i = 0; i < g_fx_subs.size(); ++i) {
+    hdcr_subspace* sub = g_fx_subs[i];
+    std::unique_lock<std::shared_mutex> own(sub->fx_mu);
+    if (sub->device != dev || sub->fx_captured) continue;
+    if (cudaDeviceSynchronize() != cudaSuccess || cudaFree(sub->fx) != cudaSuccess) return false;
+    sub->fx = nullptr;
+    g_fx_subs.erase(g_fx_subs.begin() + i);
+    return true;
+  }
+  return false;
+}
+
+cudaError_t dev_malloc_bytes(void** p, size_t bytes) {
+  for (;;) {
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    if (!give_back_one()) return e;
+  }
 }
 
 int launch_restrict_fx(const hdcr_subspace* sub, const cpx<double>* fine, cpx<double>* coarse, int nrhs,

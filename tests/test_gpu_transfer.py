@@ -190,3 +190,42 @@ def test_block_orthonormalisation_of_vectors_at_opposite_walls(hd, nvec):
     e = np.sqrt((np.abs((got - q).reshape(shape)) ** 2).sum((1, 2, 3)))
     w = np.sqrt((np.abs(q.reshape(shape)) ** 2).sum((1, 2, 3)))
     assert (e <= 1e-13 * w).all(), e / w
+
+
+def test_copy_of_the_basis_is_given_back(hd):
+    """With the device's memory nearly taken, a solve's workspace that does not fit beside the fixed-point
+    copies of two bases is allocated all the same, and what used a copy runs on without it."""
+    L, Ls, block, M5, mf = (16, 16, 8, 8), 8, (4, 4, 4, 4), 1.8, 0.3
+    lat = hd.Lattice(L, Ls)
+    U = dev(synth.gauge_field((4, 4, 4, 4), 0.3, 6500).reshape(4, -1, 3, 3))
+    U = U.repeat(1, lat.V4 // 256, 1, 1).contiguous()
+    gen = torch.Generator(device="cuda").manual_seed(6501)
+    noise = torch.randn(8, lat.V4, 12, Ls, generator=gen, device="cuda", dtype=torch.complex128)
+    b = noise[0].clone()
+    sub = hd.build_subspace(lat, U, noise[:4].contiguous(), M5, mf, block, order=60, lam_cut=0.5)
+    other = hd.subspace_from_vectors(lat, block, noise)
+    captured = hd.subspace_from_vectors(lat, block, noise)
+    del noise
+    co, again = hd.build_coarse_op(sub, U, M5, mf), hd.build_coarse_op(sub, U, M5, mf)
+    hd.coarse_invert(co)
+    hd.coarse_invert(again)
+    kw = dict(tol=1e-6, max_outer=300, inner_dtype=torch.complex128)
+    x0, _ = hd.hdcr_solve(co, U, b, restart=8, **kw)
+    c0 = hd.restrict(other, b)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):  # keeps its copy
+        out = hd.restrict(captured, b)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    field = 12 * lat.V5 * 16
+    # the workspace of restart 24 takes 55 fields in one piece and 11 more, a copy 8: all but 53 are taken
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - 53 * field, dtype=torch.uint8, device="cuda")
+    x, st = hd.hdcr_solve(again, U, b, restart=24, **kw)
+    assert st["true_resid"] <= 1e-6
+    assert float((x - x0).norm() / x0.norm()) <= 1e-4
+    c = hd.restrict(other, b)
+    assert float((c - c0).norm() / c0.norm()) <= 1e-14
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, c0)
+    del hold
