@@ -589,9 +589,9 @@ int restrict_cluster(long long ctas, long long rounds) {
 
 constexpr int RP_NR = 4;  // FP32 fields that share a pass over the basis
 
-// two FP32 elements a load: even Ls (elements of a site pair up) and 16-byte aligned fields
+// two FP32 elements a load: 16-byte aligned fields (a 4d site's 12 Ls elements pair up for every Ls)
 static bool rp_pairs(const hdcr_subspace* sub, const void* a, const void* b) {
-  return sub->g.Ls % 2 == 0 && ((((uintptr_t)sub->vecs) | ((uintptr_t)a) | ((uintptr_t)b)) & 15) == 0;
+  return ((((uintptr_t)sub->vecs) | ((uintptr_t)a) | ((uintptr_t)b)) & 15) == 0;
 }
 
 template <typename R, int V, int NR>

@@ -229,3 +229,26 @@ def test_copy_of_the_basis_is_given_back(hd):
     torch.cuda.synchronize()
     assert torch.equal(out, c0)
     del hold
+
+
+@pytest.mark.parametrize("Ls", [3, 4, 5])
+@pytest.mark.parametrize("nrhs", [1, 3])
+def test_fp32_transfer_of_unaligned_fields(hd, Ls, nrhs):
+    """A field 8 bytes off a 16-byte boundary is read one element a load: the same sums as the aligned copy's, which is
+    read in pairs of elements for odd Ls as for even, to their order."""
+    L, block = (4, 4, 4, 2), (2, 2, 2, 1)
+    lat = hd.Lattice(L, Ls)
+    sub = hd.subspace_from_vectors(lat, block, dev(planes(synth.gaussian_fermion(L, Ls, 6600, count=10))),
+                                   store_dtype=torch.complex64)
+    v = dev(planes(synth.gaussian_fermion(L, Ls, 6601, count=nrhs))).to(torch.complex64)
+    off = torch.empty(v.numel() + 1, dtype=torch.complex64, device="cuda")[1:].view(v.shape)
+    off.copy_(v)
+    assert v.data_ptr() % 16 == 0 and off.data_ptr() % 16 == 8
+    a, b = hd.restrict(sub, v), hd.restrict(sub, off)
+    phi = blocks(host(sub.vectors()), L, Ls, block)
+    want = np.stack([(np.conj(phi) * x).sum(-1).T for x in blocks(host(v), L, Ls, block)])
+    for c in (a, b):  # as in test_transfer_error
+        assert np.linalg.norm(host(c) - want) <= 2e-6 * np.linalg.norm(want)
+    f = blocks(host(hd.prolong(sub, a)), L, Ls, block)
+    wf = np.stack([(phi * x.T[:, :, None]).sum(0) for x in host(a)])
+    assert np.linalg.norm(f - wf) <= 2e-6 * np.linalg.norm(wf)
