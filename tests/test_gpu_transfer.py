@@ -252,3 +252,42 @@ def test_fp32_transfer_of_unaligned_fields(hd, Ls, nrhs):
     f = blocks(host(hd.prolong(sub, a)), L, Ls, block)
     wf = np.stack([(phi * x.T[:, :, None]).sum(0) for x in host(a)])
     assert np.linalg.norm(f - wf) <= 2e-6 * np.linalg.norm(wf)
+
+
+@pytest.mark.parametrize("value", [1e250, 1e-250, -3e-310])
+def test_results_beside_values_outside_the_format(hd, value):
+    """The blocks and elements that a value outside the format reaches, each on its own scale: what is
+    computed in FP64 there is the same sum, of the same terms."""
+    L, Ls, block = (4, 4, 2, 2), 4, (2, 2, 1, 1)
+    lat = hd.Lattice(L, Ls)
+    sub = hd.subspace_from_vectors(lat, block, dev(planes(synth.gaussian_fermion(L, Ls, 6400, count=6))))
+    phi = blocks(host(sub.vectors()), L, Ls, block).astype(np.clongdouble)  # (nvec, Vc, K)
+    v = host(dev(planes(synth.gaussian_fermion(L, Ls, 6401, count=1)))).copy()
+    v[0, 5, 3, 1] = value * (0.6 - 0.8j)
+    vb = blocks(v, L, Ls, block)[0].astype(np.clongdouble)
+    got = host(hd.restrict(sub, dev(v)))[0].T
+    want, terms = (np.conj(phi) * vb).sum(-1), (np.abs(phi) * np.abs(vb)).sum(-1)
+    # a block has 192 terms; each block and vector against its own (in extended precision, whose exponents hold them)
+    assert (np.abs(got - want) <= 1e-15 * terms).all()
+    c = host(hd.restrict(sub, dev(planes(synth.gaussian_fermion(L, Ls, 6402, count=1))))).copy()
+    c[0, 1, 2] = value * (0.6 - 0.8j)
+    got = blocks(host(hd.prolong(sub, dev(c))), L, Ls, block)[0]
+    cc = c[0].T[:, :, None].astype(np.clongdouble)
+    want, terms = (phi * cc).sum(0), (np.abs(phi) * np.abs(cc)).sum(0)
+    assert (np.abs(got - want) <= 1e-15 * terms).all()
+    # a basis vector with such a part, orthonormalised by itself
+    w = synth.gaussian_fermion(L, Ls, 6403, count=2)
+    w[..., 2, :, :] *= 1e-240
+    sub = hd.subspace_from_vectors(lat, block, dev(planes(w)))
+    phi = blocks(host(sub.vectors()), L, Ls, block).astype(np.clongdouble)
+    assert (np.abs(phi[:, :, 2]) < 1e-200).all()
+    vb = blocks(host(dev(planes(synth.gaussian_fermion(L, Ls, 6404, count=1)))), L, Ls, block)[0]
+    vb[:, np.arange(192) % Ls != 2] = 0  # a field that meets that part alone
+    n = np.zeros((1,) + vb.shape, dtype=np.complex128)
+    n[0] = vb
+    B, T = tuple(block[::-1]), tuple(L[::-1])
+    g = [t // b for t, b in zip(T, B)]
+    full = n.reshape(1, *g, *B, 12 * Ls).transpose(0, 1, 5, 2, 6, 3, 7, 4, 8, 9).reshape(1, lat.V4, 12, Ls)
+    got = host(hd.restrict(sub, dev(full)))[0].T
+    want, terms = (np.conj(phi) * vb).sum(-1), (np.abs(phi) * np.abs(vb)).sum(-1)
+    assert (np.abs(got - want) <= 1e-15 * terms + 1e-300).all()
