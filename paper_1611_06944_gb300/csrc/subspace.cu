@@ -5,11 +5,13 @@
 //   P_S = sum |phi_k^b><phi_k^b| (Eq. 4.3) is a projector (Cholesky QR twice,
 //   Gram-Schmidt for ill-conditioned blocks).
 // All of it runs in FP64; the basis is then stored in the requested dtype.
+#include <algorithm>
 #include <vector>
 
 #include "host_io.cuh"
 #include "chebyshev.cuh"
 #include "coarse.cuh"
+#include "fx_device.cuh"
 
 namespace hdcr {
 
@@ -166,6 +168,18 @@ constexpr int CQR_E = 96;         // elements (site x component) of a block per 
 constexpr int CQR_MAXV = 64;      // largest nvec handled (else Gram-Schmidt throughout)
 constexpr int CQR_TILES = 3;      // 2 x 2 Gram tiles per thread: (nvec/2)(nvec/2+1)/2 <= 3 * 256
 constexpr double CQR_TOL = 1e-8;
+constexpr int CQR_G = 16;         // elements that share an exponent in the fixed-point Gram kernel's chunk
+constexpr int CQR_GROUPS = CQR_E / CQR_G;
+constexpr int CQR_UP = 4;         // their numbers have at most 57 bits
+constexpr int CQR_EX_MIN = 400, CQR_EX_MAX = 1600;
+constexpr int CQR_BE_MIN = 70, CQR_BE_MAX = 2000;  // a sum's leading exponent, so that it stays a normal number
+// A group's sum of 32 real products errs by 0.56 of the integers' unit (the dropped L L' and the rounded cross
+// products), FP64 multiply-adds by 0.29 2^-53 of each of 32 partial sums.  So the integers are as good where the
+// partial sums after 4, 8, 12 and 16 elements, squared and added up over the groups, are 0.47 2^-20 of the
+// scales 2^63, squared and added up; Gaussian vectors have 6 times that, and 2.4 times where opposite
+// symmetry in the fifth dimension makes a group's sum vanish.
+constexpr float CQR_K2 = 0.47f * 0x1p-20f;
+constexpr int CQR_SPAN = 60;      // exponents above a thread's first group's that the sums of squares may hold
 
 // offset of element le of block a: elements ordered by the block's 4d sites, then
 // component and s, so one 4d site's 12 Ls elements are contiguous in the field
@@ -246,6 +260,178 @@ __global__ void __launch_bounds__(GS_THREADS) cqr_gram_kernel(Geom g, BlockGeom 
     P[(tj[i] + 1) * nvec + tk[i]] = cpx<double>(acc[i][4], acc[i][5]);
     P[(tj[i] + 1) * nvec + tk[i] + 1] = cpx<double>(acc[i][6], acc[i][7]);
   }
+}
+
+// The same in fixed point, for one tile a thread at most (nvec <= 44).  As FP64 multiply-adds it keeps
+// the FP64 pipe 0.79 busy: 42.4 ms a round at 16^4 x 16 with 24 vectors, 16.7 ms so.  The chunk is encoded on
+// its way to shared memory: groups of CQR_G elements of a vector share an exponent,
+// x = (2^30 H + L) 2^(ex - 1079), |H| <= 2^27, -2^29 <= L < 2^29, 57 bits below the group's
+// largest component.  A group's sum is exact in 64 bits up to the dropped L L' (H H' below
+// 2^59, the cross products below 2^62), three wide integer multiply-adds a real product, and groups are
+// added in FP64.  A pair of groups outside the format is summed in FP64 from the vectors, and so is
+// the whole of a tile with a real for which the sums of squares say that FP64 is more accurate:
+// vectors that are large where the others are small, bound to opposite walls for instance.  The groups of a
+// chunk are dealt to P sets of threads, whose sums are added in the sets' order.
+// Rows are CQR_E + 1 elements apart: the vectors of a warp's tiles then lie in different banks.
+__global__ void __launch_bounds__(GS_THREADS, 2) cqr_gram_fx_kernel(Geom g, BlockGeom bg,
+                                                                    const cpx<double>* __restrict__ vecs, int nvec,
+                                                                    int S, const int* __restrict__ skip,
+                                                                    cpx<double>* __restrict__ part) {
+  extern __shared__ int4 xe[];  // [nvec][CQR_E + 1], then the groups' exponents [nvec][CQR_GROUPS]
+  int* ex = reinterpret_cast<int*>(xe + nvec * (CQR_E + 1));
+  const int a = blockIdx.x, q = blockIdx.y;
+  if (skip[a]) return;
+  const long long fs = g.V5 * 12;
+  const long long ne = bg.K5 * 12;
+  const long long e0 = ne * q / S, e1 = ne * (q + 1) / S;
+  const int nt = nvec / 2, ntiles = nt * (nt + 1) / 2;
+  const int P = min(CQR_GROUPS, GS_THREADS / ntiles);
+  const int set = threadIdx.x / ntiles;  // P and above: threads without a tile
+  double A[8];
+  float sure[8];  // sum over the groups of (partial sums / 2^63)^2 - K2, in units of 4^ref
+  int ref = 0;    // 0: no group yet
+  int tj = -1, tk = -1;
+  if (set < P) cqr_tile((int)threadIdx.x - set * ntiles, nt, &tj, &tk);
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    A[m] = 0.0;
+    sure[m] = 0.f;
+  }
+  for (long long c0 = e0; c0 < e1; c0 += CQR_E) {
+    const int n = (int)(e1 - c0 < CQR_E ? e1 - c0 : CQR_E);
+    __syncthreads();
+    // nvec is even and CQR_E a multiple of 16: a half warp holds one group, and whole half
+    // warps leave the loop together
+    for (int i = threadIdx.x; i < nvec * CQR_E; i += GS_THREADS) {
+      const int k = i / CQR_E, e = i - k * CQR_E;
+      const cpx<double> x[1] = {e < n ? vecs[(long long)k * fs + cqr_off(g, bg, a, c0 + e)] : cpx<double>(0.0, 0.0)};
+      const unsigned half = 0xffffu << (threadIdx.x & 16);
+      unsigned top = fx_top(x), any = top & 0x80000000u;
+      top &= 0x7fffffffu;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) {
+        top = max(top, __shfl_xor_sync(half, top, o));
+        any |= __shfl_xor_sync(half, any, o);
+      }
+      const int m = fx_mark(top | any, CQR_EX_MIN, CQR_EX_MAX);
+      xe[k * (CQR_E + 1) + e] = fx_encode(x[0], m, CQR_UP);
+      if (e % CQR_G == 0) ex[k * CQR_GROUPS + e / CQR_G] = m;
+    }
+    __syncthreads();
+    if (tj < 0) continue;
+    for (int b = set; b * CQR_G < n; b += P) {
+      const int ej[2] = {ex[tj * CQR_GROUPS + b], ex[(tj + 1) * CQR_GROUPS + b]};
+      const int ek[2] = {ex[tk * CQR_GROUPS + b], ex[(tk + 1) * CQR_GROUPS + b]};
+      const int4* x0 = xe + tj * (CQR_E + 1) + b * CQR_G;
+      const int4* y0 = xe + tk * (CQR_E + 1) + b * CQR_G;
+      // 4^(be - ref) of each product, infinite above CQR_SPAN (then the tile is not certain), 0 where the
+      // integers are not used
+      float f2[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const int p = ej[m >> 1], r = ek[m & 1];
+        const int be = p + r - 1012;  // both scaled by 2^-1049 (H), a leading bit 63
+        f2[m] = 0.f;
+        if (p == 0 || r == 0 || p == FX_RAW || r == FX_RAW || be < CQR_BE_MIN || be > CQR_BE_MAX) continue;
+        if (ref == 0) ref = be;
+        const int d = be - ref;
+        f2[m] = __int_as_float(d > CQR_SPAN ? 0x7f800000 : (127 + 2 * max(d, -CQR_SPAN)) << 23);
+      }
+      i64 h[8], l[8];
+#pragma unroll
+      for (int m = 0; m < 8; ++m) h[m] = 0, l[m] = 1LL << 29;
+#pragma unroll 1
+      for (int e4 = 0; e4 < CQR_G; e4 += 4) {
+#pragma unroll 2
+        for (int e = e4; e < e4 + 4; ++e) {
+          const int4 u[2] = {x0[e], x0[e + CQR_E + 1]}, w[2] = {y0[e], y0[e + CQR_E + 1]};
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            const int4 p = u[m >> 1], r = w[m & 1];  // conj(p) r
+            const int nz = -p.z, nw = -p.w;
+            h[2 * m] = mw(p.z, r.z, mw(p.x, r.x, h[2 * m]));
+            h[2 * m + 1] = mw(nz, r.x, mw(p.x, r.z, h[2 * m + 1]));
+            l[2 * m] = mw(p.w, r.z, mw(p.z, r.w, mw(p.y, r.x, mw(p.x, r.y, l[2 * m]))));
+            l[2 * m + 1] = mw(nw, r.x, mw(nz, r.y, mw(p.y, r.z, mw(p.x, r.w, l[2 * m + 1]))));
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float x = (float)(int)(h[i] >> 32) * 0x1p-31f;
+          sure[i] = fmaf(f2[i >> 1], x * x, sure[i]);
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const int p = ej[m >> 1], r = ek[m & 1];
+        if (f2[m] != 0.f) {
+          const int be = p + r - 1012;
+#pragma unroll
+          for (int i = 2 * m; i < 2 * m + 2; ++i) {
+            if (h[i] == 0 && l[i] == 1LL << 29) continue;  // no products but zeros
+            A[i] += fx_to_double(h[i] + (l[i] >> 30), be);
+            sure[i] = fmaf(f2[m], -CQR_K2, sure[i]);
+          }
+          continue;
+        }
+        if ((p == 0 && r != FX_RAW) || (r == 0 && p != FX_RAW)) continue;
+        const cpx<double>* f = vecs + (long long)(tj + (m >> 1)) * fs;
+        const cpx<double>* s = vecs + (long long)(tk + (m & 1)) * fs;
+        for (int e = b * CQR_G; e < min(n, (b + 1) * CQR_G); ++e) {
+          const unsigned o = cqr_off(g, bg, a, c0 + e);
+          const cpx<double> u = f[o], w = s[o];
+          A[2 * m] = fma(u.re, w.re, fma(u.im, w.im, A[2 * m]));
+          A[2 * m + 1] = fma(u.re, w.im, fma(-u.im, w.re, A[2 * m + 1]));
+        }
+      }
+    }
+  }
+  // the sets' sums, one of a tile a thread
+  double* sums = reinterpret_cast<double*>(xe);
+  float* sures = reinterpret_cast<float*>(sums + 8 * GS_THREADS);
+  int* refs = reinterpret_cast<int*>(sures + 8 * GS_THREADS);
+  __syncthreads();
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    sums[m * GS_THREADS + threadIdx.x] = A[m];
+    sures[m * GS_THREADS + threadIdx.x] = sure[m];
+  }
+  refs[threadIdx.x] = ref;
+  __syncthreads();
+  if (set > 0) return;
+  int top = ref;
+  for (int p = 1; p < P; ++p) top = max(top, refs[p * ntiles + threadIdx.x]);
+  bool certain = true;
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    float y = 0.f;
+    for (int p = 0; p < P; ++p) {
+      const int t = p * ntiles + threadIdx.x;
+      const float f = __int_as_float(max(127 + refs[t] - top, 0) << 23);
+      y += f * (f * sures[m * GS_THREADS + t]);
+      if (p > 0) A[m] += sums[m * GS_THREADS + t];
+    }
+    certain = certain && y >= 0.f;
+  }
+  if (!certain) {
+    const cpx<double>* x0 = vecs + (long long)tj * fs;
+    const cpx<double>* y0 = vecs + (long long)tk * fs;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) A[m] = 0.0;
+    for (long long e = e0; e < e1; ++e) {
+      const unsigned o = cqr_off(g, bg, a, e);
+      const cpx<double> u[2] = {x0[o], x0[fs + o]}, w[2] = {y0[o], y0[fs + o]};
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const cpx<double> p = u[m >> 1], r = w[m & 1];
+        A[2 * m] = fma(p.re, r.re, fma(p.im, r.im, A[2 * m]));
+        A[2 * m + 1] = fma(p.re, r.im, fma(-p.im, r.re, A[2 * m + 1]));
+      }
+    }
+  }
+  cpx<double>* R = part + ((long long)a * S + q) * nvec * nvec;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) R[(tj + (m >> 1)) * nvec + tk + (m & 1)] = cpx<double>(A[2 * m], A[2 * m + 1]);
 }
 
 // G = sum_q part[a][q] (fixed order), G = R^dag R, rinv[a] = R^{-1}; one warp per
@@ -374,14 +560,20 @@ static int cholesky_qr2(const Geom& g, const BlockGeom& bg, cpx<double>* vecs, i
   // skip flags [0, Vc), then the list of flagged blocks handed to the caller
   if (e == cudaSuccess) e = cudaMallocAsync(&skip, sizeof(int) * (2 * (size_t)Vc + 1), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(skip, 0, sizeof(int) * (2 * (size_t)Vc + 1), st);
-  const size_t smem_gram = sizeof(cpx<double>) * (size_t)nvec * CQR_E;
+  // with more than one tile a thread the sums of squares do not fit in its registers
+  const bool fixed = (nvec / 2) * (nvec / 2 + 1) / 2 <= GS_THREADS;
+  auto gram = fixed ? cqr_gram_fx_kernel : cqr_gram_kernel;
+  const size_t smem_gram =
+      fixed ? std::max((sizeof(int4) * (CQR_E + 1) + sizeof(int) * CQR_GROUPS) * (size_t)nvec,
+                       (8 * (sizeof(double) + sizeof(float)) + sizeof(int)) * (size_t)GS_THREADS)
+            : sizeof(cpx<double>) * (size_t)nvec * CQR_E;
   const size_t smem_chol = sizeof(cpx<double>) * nn + sizeof(double) * nvec;
   const size_t smem_apply = sizeof(cpx<double>) * (nn + (size_t)nvec * CQR_E);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(cqr_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_gram);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_gram);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(cqr_chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_chol);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(cqr_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_apply);
   for (int round = 0; round < 2 && e == cudaSuccess; ++round) {
-    cqr_gram_kernel<<<dim3(Vc, S), GS_THREADS, smem_gram, st>>>(g, bg, vecs, nvec, S, skip, part);
+    gram<<<dim3(Vc, S), GS_THREADS, smem_gram, st>>>(g, bg, vecs, nvec, S, skip, part);
     cqr_chol_kernel<<<Vc, 32, smem_chol, st>>>(nvec, S, part, rinv, skip);
     cqr_apply_kernel<<<dim3(Vc, S), GS_THREADS, smem_apply, st>>>(g, bg, vecs, nvec, S, skip, rinv);
     count_launches(3);

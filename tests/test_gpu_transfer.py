@@ -95,18 +95,19 @@ def test_values_outside_the_format(hd, value):
         assert np.abs(gf[other] - wf[other]).max() <= 1e-14 * np.abs(wf[other]).max()
 
 
-# vector counts whose tiles fill one to three rounds of the threads, Ls for which the last chunk of 96
-# elements is short, shares of a block
+# vector counts whose tiles fill one to six sets of threads (in fixed point up to 44) and two and three rounds
+# of them, Ls for which the last chunk of 96 elements ends inside a group of 16, shares of a block
 @pytest.mark.parametrize("L,Ls,block,nvec", [((4, 4, 2, 2), 3, (2, 2, 1, 1), 2), ((4, 4, 4, 4), 5, (2, 2, 2, 2), 8),
                                              ((4, 4, 4, 4), 8, (2, 2, 2, 2), 24), ((6, 2, 2, 6), 7, (3, 1, 1, 3), 34),
-                                             ((4, 4, 4, 4), 4, (2, 2, 2, 2), 46), ((4, 4, 4, 4), 5, (2, 2, 2, 2), 64)])
+                                             ((4, 4, 4, 4), 3, (2, 2, 2, 2), 44), ((4, 4, 4, 4), 4, (2, 2, 2, 2), 46),
+                                             ((4, 4, 4, 4), 5, (2, 2, 2, 2), 64)])
 @pytest.mark.parametrize("scale", [None, "spread", "outside"])
 def test_block_orthonormalisation(hd, L, Ls, block, nvec, scale):
     v = synth.gaussian_fermion(L, Ls, 6100, count=nvec)
     if scale == "spread":       # the fifth dimension's profile, and vectors of different sizes
         v = v * np.exp(-3.0 * np.arange(Ls))[:, None, None]
         v = v * 10.0 ** (np.arange(nvec) % 7 - 3.0).reshape((-1,) + (1,) * 7)
-    elif scale == "outside":    # parts of one vector whose squares underflow
+    elif scale == "outside":    # groups of one vector below the format's smallest exponent
         v[0][..., :2, :] *= 1e-220
     got = host(hd.subspace_from_vectors(hd.Lattice(L, Ls), block, dev(planes(v)), store_dtype=torch.complex128).vectors())
     q = blocks(got, L, Ls, block).astype(np.clongdouble)
