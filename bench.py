@@ -82,7 +82,7 @@ def bytes_per_site(real_bytes: int, Ls: int) -> float:
 
 # DRAM traffic of one FP64 / FP32 / FP16-storage stencil launch at 16^4 x 16 from ncu, with the hash of
 # the stencil sources it was measured on (reported as null once the sources change)
-NCU_TRAFFIC = {"f64": 539.33e6, "f32": 202.18e6, "h16": 106.18e6, "src_hash": "77e7053397027943"}
+NCU_TRAFFIC = {"f64": 571.81e6, "f32": 202.18e6, "h16": 106.18e6, "src_hash": "6cf224fdd680fc72"}
 
 
 def stencil_src_hash() -> str:
@@ -360,8 +360,8 @@ def run_ours(args, world, rank, local):
                     "avg_launch_ms": round(ms64c, 4), "share_of_step": round(share64c, 3),
                     "tflops": round((FLOPS_PER_SITE + 144) * st64c["sites"] / max(st64c["launches"], 1)
                                     / max(ms64c * 1e-3, 1e-12) / 1e12, 4)},
-                "peak_note": "the kernel does its products on the integer pipe and is limited by its wide "
-                             "multiply-adds, not by memory; fp64_fma_tflops is the FP64 pipe's measured rate "
+                "peak_note": "the kernel does its products on the integer pipe and is limited by "
+                             "instruction issue, not by memory; fp64_fma_tflops is the FP64 pipe's measured rate "
                              "(hdcr_probe_fma_rate, FMA = 2 flops), which bounded the operator as FP64 FMAs"}
     roofline_fp32 = {"bound": "hbm", "kernel": "g5dwf FP32 (H = Gamma5 D_dwf)", "achieved": round(gbs32, 1),
                      "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": round(gbs32 / pk["hbm_gbs"], 4),
